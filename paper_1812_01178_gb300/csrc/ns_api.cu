@@ -97,7 +97,7 @@ ns_layout make_layout(const ns_config* c) {
   sz[LB_LAMZ] = nzh * 8;
   sz[LB_RTAB] = 3 * al256((size_t)RT_COUNT * (ny + 1) * 8) + 3 * al256((size_t)RT_COUNT * (ny + 1) * 4);
   sz[LB_DOUT] = 3 * al256((ny + 1) * nz * 8) + 256;
-  sz[LB_TWD] = nx * 32;
+  sz[LB_TWD] = nx * sizeof(FxTw);
   sz[LB_RCY] = recycle_block_doubles((int)ny) * 8;
   sz[LB_STEPK] = NS_STEPK * sizeof(StepK);
   sz[LB_PTAB] = 9 * al256(line_table_floats(c) * 4);
@@ -404,8 +404,8 @@ ns_status ns_init(ns_ctx** out, const ns_config* cfg, const ns_fields* fields, v
     for (int q = 0; q < 2; ++q) c->ytab[k][q] = base + c->lay.off[LB_YTAB] + (2 * k + q) * al256(3 * ny * c->es);
     c->ztab[k] = base + c->lay.off[LB_ZTAB] + k * al256(ztab_entries(nz) * c->es);
   }
-  c->twz = (double2*)(base + c->lay.off[LB_TWZ]);
-  c->twx = (double2*)(base + c->lay.off[LB_TWX]);
+  c->twz = (FxTw*)(base + c->lay.off[LB_TWZ]);
+  c->twx = (FxTw*)(base + c->lay.off[LB_TWX]);
   double* lamx_d = (double*)(base + c->lay.off[LB_LAMX]);
   for (int q = 0; q < 3; ++q) c->dout[q] = (double*)(base + c->lay.off[LB_DOUT] + q * al256((size_t)(ny + 1) * nz * 8));
   c->flux = (double*)(base + c->lay.off[LB_DOUT] + 3 * al256((size_t)(ny + 1) * nz * 8));
@@ -421,7 +421,7 @@ ns_status ns_init(ns_ctx** out, const ns_config* cfg, const ns_fields* fields, v
   for (int k = 0; k < 3; ++k)
     for (int q = 0; q < 3; ++q)
       c->ptab[k][q] = base + c->lay.off[LB_PTAB] + (3 * k + q) * al256(line_table_floats(cfg) * 4);
-  c->twd = (double2*)(base + c->lay.off[LB_TWD]);
+  c->twd = (FxTw*)(base + c->lay.off[LB_TWD]);
   c->pois32 = cfg->precision == NS_MIXED;
   if (c->pois32) {
     char* t32 = base + c->lay.off[LB_TW32];
@@ -479,11 +479,16 @@ ns_status ns_init(ns_ctx** out, const ns_config* cfg, const ns_fields* fields, v
   // ---------------- FFT twiddles, modified wavenumbers, Poisson y factors
   if (st == NS_OK) {
     const double PI = 3.14159265358979323846;
-    std::vector<double> tw(fft_twiddle_doubles(nz)), tx(fft_twiddle_doubles(nx));
-    fft_twiddles(nz, tw.data());
-    fft_twiddles(nx, tx.data());
-    if (upload_d(c, c->twz, tw) != cudaSuccess) st = NS_ERR_CUDA;
-    if (upload_d(c, c->twx, tx) != cudaSuccess) st = NS_ERR_CUDA;
+    if (!c->pois32) {  // fixed-point twiddles of the FP64 transforms
+      std::vector<FxTw> tw(3 * (size_t)nz), tx(3 * (size_t)nx), td(nx);
+      fx_twiddles(nz, tw.data());
+      fx_twiddles(nx, tx.data());
+      fx_dct_twiddles(nx, td.data());
+      if (upload_raw(c, c->twz, tw.data(), tw.size() * sizeof(FxTw)) != cudaSuccess ||
+          upload_raw(c, c->twx, tx.data(), tx.size() * sizeof(FxTw)) != cudaSuccess ||
+          upload_raw(c, c->twd, td.data(), td.size() * sizeof(FxTw)) != cudaSuccess)
+        st = NS_ERR_CUDA;
+    }
     std::vector<double> lx(nx), lz(c->nzh);
     for (int q = 0; q < nx; ++q) {
       if (c->bl) {  // DCT-II modes (zero gradient at x = 0 and x = Lx)
@@ -493,15 +498,17 @@ ns_status ns_init(ns_ctx** out, const ns_config* cfg, const ns_fields* fields, v
         lx[q] = (2.0 / (c->dx * c->dx)) * (1.0 - std::cos(2.0 * PI * qq / nx));
       }
     }
-    std::vector<double> td(4 * nx);  // w_l, then w_l / 2 (exact) for the forward transform
-    for (int q = 0; q < nx; ++q) {
-      td[2 * q] = std::cos(PI * q / (2.0 * nx));
-      td[2 * q + 1] = -std::sin(PI * q / (2.0 * nx));
-      td[2 * (nx + q)] = 0.5 * td[2 * q];
-      td[2 * (nx + q) + 1] = 0.5 * td[2 * q + 1];
-    }
-    if (upload_d(c, c->twd, td) != cudaSuccess) st = NS_ERR_CUDA;
-    if (c->pois32) {  // the same tables rounded to float for the FP32 transforms of the mixed form
+    if (c->pois32) {  // float twiddles of the FP32 transforms of the mixed form
+      std::vector<double> tw(fft_twiddle_doubles(nz)), tx(fft_twiddle_doubles(nx));
+      fft_twiddles(nz, tw.data());
+      fft_twiddles(nx, tx.data());
+      std::vector<double> td(4 * nx);  // w_l, then w_l / 2 (exact) for the forward cosine transform
+      for (int q = 0; q < nx; ++q) {
+        td[2 * q] = std::cos(PI * q / (2.0 * nx));
+        td[2 * q + 1] = -std::sin(PI * q / (2.0 * nx));
+        td[2 * (nx + q)] = 0.5 * td[2 * q];
+        td[2 * (nx + q) + 1] = 0.5 * td[2 * q + 1];
+      }
       const std::vector<float> fz(tw.begin(), tw.end()), fx(tx.begin(), tx.end()), fd(td.begin(), td.end());
       const std::vector<float> pa32(gc.begin() + (size_t)GC_PA * G, gc.begin() + (size_t)GC_PA * G + ny);
       std::vector<float> rows32(4 * (size_t)ny, 0.0f);  // (a_j, c_j, -(a_j + c_j), a_j - (float)a_j)

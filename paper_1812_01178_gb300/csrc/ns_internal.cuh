@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/ns.h"
+#include "fx64.cuh"
 
 // FFT plan of a length N = 2^a 3^b: a | (b << 8), or -1 for any other N.
 inline __host__ __device__ int fft_plan(int N) {
@@ -63,6 +64,53 @@ inline void fft_twiddles(int N, double* out) {
       e[4] = 0.5 * c1;
       e[5] = S3 * c1;
     }
+}
+
+// Twiddles of the fixed-point transforms (fx64.cuh): w = exp(-i th) of input r of a stage that
+// follows sub-transforms of length Ns, th = 2 pi r k / (R Ns), at 3 (Ns + k) + r - 1 (the stage order
+// and index ranges of fft_twiddles; a radix-3 entry leaves its third place zero).  out has room for
+// 3 N entries, the bytes of fft_twiddle_doubles(N).
+inline FxCoef fx_coef(long double w) {
+  const fx_t x = (fx_t)llroundl(w * 4611686018427387904.0L);  // w 2^62
+  FxCoef c = fx_limbs(x);
+  if (c.l == INT32_MIN) ++c.l;  // the limbs are negated for conjugates
+  return c;
+}
+inline FxTw fx_twiddle(long num, long den) {  // exp(-2 pi i num / den), 0 <= num <= den / 8
+  const long double PI = 3.14159265358979323846264338327950288L;
+  const long double th = 2.0L * PI * (long double)num / (long double)den;
+  return FxTw{fx_coef(cosl(th)), fx_coef(sinl(th))};
+}
+// exp(-2 pi i m / N) for any m, from the first octant oct[0 .. N / 8] (N a multiple of 8; long double
+// functions are slow where it is a 128-bit format)
+inline FxTw fx_root(const FxTw* oct, long N, long m) {
+  m %= N;
+  const int quad = (int)(4 * m / N);
+  m -= quad * (N / 4);
+  FxTw w = m <= N / 8 ? oct[m] : FxTw{oct[N / 4 - m].s, oct[N / 4 - m].c};
+  for (int q = 0; q < quad; ++q) w = FxTw{fx_neg(w.s), w.c};  // th + pi / 2: cos -> -sin, sin -> cos
+  return w;
+}
+inline void fx_twiddles(int N, FxTw* out) {
+  for (int q = 0; q < 3 * N; ++q) out[q] = FxTw{{0, 0}, {0, 0}};
+  const int plan = fft_plan(N);
+  if (plan < 0 || N % 8 || N > 4096) return;
+  FxTw oct[4096 / 8 + 1];
+  for (int q = 0; q <= N / 8; ++q) oct[q] = fx_twiddle(q, N);
+  const int a = plan & 0xff, b = plan >> 8;
+  int Ns = (a & 1) ? 2 : 1;
+  for (int s = 0; s < (a >> 1) + b; ++s) {
+    const int R = s < (a >> 1) ? 4 : 3;
+    for (int k = 0; k < Ns && Ns > 1; ++k)
+      for (int r = 1; r < R; ++r) out[3 * (Ns + k) + r - 1] = fx_root(oct, N, (long)r * k * (N / (R * Ns)));
+    Ns *= R;
+  }
+}
+// exp(-i pi l / (2 N)), l < N: the cosine transform's twiddles
+inline void fx_dct_twiddles(int N, FxTw* out) {
+  std::vector<FxTw> oct(N / 2 + 1);
+  for (int q = 0; q <= N / 2; ++q) oct[q] = fx_twiddle(q, 4L * N);
+  for (int q = 0; q < N; ++q) out[q] = fx_root(oct.data(), 4L * N, q);
 }
 
 // Partition shapes the x solver is built for: P lanes (a power of two <= 32) of M rows, with
@@ -236,13 +284,13 @@ struct ns_ctx {
   int yL[3] = {0, 0, 0}, zL[3] = {0, 0, 0};
   void* ptab[3][3] = {};
   double ypdd_drop = 0.0, zpdd_drop = 0.0;
-  double2* twz;
-  double2* twx;
+  FxTw* twz;                // fixed-point twiddles (fx_twiddles)
+  FxTw* twx;
   double* rtab[3];
   float* rtabf[3];          // float copies of rtab for the FP32 form
   int bl;                   // inflow / convective outflow in x
   double* dout[3];          // outflow-plane increments of the current sub-step (u, v, w)
-  double2* twd;             // exp(-i pi l / (2 nx)), l < nx, then the same halved: x cosine transform twiddles
+  FxTw* twd;                // exp(-i pi l / (2 nx)), l < nx: x cosine transform twiddles
   // the mixed form's Poisson solve: FP32 transforms (twiddles rounded to float) and one FP64
   // refinement (k_poisson.cu); off for FP64 contexts
   bool pois32 = false;

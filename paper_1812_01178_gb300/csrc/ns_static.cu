@@ -28,8 +28,8 @@ void* g_scratch[kMaxDevices] = {};  // device address of g_ns_static_scratch, pe
 
 // host staging for the small tables (static: no allocation at call time); guarded by g_mu
 double h_gc[NS_GC_COUNT * 1025];
-double h_twz[6 * 4096];
-double h_twx[6 * 4096];
+FxTw h_twz[3 * 4096];
+FxTw h_twx[3 * 4096];
 double h_lamx[4096];
 double h_lamz[2049];
 StepK h_stepk[NS_STEPK];
@@ -130,8 +130,8 @@ extern "C" ns_status ns_poisson_solve_static(const ns_config* cfg, const double*
   for (int j = 0; j + 1 < ny; ++j) GC(GC_PC, j) = 1.0 / ((yf[j + 1] - yf[j]) * (yc(j + 1) - yc(j)));
   const double PI = 3.14159265358979323846;
   const double dx = cfg->lx / nx, dz = cfg->lz / nz;
-  fft_twiddles(nz, h_twz);
-  fft_twiddles(nx, h_twx);
+  fx_twiddles(nz, h_twz);
+  fx_twiddles(nx, h_twx);
   for (int q = 0; q < nx; ++q) {
     const int qq = q <= nx - q ? q : nx - q;
     h_lamx[q] = (2.0 / (dx * dx)) * (1.0 - std::cos(2.0 * PI * qq / nx));
@@ -173,8 +173,8 @@ extern "C" ns_status ns_poisson_solve_static(const ns_config* cfg, const double*
   c.spec = (double2*)(base + R.spec);
   c.pois = (double2*)(base + R.pois);
   c.gc = (double*)(base + R.gc);
-  c.twz = (double2*)(base + R.twz);
-  c.twx = (double2*)(base + R.twx);
+  c.twz = (FxTw*)(base + R.twz);
+  c.twx = (FxTw*)(base + R.twx);
   c.stepk = (StepK*)(base + R.stepk);
   if ((e = launch_pois_factor(&c, (const double*)(base + R.lamx), (const double*)(base + R.lamz))) != cudaSuccess)
     return fail(NS_ERR_CUDA, std::string("factor table: ") + cudaGetErrorString(e));
