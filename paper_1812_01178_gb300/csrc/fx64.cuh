@@ -23,7 +23,17 @@ typedef long long fx_t;
 
 FX_HD int fx_hi(fx_t x) { return (int)(x >> 32); }
 FX_HD unsigned fx_lo(fx_t x) { return (unsigned)x; }
-FX_HD fx_t fx_mad(int a, int b, fx_t c) { return (fx_t)a * b + c; }  // one IMAD.WIDE
+// One multiply-add of 32 x 32 + 64 bits.  (Written as a C product of operands cut out of 64-bit values
+// the compiler forms some of them from three or four multiplications.)
+FX_HD fx_t fx_mad(int a, int b, fx_t c) {
+#ifdef __CUDA_ARCH__
+  fx_t r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return (fx_t)a * b + c;
+#endif
+}
 FX_HD uint64_t fx_bits(double d) {
 #ifdef __CUDA_ARCH__
   return (uint64_t)__double_as_longlong(d);
@@ -162,3 +172,79 @@ FX_HD unsigned fx_span(Fx2 a) {
 }
 // Right shift before a stage that sums up to four values: keeps the sums below 2^61.5 in modulus
 FX_HD int fx_stage_shift(unsigned span) { return (span >> 28) ? 2 : (span >> 27) ? 1 : 0; }
+
+// ---- sums of products with coefficients of any size (the stencils)
+//
+// A coefficient c meeting values whose bit 62 stands for the exponent et enters a sum whose bit 62
+// stands for er as w = c 2^(et + 2 - er), |w| < 1; the sum of X w / 4 over terms |X| <= 2^62 whose
+// |w| add up to less than 1 stays below 2^60.
+FX_HD FxCoef fx_wcoef(double c, int et, int er) { return fx_limbs(fx_from(c, 1021 - et + er)); }
+// h + m / 2^32.  Room in m: the |X| of the terms between two folds add up to at most 2^63.3 (2.5
+// times 2^62).
+struct FxAcc {
+  fx_t h, m;
+};
+FX_HD FxAcc fx_wacc(fx_t x) { return FxAcc{x, (fx_t)1 << 31}; }
+FX_HD void fx_wmac(FxAcc& a, fx_t v, FxCoef w) {  // adds X w / 4
+  const FxCoef x = fx_limbs(v);
+  a.h = fx_mad(x.h, w.h, a.h);
+  a.m = fx_mad(x.l, w.h, fx_mad(x.h, w.l, a.m));
+}
+FX_HD void fx_wfold(FxAcc& a) {
+  a.h += a.m >> 32;
+  a.m = (fx_t)(uint32_t)a.m;
+}
+FX_HD fx_t fx_wsum(const FxAcc& a) { return a.h + (a.m >> 32); }
+// x0 c0 + x1 c1 of weights c0 + c1 <= 1 and values up to 2^61, brought up to 2^62
+FX_HD fx_t fx_interpolate(fx_t x0, fx_t x1, FxCoef c0, FxCoef c1) {
+  FxAcc s = {0, (fx_t)1 << 28};
+  fx_wmac(s, x0, c0);
+  fx_wmac(s, x1, c1);
+  return s.h * 8 + (s.m >> 29);
+}
+// The part of the sum of |c| 2^(et + 2) one term takes, relative to 2^(emax - 1023 - 20) (emax: the
+// largest ee of the terms), rounded up; ee = fx_wexp(c, et)
+constexpr int FX_NONE = -100000;
+FX_HD int fx_wexp(double c, int et) {
+  const int ec = (int)(fx_mag(c) >> 20);
+  return ec == 0 ? FX_NONE : ec + et + 2;
+}
+FX_HD unsigned fx_wpart(double c, int ee, int emax) {
+  const int d = emax - ee;
+  return ee == FX_NONE ? 0u : d > 24 ? 1u : ((((fx_mag(c) & 0xfffffu) | 0x100000u) + 1) >> d) + 1;
+}
+FX_HD int fx_wscale(int emax, unsigned parts) {  // er
+  return emax == FX_NONE ? 1023 : emax - 1023 - 20 + (64 - fx_clz(parts));
+}
+// X Y / 2^64 of |X|, |Y| <= 2^62, to about one unit
+FX_HD fx_t fx_mulhi(fx_t a, fx_t b) {
+  const FxCoef x = fx_limbs(a), y = fx_limbs(b);
+  return fx_mad(x.h, y.h, 0) + (fx_mad(x.l, y.h, fx_mad(x.h, y.l, (fx_t)1 << 31)) >> 32);
+}
+FX_HD fx_t fx_sqrhi(fx_t a) {
+  const FxCoef x = fx_limbs(a);
+  return fx_mad(x.h, x.h, 0) + (fx_mad(x.l, x.h, (fx_t)1 << 30) >> 31);
+}
+// fx_from for planes of a common exponent e = s - 2, cut towards zero
+FX_HD fx_t fx_cut(double d, int s) {
+  const uint64_t b = fx_bits(d);
+  const unsigned hi = (unsigned)(b >> 32);
+  int sh = s - 2 - (int)((hi >> 20) & 0x7ffu);
+  sh = sh < 63 ? sh : 63;
+  const fx_t v = (fx_t)((((((uint64_t)((hi & 0xfffffu) | 0x100000u)) << 32) | (uint32_t)b) << 8) >> sh);
+  const fx_t sg = (fx_t)((int)hi >> 31);
+  return (v ^ sg) - sg;
+}
+// x as a double, rounded, by two FP64 instructions (the high limb scaled by 2^32 is exact)
+FX_HD double fx_double(fx_t x) {
+  const double h = fx_from_bits(0x4330000000000000ull | ((uint64_t)(x >> 32) & 0xffffffffull) ^ 0x80000000ull);
+  const double l = fx_from_bits(0x4330000000000000ull | (uint64_t)(uint32_t)x);
+  // h = 2^52 + 2^31 + hi, l = 2^52 + lo
+#ifdef __CUDA_ARCH__
+  return fma(h, 0x1p32, -(0x1p84 + 0x1p63 + 0x1p52)) + l;
+#else
+  return (h * 0x1p32 - (0x1p84 + 0x1p63 + 0x1p52)) + l;
+#endif
+}
+// the unit of a sum at scale e: 2^(e - 1023 - 62)
+FX_HD double fx_unit(int e) { return fx_from_bits((uint64_t)(uint32_t)(e - 62) << 52); }

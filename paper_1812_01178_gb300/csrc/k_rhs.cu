@@ -5,9 +5,9 @@
 // distance-weighted linear interpolation in y.  L is the viscous operator (uniform second
 // differences in x and z, the three-point non-uniform formula in y).  G is the pressure gradient.
 //
-// rhs_kernel: one thread per (i, j) of one z-plane, j = 0..ny (row ny only writes the v wall row),
-// used when nx is not a multiple of 32 or nz not a multiple of 8; rhs_tiled_kernel otherwise.
-// T is the arithmetic type (double, or float for the mixed form), TR the storage type of r and N.
+// RhsFxK: the FP64 form, in 64-bit fixed point.  The mixed form (FP32): RhsTiledK where nx is a
+// multiple of 32, else RhsK, one thread per (i, j) of one z-plane, j = 0..ny (row ny only writes the v
+// wall row).  T is the arithmetic type, TR the storage type of r and N.
 #include "ns_internal.cuh"
 
 namespace {
@@ -45,26 +45,10 @@ struct RhsArgs {
 
 namespace {
 
-// Dyn: the sub-step constants are read from device memory (a step graph that outlives changes of
-// dt); otherwise from the kernel arguments, where they cost no registers.
-template <typename T, typename TR, bool Dyn>
-struct RhsK {
-  struct Args {
-    RhsArgs a;
-  };
-  static constexpr int kThreads = 128;
-  static constexpr int kMinBlocks = 7;
-  static Args make(RhsArgs a) { return Args{a}; }
-  static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3 gdim_) {
-    const RhsArgs& a = a_.a;
-
+// The right-hand side at (i, j, k): u, w of cell row j (j < ny) and v of face row j (zero on the walls)
+template <typename T, typename TR>
+__device__ __forceinline__ void rhs_cell(const RhsArgs& a, int i, int j, int k, T dt) {
   const int nx = a.nx, ny = a.ny, nz = a.nz;
-  const long plane = (long)nx * (ny + 1);
-  const long q = (long)bid_.x * blockDim.x + threadIdx.x;
-  if (q >= plane) return;
-  const int j = (int)(q / nx);
-  const int i = (int)(q - (long)j * nx);
-  const int k = bid_.y;
   const int ip = (i + 1 == nx) ? 0 : i + 1;
   const int im = (i == 0) ? nx - 1 : i - 1;
   const int kp = (k + 1 == nz) ? 0 : k + 1;
@@ -97,7 +81,7 @@ struct RhsK {
   auto C = [&](int f, int jj) -> T { return from_double<T>(__ldg(a.gc + f * G + jj)); };
 
   const T idx = (T)a.idx, idz = (T)a.idz, idx2 = (T)a.idx2, idz2 = (T)a.idz2;
-  const T dt = (T)(Dyn ? a.sk->dt : a.kc.dt), alp = (T)a.alp;
+  const T alp = (T)a.alp;
   const T avis = (T)(a.alp * a.inv_re);
   // N is stored pre-multiplied by cn = -dt gamma_k, as in the tiled form; the stored N of the
   // previous sub-step enters with zeta_k / gamma_(k-1)
@@ -205,12 +189,30 @@ struct RhsK {
     rv[cf] = (TR)r;
     nv[cf] = (TR)nt;
   }
+}
 
+// One thread per (i, j): the FP32 form on grids the tile does not fit.  Dyn: the sub-step constants
+// are read from device memory (a step graph that outlives changes of dt); otherwise from the kernel
+// arguments, where they cost no registers.
+template <typename T, typename TR, bool Dyn>
+struct RhsK {
+  struct Args {
+    RhsArgs a;
+  };
+  static constexpr int kThreads = 128;
+  static constexpr int kMinBlocks = 7;
+  static Args make(RhsArgs a) { return Args{a}; }
+  static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3) {
+    const RhsArgs& a = a_.a;
+    const long q = (long)bid_.x * blockDim.x + threadIdx.x;
+    if (q >= (long)a.nx * (a.ny + 1)) return;
+    const int j = (int)(q / a.nx);
+    rhs_cell<T, TR>(a, (int)(q - (long)j * a.nx), j, bid_.y, (T)(Dyn ? a.sk->dt : a.kc.dt));
   }
 };
 
 // ---------------------------------------------------------------------------------------------
-// Tiled form of the same right-hand side.  A block of TX x TZ threads owns a TX (x) by TZ (z)
+// Tiled form of the same right-hand side in FP32 (mixed form).  A block of TX x TZ threads owns a TX (x) by TZ (z)
 // column of cells and marches along y over [jb, je).  Four rolling planes of u, v, w, p (with a
 // one-cell halo in x and z, periodic wrap) sit in shared memory.  Every product the
 // divergence-form convection needs is computed once per tile and then differenced:
@@ -228,8 +230,8 @@ constexpr int RT_PZ = RT_Z + 2;
 constexpr int RT_PLANE = RT_PX * RT_PZ;
 constexpr int RT_NPL = 4;         // rolling planes per field
 
-template <typename T>
 struct RhsTile {
+  using T = float;
   T pl[4][RT_NPL][RT_PLANE];                 // u, v, w, p planes (j mod 4), index (kk+1)*RT_PX + (ii+1)
   T fuv[2][RT_Z][RT_X + 1];                  // Fuv on y-face (parity), x = i0 .. i0+TX
   T fvw[2][RT_Z + 1][RT_X];                  // Fvw on y-face (parity), z = k0 .. k0+TZ
@@ -240,36 +242,29 @@ struct RhsTile {
   T wf[RT_NPL];                              // RHO = WHI / WLO of face j (j mod 4), zero at the walls
 };
 
-// State values entering the FP32 tile: the hardware conversion (one instruction on the FP64
-// pipe, which the FP32 RHS leaves idle) instead of the integer-pipe d2f_rn (about a dozen
-// instructions on the issue-bound FP32 RHS).
-template <typename T>
-__device__ __forceinline__ T plane_cvt(double x) {
-  if constexpr (sizeof(T) == 4) return __double2float_rn(x);
-  else return x;
-}
-
 // 8-byte global -> shared copy that completes asynchronously (cp.async, waited for by
 // cp.async.wait_all); with valid false nothing is read and the 8 bytes are zero-filled
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem, bool valid) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "r"(valid ? 8 : 0) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit8() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all8() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-template <typename T, typename TR, bool Dyn>
+// State values enter by the hardware conversion (one instruction on the FP64 pipe, which the FP32
+// RHS leaves idle) instead of the integer-pipe d2f_rn (about a dozen instructions on this issue-bound
+// kernel).
+template <bool Dyn>
 struct RhsTiledK {
+  using T = float;
   struct Args {
     RhsArgs a;
     int jchunk;
   };
   static constexpr int kThreads = RT_X * RT_Z;
-  // FP64: shared memory allows 3 resident blocks, so up to 85 registers cost nothing.  FP32: 6
-  // blocks of up to 40 registers (the kernel waits on memory and shared memory, so occupancy pays
+  // 6 blocks of up to 40 registers (the kernel waits on memory and shared memory, so occupancy pays
   // more than registers: 0.314 ms at 6 blocks against 0.338 at 5, 0.352 at 4 and 0.434 at 3), or 4
   // of up to 64 when the sub-step constants come from device memory (fewer spill)
-  static constexpr int kMinBlocks = sizeof(T) == 8 ? 3 : (Dyn ? 4 : 6);
+  static constexpr int kMinBlocks = Dyn ? 4 : 6;
   static Args make(RhsArgs a, int jchunk) { return Args{a, jchunk}; }
   static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3 gdim_) {
     const RhsArgs& a = a_.a;
@@ -277,7 +272,7 @@ struct RhsTiledK {
     const int jb = bid_.z * a_.jchunk;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  RhsTile<T>& S = *reinterpret_cast<RhsTile<T>*>(smem_raw);
+  RhsTile& S = *reinterpret_cast<RhsTile*>(smem_raw);
   const int nx = a.nx, ny = a.ny, nz = a.nz, ny1 = ny + 1, G = ny + 1;
   const int tx = threadIdx.x, tz = threadIdx.y, tid = tz * RT_X + tx;
   const int je = min(jb + a_.jchunk, ny);
@@ -313,33 +308,21 @@ struct RhsTiledK {
       }
     }
   }
-  // FP64: planes are copied global -> shared by cp.async one step ahead (plane j + 2 is issued in
-  // step j, after the barrier that ends every read of plane j - 2 in its buffer, and waited for in
-  // step j + 1), so that no block stalls on its own plane loads; x-boundary halo positions are
-  // formed by plain loads.  FP32 converts on the way and loads through registers.
-  constexpr bool kAsync = sizeof(T) == 8;
   auto load_plane = [&](int j) {
     const bool jc = j >= 0 && j < ny, jv = j >= 0 && j <= ny;
     const long jo = (long)j * nx;
 #pragma unroll
     for (int r = 0; r < kPos; ++r) {
-      if (kAsync && pos[r] >= 0) {
-        const int e = pos[r];
-        const long o = oc[r] + jo, q = ov[r] + jo;
-        cp_async8(&S.pl[0][j & 3][e], a.u + (jc ? o : 0), jc);
-        cp_async8(&S.pl[1][j & 3][e], a.v + (jv ? q : 0), jv);
-        cp_async8(&S.pl[2][j & 3][e], a.w + (jc ? o : 0), jc);
-        cp_async8(&S.pl[3][j & 3][e], a.p + (jc ? o : 0), jc);
-      } else if (pos[r] >= 0) {
+      if (pos[r] >= 0) {
         const int e = pos[r];
         const long o = oc[r] + jo, q = ov[r] + jo;
         T vu = (T)0, vv = (T)0, vw = (T)0, vp = (T)0;
         if (jc) {
-          vu = plane_cvt<T>(__ldg(a.u + o));
-          vw = plane_cvt<T>(__ldg(a.w + o));
-          vp = plane_cvt<T>(__ldg(a.p + o));
+          vu = __double2float_rn(__ldg(a.u + o));
+          vw = __double2float_rn(__ldg(a.w + o));
+          vp = __double2float_rn(__ldg(a.p + o));
         }
-        if (jv) vv = plane_cvt<T>(__ldg(a.v + q));
+        if (jv) vv = __double2float_rn(__ldg(a.v + q));
         S.pl[0][j & 3][e] = vu;
         S.pl[1][j & 3][e] = vv;
         S.pl[2][j & 3][e] = vw;
@@ -365,14 +348,10 @@ struct RhsTiledK {
         S.pl[3][j & 3][e] = (T)0;
       }
     }
-    if (kAsync) cp_async_commit8();
   };
   // Each product loop gives every thread the item q = tid first (every loop has at least 256
-  // items).  In the FP32 form that item's tile offsets are worked out once, before the march in y,
-  // and only the few items q >= 256 take the general index arithmetic: the FP32 RHS is
-  // issue-bound.  (The FP64 form takes the general index arithmetic for both: the offsets cost it
-  // registers.)
-  constexpr bool kHoist = sizeof(T) == 4;
+  // items); that item's tile offsets are worked out once, before the march in y, and only the few
+  // items q >= 256 take the general index arithmetic: the FP32 RHS is issue-bound.
   const int hk = tid / (RT_X + 1), hi = tid % (RT_X + 1);   // items of the (RT_X + 1)-wide loops
   const int gk = tid / RT_X, gi = tid % RT_X;               // items of the RT_X-wide loops
   const int eA = (hk + 1) * RT_PX + hi + 1, fA = hk * (RT_X + 1) + hi;
@@ -381,12 +360,10 @@ struct RhsTiledK {
   // y-face fluxes on face jf, zero on the walls, each divided by the interpolation weight WLO_jf
   // (which the difference weights carry): Fuv = (u_{j-1} + RHO u_j)(v_{i-1} + v_i) and
   // Fvw = (v_{k-1} + v_k)(w_{j-1} + RHO w_j), one FMA, one add and one product each
-  // Every product loop has NT <= n < 2 NT items: thread tid takes item tid.  In the FP32 form the
-  // n - NT items past NT go to the threads from `off` on: Fuv and Q1's extra items to warp 0,
-  // Fvw and Q3's to warp 1 and Fuw's to warps 2 and 3, so that the four SM sub-partitions (warp w
-  // issues on sub-partition w mod 4) share them (FP32 RHS 0.242 -> 0.237 ms).  The FP64 form keeps
-  // them on the first threads (spread, it took 74 registers instead of 67 and 1.58 ms instead of
-  // 1.55).
+  // Every product loop has NT <= n < 2 NT items: thread tid takes item tid, and the n - NT items past
+  // NT go to the threads from `off` on: Fuv and Q1's extra items to warp 0, Fvw and Q3's to warp 1
+  // and Fuw's to warps 2 and 3, so that the four SM sub-partitions (warp w issues on sub-partition w
+  // mod 4) share them (0.242 -> 0.237 ms).
   constexpr int NT = RT_X * RT_Z;
   auto second = [&](int n, int off) {
     const int x = tid - off;
@@ -409,20 +386,15 @@ struct RhsTiledK {
         f = (P(1, jf, kk - 1, ii) + P(1, jf, kk, ii)) * (P(2, jf - 1, kk, ii) + rho * P(2, jf, kk, ii));
       S.fvw[jf & 1][kk][ii] = f;
     };
-    if constexpr (kHoist) {
-      const T* u0 = PL(0, jf - 1);
-      const T* u1 = PL(0, jf);
-      const T* v1 = PL(1, jf);
-      const T* w0 = PL(2, jf - 1);
-      const T* w1 = PL(2, jf);
-      (&S.fuv[jf & 1][0][0])[fA] = inner ? (u0[eA] + rho * u1[eA]) * (v1[eA - 1] + v1[eA]) : (T)0;
-      (&S.fvw[jf & 1][0][0])[fB] = inner ? (v1[eB - RT_PX] + v1[eB]) * (w0[eB] + rho * w1[eB]) : (T)0;
-      if (const int q = second(RT_Z * (RT_X + 1), 0); q >= 0) fuv_at(q);
-      if (const int q = second((RT_Z + 1) * RT_X, 32); q >= 0) fvw_at(q);
-    } else {
-      for (int q = tid; q < RT_Z * (RT_X + 1); q += NT) fuv_at(q);
-      for (int q = tid; q < (RT_Z + 1) * RT_X; q += NT) fvw_at(q);
-    }
+    const T* u0 = PL(0, jf - 1);
+    const T* u1 = PL(0, jf);
+    const T* v1 = PL(1, jf);
+    const T* w0 = PL(2, jf - 1);
+    const T* w1 = PL(2, jf);
+    (&S.fuv[jf & 1][0][0])[fA] = inner ? (u0[eA] + rho * u1[eA]) * (v1[eA - 1] + v1[eA]) : (T)0;
+    (&S.fvw[jf & 1][0][0])[fB] = inner ? (v1[eB - RT_PX] + v1[eB]) * (w0[eB] + rho * w1[eB]) : (T)0;
+    if (const int q = second(RT_Z * (RT_X + 1), 0); q >= 0) fuv_at(q);
+    if (const int q = second((RT_Z + 1) * RT_X, 32); q >= 0) fvw_at(q);
   };
   // centre-plane products of plane j (Q1, Q3, Fuw)
   auto centre_products = [&](int j) {
@@ -440,22 +412,16 @@ struct RhsTiledK {
       const int kk = q / (RT_X + 1), ii = q % (RT_X + 1);
       S.fuw[kk][ii] = (P(0, j, kk - 1, ii) + P(0, j, kk, ii)) * (P(2, j, kk, ii - 1) + P(2, j, kk, ii));
     };
-    if constexpr (kHoist) {
-      const T* u = PL(0, j);
-      const T* w = PL(2, j);
-      const T s1 = u[eA - 1] + u[eA];  // Q1 item: x = i0 - 1 + hi, z row hk
-      (&S.q1[0][0])[fA] = s1 * s1;
-      const T s3 = w[eB - RT_PX] + w[eB];  // Q3 item: z = k0 - 1 + gk
-      (&S.q3[0][0])[fB] = s3 * s3;
-      (&S.fuw[0][0])[fA] = (u[eA - RT_PX] + u[eA]) * (w[eA - 1] + w[eA]);
-      if (const int q = second(RT_Z * (RT_X + 1), 0); q >= 0) q1_at(q);
-      if (const int q = second((RT_Z + 1) * RT_X, 32); q >= 0) q3_at(q);
-      if (const int q = second((RT_Z + 1) * (RT_X + 1), 64); q >= 0) fuw_at(q);
-    } else {
-      for (int q = tid; q < RT_Z * (RT_X + 1); q += NT) q1_at(q);
-      for (int q = tid; q < (RT_Z + 1) * RT_X; q += NT) q3_at(q);
-      for (int q = tid; q < (RT_Z + 1) * (RT_X + 1); q += NT) fuw_at(q);
-    }
+    const T* u = PL(0, j);
+    const T* w = PL(2, j);
+    const T s1 = u[eA - 1] + u[eA];  // Q1 item: x = i0 - 1 + hi, z row hk
+    (&S.q1[0][0])[fA] = s1 * s1;
+    const T s3 = w[eB - RT_PX] + w[eB];  // Q3 item: z = k0 - 1 + gk
+    (&S.q3[0][0])[fB] = s3 * s3;
+    (&S.fuw[0][0])[fA] = (u[eA - RT_PX] + u[eA]) * (w[eA - 1] + w[eA]);
+    if (const int q = second(RT_Z * (RT_X + 1), 0); q >= 0) q1_at(q);
+    if (const int q = second((RT_Z + 1) * RT_X, 32); q >= 0) q3_at(q);
+    if (const int q = second((RT_Z + 1) * (RT_X + 1), 64); q >= 0) fuw_at(q);
   };
 
   // r = cn N + cp N_prev + cgx (p_i - p_{i-1}) + cx (f_{i+1} + f_{i-1}) + cz (f_{k+1} + f_{k-1})
@@ -463,36 +429,32 @@ struct RhsTiledK {
   // cn N is formed directly (the difference weights carry cn) and stored as the next N_prev
   auto K = [&](int q) -> T {
     const StepK& sk = Dyn ? *a.sk : a.kc;
-    if constexpr (sizeof(T) == 4) return sk.kf[q];
-    else return sk.kd[q];
+    return sk.kf[q];
   };
   const T qidx = K(RK_QIDX), qidz = K(RK_QIDZ);
   const T cp = K(RK_CP), cgx = K(RK_CGX), cgz = K(RK_CGZ), cx = K(RK_CX), cz = K(RK_CZ);
   const T cb = K(RK_CB);
   const bool use_prev = a.zet != 0.0;
   auto R = [&](int f, int jj) -> T {
-    if constexpr (sizeof(T) == 4) return __ldg(a.rtf + f * G + jj);
-    else return (T)__ldg(a.rt + f * G + jj);
+    return __ldg(a.rtf + f * G + jj);
   };
-  TR* ru = (TR*)a.ru;
-  TR* rv = (TR*)a.rv;
-  TR* rw = (TR*)a.rw;
-  TR* nu = (TR*)a.nu;
-  TR* nv = (TR*)a.nv;
-  TR* nw = (TR*)a.nw;
+  T* ru = (T*)a.ru;
+  T* rv = (T*)a.rv;
+  T* rw = (T*)a.rw;
+  T* nu = (T*)a.nu;
+  T* nv = (T*)a.nv;
+  T* nw = (T*)a.nw;
   const int i = i0 + tx, k = k0 + tz;
 
   // The per-row coefficients every thread of the block reads (R, and the face weights of the
   // y fluxes) are fetched by a few threads into a small ring in shared memory, one step ahead of
   // their use, instead of by every thread through the read-only path.
   auto fetch_face = [&](int jf) { S.wf[jf & 3] = (jf >= 1 && jf <= ny - 1) ? R(RT_RHO, jf) : (T)0; };
-  // prologue: planes jb-1, jb (jb+1 in flight); fluxes of face jb; Q2 of centre jb-1
+  // prologue: planes jb-1, jb; fluxes of face jb; Q2 of centre jb-1
   load_plane(jb - 1);
   load_plane(jb);
-  if (kAsync) cp_async_wait_all8();
   if (tid == 0) fetch_face(jb);
   __syncthreads();
-  if (kAsync) load_plane(jb + 1);
   face_fluxes(jb);
   T q2prev = 0;
   {
@@ -502,16 +464,14 @@ struct RhsTiledK {
   for (int j = jb; j <= jlast; ++j) {
     if (tid < RT_COUNT) S.rt[j & 3][tid] = R(tid, j);
     else if (tid == RT_COUNT) fetch_face(j + 1);
-    if (kAsync) cp_async_wait_all8();  // this thread's copies of plane j + 1
-    else load_plane(j + 1);
+    load_plane(j + 1);
     __syncthreads();
-    if (kAsync && j + 1 <= jlast) load_plane(j + 2);
     face_fluxes(j + 1);
     centre_products(j);
     __syncthreads();
     // The three components are assembled in one straight-line block (v also on the wall faces
     // and u, w also on the face row j = ny, where the planes read are zero and the results are
-    // not stored), so that the compiler can interleave their three FP64 chains.
+    // not stored), so that the compiler can interleave their three chains.
     const bool vrow = j > 0 && j < ny;  // interior v face
     const bool crow = j < ny;           // a row of cells
     const long cf = ((long)k * ny1 + j) * nx + i;
@@ -562,37 +522,594 @@ struct RhsTiledK {
         rw_ += cp * (T)nw[cc];
       }
     }
-    rv[cf] = vrow ? (TR)rv_ : (TR)0;
-    nv[cf] = vrow ? (TR)nvv : (TR)0;
+    rv[cf] = vrow ? rv_ : 0;
+    nv[cf] = vrow ? nvv : 0;
     if (crow) {
       const bool fixed = a.bl && i == 0;  // inflow face of u
-      ru[cc] = fixed ? (TR)0 : (TR)ru_;
-      nu[cc] = fixed ? (TR)0 : (TR)nuu;
-      rw[cc] = (TR)rw_;
-      nw[cc] = (TR)nww;
+      ru[cc] = fixed ? 0 : ru_;
+      nu[cc] = fixed ? 0 : nuu;
+      rw[cc] = rw_;
+      nw[cc] = nww;
     }
   }
 
   }
 };
 
+// ---------------------------------------------------------------------------------------------
+// The FP64 right-hand side in 64-bit fixed point (fx64.cuh).
+//
+// In FP64 arithmetic the tile was bound by the FP64 pipe: 64.8 instructions a cell of 16 cycles a
+// warp, 1.547 ms on 256 x 192 x 256 cells with the pipe 88 % busy.  Here the products and the viscous
+// sums run on the integer pipes; the FP64 pipe keeps 12 instructions a cell (pressure gradient, the
+// stored N, closing the sum): 0.737 ms, about 1000 instructions a cell and warp at 1.77 a cycle, bound
+// by the latency of their chains at 18 warps an SM (one cell a thread and twice the warps spilled at
+// 56 registers: 0.849 ms).  r is 3 to 10 times nearer to the exact sums than FP64 arithmetic was.
+//
+// A block marches a 32 x 16 (x, z) column along y.  The planes of u, v, w around the row stand in
+// shared memory as integers, each plane of each field scaled by its own largest magnitude in the
+// tile, so that 60 bits lie below the largest value near a cell (an FP64 result keeps 53 below its
+// own terms); p stands there in FP64.  Sums whose terms have different scales are sums of products
+// with coefficients into which the scales are folded (fx_wcoef).  One warp of the nine does nothing
+// else: it forms the coefficients of row j + 1, a term per lane and the scale of each sum from the
+// bounds of its terms, while the others (two cells in z a thread) work on row j.
+//
+// A row next to a plane of u, v or w that holds an infinity, a NaN or values near the ends of the
+// binary64 range is formed in FP64 arithmetic (rhs_cell).
+// ---------------------------------------------------------------------------------------------
+constexpr int FXR_X = 32, FXR_Z = 16;
+constexpr int FXR_PX = FXR_X + 2, FXR_PZ = FXR_Z + 2, FXR_PLANE = FXR_PX * FXR_PZ;
+constexpr int FXR_WARPS = FXR_Z / 2;  // worker warps, two z rows each; one more forms coefficients
+constexpr int FXR_THREADS = 32 * (FXR_WARPS + 1);
+
+struct RhsFxTile {
+  // u, v, w planes (ring of 5: three in use, one being converted, one arriving as FP64), p planes
+  // (ring of 3), index (kk + 1) * FXR_PX + ii + 1
+  fx_t pl[3][5][FXR_PLANE];
+  double pp[3][FXR_PLANE];
+  fx_t fuv[2][FXR_Z][FXR_X + 1];   // the products of RhsTile that neighbours share
+  fx_t fvw[2][FXR_Z + 1][FXR_X];
+  fx_t fuw[FXR_Z + 1][FXR_X + 1];
+  // by row parity: [3][4] terms of n (v, u, w), [3][8] terms of the viscous sums (5 used)
+  FxCoef cn[2][12], cr[2][24];
+  FxCoef cf[2][4];                 // face parity: weights of u_{j-1}, u_j, w_{j-1}, w_j
+  fx_t cb[2];                      // body force, at the scale of u's viscous sum
+  double cgy[2];                   // pressure weight of v (zero on the wall)
+  int en[2][4];                    // scales of n
+  double sr[2][4];                 // units of the viscous sums
+  int bad[2];                      // the row takes FP64 arithmetic
+  unsigned mag[4][4];              // largest high words of the planes (j mod 4) of u, v, w
+};
+
+__device__ __noinline__ void rhs_cell_fp64(const RhsArgs& a, int i, int j, int k) {
+  rhs_cell<double, double>(a, i, j, k, a.sk->dt);
+}
+
+struct RhsFxK {
+  struct Args {
+    RhsArgs a;
+    int jchunk;
+  };
+  static constexpr int kThreads = FXR_THREADS;
+  static constexpr int kMinBlocks = 2;  // shared memory holds two
+
+  // exponent of a plane (bit 62 of its integers); zero planes take the lowest, to raise no bound
+  static __device__ __forceinline__ int plane_e(unsigned m) { return (m == 0 ? 128 : (int)(m >> 20)) + 2; }
+  static __device__ __forceinline__ bool plane_ok(unsigned m) { return m == 0 || fx_exponent_ok((int)(m >> 20)); }
+
+  // ---- the coefficient warp ------------------------------------------------------------------
+  // One lane's term of a sum: the coefficient mult * p[J * stride] and the scale of its values,
+  // max(plane a, plane b) + max(plane c, plane d) + add, where a plane is field | (J offset + 1) << 2
+  // and code 15 stands for 0.
+  struct Term {
+    const double* p;
+    int stride;
+    double mult;
+    int a, b, c, d, add;
+  };
+  static __device__ __forceinline__ void coef_warp(const RhsArgs& a, RhsFxTile& S, int jb, int je) {
+    const int lane = threadIdx.x & 31, G = a.ny + 1, ny = a.ny;
+    const double* kd = a.sk->kd;
+    enum { U = 0, V = 1, W = 2, LO = 0, AT = 4, UP = 8, ZERO = 15 };
+    Term tn, tr;
+    auto none = [&](Term& t) {
+      t.p = kd;
+      t.stride = 0;
+      t.mult = 0.0;
+      t.a = t.b = U | AT;
+      t.c = t.d = ZERO;
+      t.add = 0;
+    };
+    none(tn);
+    none(tr);
+    {  // n: lanes 4 g + q
+      const int g = lane >> 2, q = lane & 3;
+      auto flux = [&](Term& t, int f, int at) {  // flux of f v on the face `at` rows above J
+        t.a = f | (at ? AT : LO);
+        t.b = f | (at ? UP : AT);
+        t.c = t.d = V | (at ? UP : AT);
+        t.add = -1022;
+      };
+      auto prod = [&](Term& t, int f, int h) {  // product of plane values of f and h
+        t.a = t.b = f | AT;
+        t.c = t.d = h | AT;
+        t.add = -1021;
+      };
+      if (g == 0) {
+        tn.mult = 1.0;
+        if (q == 0) tn.p = kd + RK_HIDX, flux(tn, U, 0);
+        if (q == 3) tn.p = kd + RK_HIDZ, flux(tn, W, 0);
+        if (q == 1 || q == 2) {  // squares of v at centres J and J - 1
+          tn.p = a.rt + RT_QIHC * G;
+          tn.stride = 1;
+          tn.mult = q == 1 ? 1.0 : -1.0;
+          tn.a = tn.c = V | (q == 1 ? AT : LO);
+          tn.b = tn.d = V | (q == 1 ? UP : AT);
+          tn.add = -1021;
+        }
+      } else if (g < 3) {
+        const int f = g == 1 ? U : W;
+        tn.mult = 1.0;
+        if (q == 0) tn.p = kd + RK_QIDX, prod(tn, U, f);
+        if (q == 3) tn.p = kd + RK_QIDZ, prod(tn, f, W);
+        if (q == 1 || q == 2) {  // y fluxes on faces J + 1 and J
+          tn.p = a.gc + GC_IDY * G;
+          tn.stride = 1;
+          tn.mult = (q == 1 ? 0.5 : -0.5) * kd[RK_CN];
+          flux(tn, f, q == 1);
+        }
+      }
+    }
+    const int gr = lane >> 3, qr = lane & 7;
+    if (gr < 3 && qr < 6) {  // viscous sums: lanes 8 g + q: x, z, centre, below, above; u: body force
+      const int f = gr == 0 ? V : gr == 1 ? U : W;
+      tr.a = tr.b = f | AT;
+      tr.mult = 1.0;
+      if (qr == 0) tr.p = kd + RK_CX;
+      if (qr == 1) tr.p = kd + RK_CZ;
+      if (qr >= 2 && qr < 5) {
+        const int row = gr == 0 ? (qr == 2 ? RT_DF : qr == 3 ? RT_AF : RT_CF) : (qr == 2 ? RT_DC : qr == 3 ? RT_AC : RT_CC);
+        tr.p = a.rt + row * G;
+        tr.stride = 1;
+        if (qr == 3) tr.a = tr.b = f | LO;
+        if (qr == 4) tr.a = tr.b = f | UP;
+      }
+      if (qr == 5) {
+        tr.mult = gr == 1 ? 1.0 : 0.0;
+        tr.p = kd + RK_CB;
+        tr.a = tr.b = ZERO;
+        tr.add = 1023;
+      }
+    }
+    auto scale = [&](const Term& t, int J) {
+      auto pe = [&](int s) { return s == ZERO ? 0 : plane_e(S.mag[(J - 1 + (s >> 2)) & 3][s & 3]); };
+      return max(pe(t.a), pe(t.b)) + max(pe(t.c), pe(t.d)) + t.add;
+    };
+    auto row = [&](int J) {  // planes J - 1 .. J + 1 are known
+      const int par = J & 1;
+      const bool wall = J == 0;  // v stays 0 there
+      double cn = tn.mult * __ldg(tn.p + (long)J * tn.stride), cr = tr.mult * __ldg(tr.p + (long)J * tr.stride);
+      if (wall && lane < 4) cn = 0.0;
+      if (wall && gr == 0) cr = 0.0;
+      const int etn = scale(tn, J), etr = scale(tr, J);
+      const int een = fx_wexp(cn, etn), eer = fx_wexp(cr, etr);
+      int mn = een, mr = eer;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        if (o < 4) mn = max(mn, __shfl_xor_sync(NS_FULL_MASK, mn, o));
+        mr = max(mr, __shfl_xor_sync(NS_FULL_MASK, mr, o));
+      }
+      unsigned pn = fx_wpart(cn, een, mn), pr = fx_wpart(cr, eer, mr);
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        if (o < 4) pn += __shfl_xor_sync(NS_FULL_MASK, pn, o);
+        pr += __shfl_xor_sync(NS_FULL_MASK, pr, o);
+      }
+      const int en = fx_wscale(mn, pn), er = fx_wscale(mr, pr);
+      bool ok = en >= 128 && en <= 1920 && er >= 128 && er <= 1920;
+      if (lane < 9) ok = ok && plane_ok(S.mag[(J - 1 + lane / 3) & 3][lane % 3]);
+      if (lane < 12) {
+        S.cn[par][lane] = een == FX_NONE ? FxCoef{0, 0} : fx_wcoef(cn, etn, en);
+        if ((lane & 3) == 0) S.en[par][lane >> 2] = en;
+      }
+      if (gr < 3) {
+        if (qr < 5) S.cr[par][lane] = eer == FX_NONE ? FxCoef{0, 0} : fx_wcoef(cr, etr, er);
+        if (qr == 0) S.sr[par][gr] = fx_unit(er);
+        if (lane == 13) S.cb[par] = eer == FX_NONE ? 0 : fx_from(cr, er);
+      }
+      const bool good = __all_sync(NS_FULL_MASK, ok);
+      if (lane == 0) {
+        S.bad[par] = !good;
+        S.cgy[par] = wall ? 0.0 : __ldg(a.rt + RT_CGY * G + J);
+      }
+    };
+    auto face = [&](int jf) {  // weights of the interpolation to face jf, brought to the larger scale
+      if (lane < 4) {
+        const int f = lane < 2 ? U : W;
+        FxCoef w{0, 0};  // no flux through the walls
+        if (jf >= 1 && jf <= ny - 1) {
+          const int e0 = plane_e(S.mag[(jf - 1) & 3][f]), e1 = plane_e(S.mag[jf & 3][f]);
+          w = fx_limbs(fx_from(__ldg(a.gc + ((lane & 1) ? GC_WHI : GC_WLO) * G + jf), 1023 + max(e0, e1) - ((lane & 1) ? e1 : e0)));
+        }
+        S.cf[jf & 1][lane] = w;
+      }
+    };
+    __syncthreads();
+    for (int j = jb - 1; j <= jb + 1; ++j) __syncthreads();
+    face(jb);
+    face(jb + 1);
+    row(jb);
+    __syncthreads();
+    for (int j = jb; j < je; ++j) {
+      __syncthreads();
+      if (lane < 4) S.mag[(j + 3) & 3][lane] = 0;  // plane j - 1 is done with
+      __syncthreads();
+      if (j + 1 < je) {
+        face(j + 2);
+        row(j + 1);
+      }
+    }
+  }
+
+  static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3) {
+    const RhsArgs& a = a_.a;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    RhsFxTile& S = *reinterpret_cast<RhsFxTile*>(smem_raw);
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const int tid = threadIdx.x, lane = tid & 31, wz = tid >> 5;
+    const int i0 = bid_.x * FXR_X, k0 = bid_.y * FXR_Z;
+    const int jb = bid_.z * a_.jchunk, je = min(jb + a_.jchunk, ny);
+    if (wz == FXR_WARPS) {
+      if (lane < 16) S.mag[lane >> 2][lane & 3] = 0;
+      coef_warp(a, S, jb, je);
+      return;
+    }
+    const int i = i0 + lane, kt = 2 * wz, k = k0 + kt;
+    const bool active0 = i < nx && k < nz, active1 = i < nx && k + 1 < nz;  // the last tiles may reach past the grid
+
+    // Plane positions of this thread: rows wz and wz + 8 of the 18, and a third: rows 16, 17 (warps
+    // 0, 1) or the halo columns (warps 2, 3).  gi = -2: nothing there.
+    int gk[3], gi[3], pos[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      int row = wz + 8 * r, ii = lane;
+      bool any = true;
+      if (r == 2 && wz >= 2) {
+        any = wz < 4 && lane < FXR_PZ;
+        row = any ? lane : 0;
+        ii = wz == 2 ? -1 : FXR_X;
+      }
+      const int kk = k0 + row - 1;
+      gk[r] = kk < 0 ? kk + nz : kk >= nz ? kk - nz : kk;
+      any = any && kk <= nz && i0 + ii <= nx;  // up to the wrapped neighbour
+      gi[r] = any ? i0 + ii : -2;
+      pos[r] = row * FXR_PX + ii + 1;
+      if (!a.bl) gi[r] = gi[r] == -1 ? nx - 1 : gi[r] == nx ? 0 : gi[r];
+    }
+    // Plane j of p starts on its way into slot sp
+    auto fetch_p = [&](int j, int sp) {
+      const bool jc = j >= 0 && j < ny;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        if (r == 2 && gi[r] == -2) continue;
+        const bool in = jc && gi[r] >= 0 && gi[r] < nx;
+        cp_async8(S.pp[sp] + pos[r], a.p + (in ? (long)(gk[r] * ny + j) * nx + gi[r] : 0), in);
+      }
+    };
+    // Plane j of u, v, w starts on its way into slot sl
+    auto fetch = [&](int j, int sl) {
+      const bool jc = j >= 0 && j < ny, jv = j >= 0 && j <= ny;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        if (r == 2 && gi[r] == -2) continue;
+        double* d[3] = {(double*)S.pl[0][sl] + pos[r], (double*)S.pl[1][sl] + pos[r], (double*)S.pl[2][sl] + pos[r]};
+        if (gi[r] >= 0 && gi[r] < nx) {
+          const long oc = (long)(gk[r] * ny + j) * nx + gi[r];
+          cp_async8(d[0], a.u + (jc ? oc : 0), jc);
+          cp_async8(d[1], a.v + (jv ? oc + (long)gk[r] * nx : 0), jv);
+          cp_async8(d[2], a.w + (jc ? oc : 0), jc);
+        } else {
+          // nothing, or an x-boundary halo: outflow plane of u, linear ghosts of v and w
+          const bool out = gi[r] == nx;
+          const int ib = out ? nx - 1 : 0;
+          double vu = 0.0, vv = 0.0, vw = 0.0;
+          if (jc && gi[r] != -2) {
+            const long q = (long)gk[r] * ny + j;
+            if (out) vu = __ldg(a.u_out + q);
+            vw = 2.0 * __ldg((out ? a.w_out : a.w_in) + q) - __ldg(a.w + q * nx + ib);
+          }
+          if (jv && gi[r] != -2) {
+            const long q = (long)gk[r] * (ny + 1) + j;
+            vv = 2.0 * __ldg((out ? a.v_out : a.v_in) + q) - __ldg(a.v + q * nx + ib);
+          }
+          *d[0] = vu;
+          *d[1] = vv;
+          *d[2] = vw;
+        }
+      }
+    };
+    double pv[3][3];  // this thread's values of the plane that has arrived
+    auto gather = [&](int j, int sl) {  // ... join the maxima of plane j
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        unsigned m = 0;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          pv[r][f] = r < 2 || gi[r] != -2 ? ((const double*)S.pl[f][sl])[pos[r]] : 0.0;
+          m = max(m, fx_mag(pv[r][f]));
+        }
+        m = __reduce_max_sync(NS_FULL_MASK, m);
+        if (lane == 0) atomicMax(&S.mag[j & 3][f], m);
+      }
+    };
+    auto convert = [&](int j, int sl) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const int s = plane_e(S.mag[j & 3][f]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+          if (r < 2 || gi[r] != -2) S.pl[f][sl][pos[r]] = fx_cut(pv[r][f], s);
+      }
+    };
+    // plane element (z row kk, column ii) of this thread's warp: kk relative to its first cell
+    const int e0 = (kt + 1) * FXR_PX + lane + 1;
+
+    // y-face fluxes of face jf, its planes jf - 1 and jf in slots sa and sb
+    auto face_fluxes = [&](int jf, int sa, int sb) {
+      const fx_t *u0 = S.pl[0][sa], *u1 = S.pl[0][sb], *v1 = S.pl[1][sb];
+      const fx_t *w0 = S.pl[2][sa], *w1 = S.pl[2][sb];
+      const FxCoef cu0 = S.cf[jf & 1][0], cu1 = S.cf[jf & 1][1], cw0 = S.cf[jf & 1][2], cw1 = S.cf[jf & 1][3];
+      auto uv = [&](int z, int x) {  // tile row z, column x
+        const int e = (z + 1) * FXR_PX + x + 1;
+        S.fuv[jf & 1][z][x] = fx_mulhi(fx_interpolate(u0[e], u1[e], cu0, cu1), v1[e - 1] + v1[e]);
+      };
+      auto vw = [&](int z, int x) {
+        const int e = (z + 1) * FXR_PX + x + 1;
+        S.fvw[jf & 1][z][x] = fx_mulhi(fx_interpolate(w0[e], w1[e], cw0, cw1), v1[e - FXR_PX] + v1[e]);
+      };
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uv(kt + c, lane);
+        vw(kt + c, lane);
+      }
+      if (wz == 4) vw(FXR_Z, lane);  // the extra row and column (warps 0 to 3 convert the halo)
+      if (wz == 5 && lane < FXR_Z) uv(lane, FXR_X);
+    };
+    // Fuw of the plane in slot sl
+    auto centre_products = [&](int sl) {
+      const fx_t *u = S.pl[0][sl], *w = S.pl[2][sl];
+      auto uw = [&](int z, int x) {
+        const int e = (z + 1) * FXR_PX + x + 1;
+        S.fuw[z][x] = fx_mulhi(u[e - FXR_PX] + u[e], w[e - 1] + w[e]);
+      };
+#pragma unroll
+      for (int c = 0; c < 2; ++c) uw(kt + c, lane);
+      if (wz == 6) uw(FXR_Z, lane);
+      if (wz == 7 && lane <= FXR_Z) uw(lane, FXR_X);
+    };
+    // (v_j + v_{j+1})^2 of the two cells' centres j, at the larger of the planes' scales
+    auto square_v = [&](int j, int sa, int sb, fx_t* q) {
+      const int ea = plane_e(S.mag[j & 3][1]), eb = plane_e(S.mag[(j + 1) & 3][1]), em = max(ea, eb);
+      const int da = min(em - ea, 63), db = min(em - eb, 63);
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        q[c] = fx_sqrhi((S.pl[1][sa][e0 + c * FXR_PX] >> da) + (S.pl[1][sb][e0 + c * FXR_PX] >> db));
+    };
+
+    // ---- prologue: planes jb - 1 .. jb + 1, then (coefficients) the fluxes of face jb.  Slots of planes
+    // j - 1, j, j + 1, j + 2, j + 3 and of p's planes j - 1, j:
+    int sm = 0, s0 = 1, s1 = 2, s2 = 3, s3 = 4, pm = 0, pc = 1, pn = 2;
+    __syncthreads();
+    for (int j = jb - 1; j <= jb + 1; ++j) {
+      const int q = j - jb + 1;
+      fetch(j, q);
+      if (q < 2) fetch_p(j, q);
+      cp_async_wait_all8();
+      gather(j, q);
+      __syncthreads();
+      convert(j, q);
+    }
+    if (jb + 1 < je) fetch(jb + 2, s2);
+    __syncthreads();
+    face_fluxes(jb, sm, s0);
+    fx_t q2prev[2] = {0, 0};
+    if (jb >= 1) square_v(jb - 1, sm, s0, q2prev);
+
+    const bool use_prev = a.zet != 0.0;
+    const double* kd = a.sk->kd;
+    const double cp = kd[RK_CP], cgx = kd[RK_CGX], cgz = kd[RK_CGZ];
+    double* __restrict__ ru = (double*)a.ru;
+    double* __restrict__ rv = (double*)a.rv;
+    double* __restrict__ rw = (double*)a.rw;
+    double* nu = (double*)a.nu;
+    double* nv = (double*)a.nv;
+    double* nw = (double*)a.nw;
+    const long sc = (long)ny * nx, sv = (long)(ny + 1) * nx;  // z strides
+    for (int j = jb; j < je; ++j) {
+      const bool next = j + 1 < je;  // another row follows
+      cp_async_wait_all8();
+      if (next) gather(j + 2, s2);
+      __syncthreads();
+      const long cc = ((long)k * ny + j) * nx + i, cf = cc + (long)k * nx;
+      if (next) {
+        convert(j + 2, s2);
+        if (j + 2 < je) fetch(j + 3, s3);
+        fetch_p(j + 1, pn);
+      }
+      double prev[3][2] = {};  // the stored N of the last sub-step (v, u, w)
+      if (use_prev) {
+        if (active0) {
+          prev[0][0] = nv[cf];
+          prev[1][0] = nu[cc];
+          prev[2][0] = nw[cc];
+        }
+        if (active1) {
+          prev[0][1] = nv[cf + sv];
+          prev[1][1] = nu[cc + sc];
+          prev[2][1] = nw[cc + sc];
+        }
+      }
+      face_fluxes(j + 1, s0, s1);
+      centre_products(s0);
+      fx_t q2[2];
+      square_v(j, s0, s1, q2);
+      __syncthreads();
+      const int par = j & 1, f0 = j & 1, f1 = f0 ^ 1;
+      if (S.bad[par]) {
+        if (active0) rhs_cell_fp64(a, i, j, k);
+        if (active1) rhs_cell_fp64(a, i, j, k + 1);
+      } else {
+        const FxCoef* cn = S.cn[par];
+        const FxCoef* cr = S.cr[par];
+        // The viscous sums of field f at the two cells; o: the plane's values (0, 1 the cells, 2, 3 the
+        // z neighbours below and above, 4, 5 and 6, 7 the x neighbours before and after)
+        auto viscous = [&](FxAcc* s, int f, const FxCoef* c, fx_t* o) {
+          const fx_t* p = S.pl[f][s0] + e0;
+          const fx_t *lo = S.pl[f][sm] + e0, *up = S.pl[f][s1] + e0;
+          o[0] = p[0];
+          o[1] = p[FXR_PX];
+          o[2] = p[-FXR_PX];
+          o[3] = p[2 * FXR_PX];
+          o[4] = p[-1];
+          o[5] = p[FXR_PX - 1];
+          o[6] = p[1];
+          o[7] = p[FXR_PX + 1];
+          const FxCoef wx = c[0], wz_ = c[1], wc = c[2], wl = c[3], wu = c[4];
+          fx_wmac(s[0], o[4] + o[6], wx);
+          fx_wmac(s[1], o[5] + o[7], wx);
+          fx_wmac(s[0], o[1] + o[2], wz_);
+          fx_wmac(s[1], o[3] + o[0], wz_);
+          fx_wmac(s[0], o[0], wc);
+          fx_wmac(s[1], o[1], wc);
+          fx_wfold(s[0]);
+          fx_wfold(s[1]);
+          fx_wmac(s[0], lo[0], wl);
+          fx_wmac(s[1], lo[FXR_PX], wl);
+          fx_wmac(s[0], up[0], wu);
+          fx_wmac(s[1], up[FXR_PX], wu);
+        };
+        const double* pj = S.pp[pc] + e0;
+        const double p0 = pj[0], p1 = pj[FXR_PX];
+        fx_t o[8];
+        double nd[3][2], rd[3][2];  // stored together at the end: the FP64 sums finish meanwhile
+        // ---------------- v at face j
+        {
+          FxAcc n[2] = {fx_wacc(0), fx_wacc(0)}, s[2] = {fx_wacc(0), fx_wacc(0)};
+          const fx_t wm = S.fvw[f0][kt][lane], w0 = S.fvw[f0][kt + 1][lane], wp = S.fvw[f0][kt + 2][lane];
+          fx_wmac(n[0], S.fuv[f0][kt][lane + 1] - S.fuv[f0][kt][lane], cn[0]);
+          fx_wmac(n[1], S.fuv[f0][kt + 1][lane + 1] - S.fuv[f0][kt + 1][lane], cn[0]);
+          fx_wmac(n[0], w0 - wm, cn[3]);
+          fx_wmac(n[1], wp - w0, cn[3]);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            fx_wmac(n[c], q2[c], cn[1]);
+            fx_wmac(n[c], q2prev[c], cn[2]);
+          }
+          viscous(s, 1, cr, o);
+          const double* pb = S.pp[pm] + e0;
+          const double cgy = S.cgy[par], sr = S.sr[par][0];
+          const int en = S.en[par][0];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            nd[0][c] = fx_to(fx_wsum(n[c]), en);
+            const double dp = (c ? p1 : p0) - pb[c * FXR_PX];
+            rd[0][c] = fma(fx_double(fx_wsum(s[c])), sr, fma(cgy, dp, fma(cp, prev[0][c], nd[0][c])));
+          }
+        }
+        // ---------------- u at (xf_i, yc_j, zc_k)
+        {
+          const fx_t cb = S.cb[par];
+          FxAcc n[2] = {fx_wacc(0), fx_wacc(0)}, s[2] = {fx_wacc(cb), fx_wacc(cb)};
+          const fx_t um = S.fuw[kt][lane], u0 = S.fuw[kt + 1][lane], up = S.fuw[kt + 2][lane];
+          fx_wmac(n[0], u0 - um, cn[7]);
+          fx_wmac(n[1], up - u0, cn[7]);
+          viscous(s, 0, cr + 8, o);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            fx_wmac(n[c], fx_sqrhi(o[c] + o[6 + c]) - fx_sqrhi(o[4 + c] + o[c]), cn[4]);
+            fx_wmac(n[c], S.fuv[f1][kt + c][lane], cn[5]);
+            fx_wmac(n[c], S.fuv[f0][kt + c][lane], cn[6]);
+          }
+          const double sr = S.sr[par][1];
+          const int en = S.en[par][1];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            nd[1][c] = fx_to(fx_wsum(n[c]), en);
+            const double dp = (c ? p1 : p0) - pj[c * FXR_PX - 1];
+            rd[1][c] = fma(fx_double(fx_wsum(s[c])), sr, fma(cgx, dp, fma(cp, prev[1][c], nd[1][c])));
+          }
+        }
+        // ---------------- w at (xc_i, yc_j, zf_k)
+        {
+          FxAcc n[2] = {fx_wacc(0), fx_wacc(0)}, s[2] = {fx_wacc(0), fx_wacc(0)};
+          viscous(s, 2, cr + 16, o);
+          const fx_t qm = fx_sqrhi(o[2] + o[0]), q0 = fx_sqrhi(o[0] + o[1]), qp = fx_sqrhi(o[1] + o[3]);
+          fx_wmac(n[0], q0 - qm, cn[11]);
+          fx_wmac(n[1], qp - q0, cn[11]);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            fx_wmac(n[c], S.fuw[kt + c][lane + 1] - S.fuw[kt + c][lane], cn[8]);
+            fx_wmac(n[c], S.fvw[f1][kt + c][lane], cn[9]);
+            fx_wmac(n[c], S.fvw[f0][kt + c][lane], cn[10]);
+          }
+          const double sr = S.sr[par][2];
+          const int en = S.en[par][2];
+          const double dp0 = p0 - pj[-FXR_PX], dp1 = p1 - p0;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            nd[2][c] = fx_to(fx_wsum(n[c]), en);
+            rd[2][c] = fma(fx_double(fx_wsum(s[c])), sr, fma(cgz, c ? dp1 : dp0, fma(cp, prev[2][c], nd[2][c])));
+          }
+        }
+        const bool wall = j == 0, fixed = a.bl && i == 0;  // the wall row of v, the inflow face of u
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          if (c ? active1 : active0) {
+            nv[cf + c * sv] = nd[0][c];
+            rv[cf + c * sv] = wall ? 0.0 : rd[0][c];
+            nu[cc + c * sc] = fixed ? 0.0 : nd[1][c];
+            ru[cc + c * sc] = fixed ? 0.0 : rd[1][c];
+            nw[cc + c * sc] = nd[2][c];
+            rw[cc + c * sc] = rd[2][c];
+          }
+      }
+      {  // the rings move on by one plane
+        const int t = sm;
+        sm = s0;
+        s0 = s1;
+        s1 = s2;
+        s2 = s3;
+        s3 = t;
+        pm = pc;
+        pc = pn;
+        pn = 3 - pm - pc;
+      }
+      q2prev[0] = q2[0];
+      q2prev[1] = q2[1];
+    }
+    if (je == ny) {  // the top wall row of v
+      const long cf = ((long)k * (ny + 1) + ny) * nx + i;
+      if (active0) nv[cf] = rv[cf] = 0.0;
+      if (active1) nv[cf + sv] = rv[cf + sv] = 0.0;
+    }
+  }
+};
+
 }  // namespace
 
-template <typename T, bool Dyn>
-cudaError_t rhs_attributes(int* bps) {
-  using K = RhsTiledK<T, T, Dyn>;
-  const cudaError_t e = set_smem_limit<K>((int)sizeof(RhsTile<T>));
+template <typename K>
+cudaError_t rhs_attributes(int* bps, size_t smem) {
+  const cudaError_t e = set_smem_limit<K>((int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, single_kernel<K>, RT_X * RT_Z, sizeof(RhsTile<T>));
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, single_kernel<K>, K::kThreads, smem);
 }
 
 cudaError_t rhs_set_attributes(int* bps) {
   cudaError_t e;
-  if ((e = rhs_attributes<double, false>(bps + 0)) != cudaSuccess ||
-      (e = rhs_attributes<double, true>(bps + 1)) != cudaSuccess ||
-      (e = rhs_attributes<float, false>(bps + 2)) != cudaSuccess)
+  if ((e = rhs_attributes<RhsFxK>(bps + 0, sizeof(RhsFxTile))) != cudaSuccess ||
+      (e = rhs_attributes<RhsTiledK<false>>(bps + 1, sizeof(RhsTile))) != cudaSuccess)
     return e;
-  return rhs_attributes<float, true>(bps + 3);
+  return rhs_attributes<RhsTiledK<true>>(bps + 2, sizeof(RhsTile));
 }
 
 cudaError_t launch_rhs(ns_ctx* c, int k) {
@@ -600,31 +1117,34 @@ cudaError_t launch_rhs(ns_ctx* c, int k) {
   return stage_rhs(s, k);
 }
 
-template <typename T, bool Dyn>
-cudaError_t emit_tiled(LaunchSink& s, const RhsArgs& a) {
-  // split y into chunks (each re-derives one face and two planes) so that the blocks fill whole
-  // waves of the resident capacity: minimise waves * (planes per chunk + prologue).  (Chunks of
-  // equal rows in one single wave, some spanning two tiles, were slower on both forms: neighbouring
-  // tiles then march at different y.)
-  ns_ctx* c = s.c;
-  const int tiles = (a.nx / RT_X) * (a.nz / RT_Z);
-  const int resident = c->num_sms * std::max(c->rhs_bps[(sizeof(T) == 4 ? 2 : 0) + (Dyn ? 1 : 0)], 1);
+// Rows of y a block marches: chunks (each re-derives one face and two or three planes) so that the
+// blocks fill whole waves of the resident capacity, minimising waves * (rows per chunk + prologue).
+// Small grids come down to a row or two a block: the march is one serial chain, and 64 x 64 x 32 cells
+// in chunks of six rows filled 44 of 152 SMs.  (Chunks of equal rows in one single wave, some spanning
+// two tiles, were slower: neighbouring tiles then march at different y.)
+int rhs_chunk(const ns_ctx* c, int tiles, int bps, double prologue) {
+  const int ny = c->cfg.ny, resident = c->num_sms * std::max(bps, 1);
   int best_nch = 1;
   double best = 1e300;
-  for (int nch = 1; nch <= (a.ny + 5) / 6 && nch <= 64; ++nch) {
-    const int jc = (a.ny + nch - 1) / nch;
-    const long nb = (long)tiles * ((a.ny + jc - 1) / jc);
+  for (int nch = 1; nch <= ny; ++nch) {
+    const int jc = (ny + nch - 1) / nch;
+    const long nb = (long)tiles * ((ny + jc - 1) / jc);
     const long waves = (nb + resident - 1) / resident;
-    const double cost = (double)waves * (jc + 2.0);
+    const double cost = (double)waves * (jc + prologue);
     if (cost < best - 1e-9) {
       best = cost;
       best_nch = nch;
     }
   }
-  const int jchunk = (a.ny + best_nch - 1) / best_nch;
-  const int nch = (a.ny + jchunk - 1) / jchunk;
-  return emit<RhsTiledK<T, T, Dyn>>(s, RhsTiledK<T, T, Dyn>::make(a, jchunk), dim3(a.nx / RT_X, a.nz / RT_Z, nch),
-                                    dim3(RT_X, RT_Z), sizeof(RhsTile<T>));
+  return (ny + best_nch - 1) / best_nch;
+}
+
+template <bool Dyn>
+cudaError_t emit_tiled(LaunchSink& s, const RhsArgs& a) {
+  using K = RhsTiledK<Dyn>;
+  const int jchunk = rhs_chunk(s.c, (a.nx / RT_X) * (a.nz / RT_Z), s.c->rhs_bps[Dyn ? 2 : 1], 2.0);
+  return emit<K>(s, K::make(a, jchunk), dim3(a.nx / RT_X, a.nz / RT_Z, (a.ny + jchunk - 1) / jchunk), dim3(RT_X, RT_Z),
+                 sizeof(RhsTile));
 }
 
 cudaError_t stage_rhs(LaunchSink& s, int k) {
@@ -665,18 +1185,15 @@ cudaError_t stage_rhs(LaunchSink& s, int k) {
   a.w_out = c->f.w_out;
   a.sk = c->stepk + k;
   a.kc = c->stepk_h[k];
-  if (a.nx % RT_X == 0 && a.nz % RT_Z == 0) {
-    if (c->cfg.precision == NS_MIXED)
-      return c->dyn_consts ? emit_tiled<float, true>(s, a) : emit_tiled<float, false>(s, a);
-    // FP64 always reads them from device memory: the register allocation of that variant is
-    // faster than the one with constant-bank operands on this kernel
-    return emit_tiled<double, true>(s, a);
+  if (c->cfg.precision != NS_MIXED) {
+    const int tx = (a.nx + FXR_X - 1) / FXR_X, tz = (a.nz + FXR_Z - 1) / FXR_Z;
+    const int jchunk = rhs_chunk(c, tx * tz, c->rhs_bps[0], 4.0);
+    return emit<RhsFxK>(s, RhsFxK::Args{a, jchunk}, dim3(tx, tz, (a.ny + jchunk - 1) / jchunk), dim3(FXR_THREADS),
+                        sizeof(RhsFxTile));
   }
+  if (a.nx % RT_X == 0) return c->dyn_consts ? emit_tiled<true>(s, a) : emit_tiled<false>(s, a);
   const long plane = (long)a.nx * (a.ny + 1);
   dim3 grid((unsigned)((plane + 127) / 128), (unsigned)a.nz);
-  if (c->cfg.precision == NS_MIXED)
-    return c->dyn_consts ? emit<RhsK<float, float, true>>(s, RhsK<float, float, true>::make(a), grid, 128, 0)
-                         : emit<RhsK<float, float, false>>(s, RhsK<float, float, false>::make(a), grid, 128, 0);
-  return c->dyn_consts ? emit<RhsK<double, double, true>>(s, RhsK<double, double, true>::make(a), grid, 128, 0)
-                       : emit<RhsK<double, double, false>>(s, RhsK<double, double, false>::make(a), grid, 128, 0);
+  return c->dyn_consts ? emit<RhsK<float, float, true>>(s, RhsK<float, float, true>::make(a), grid, 128, 0)
+                       : emit<RhsK<float, float, false>>(s, RhsK<float, float, false>::make(a), grid, 128, 0);
 }

@@ -329,7 +329,7 @@ struct ns_ctx {
   size_t dt_xs = 0, dt_ls = 0;
   std::vector<std::pair<size_t, size_t>> dirty;  // (workspace offset, bytes) written while staging
   int num_sms;
-  int rhs_bps[4];           // resident blocks per SM of the tiled RHS (FP64, FP64 dyn, FP32, FP32 dyn)
+  int rhs_bps[3];           // resident blocks per SM of the tiled RHS (FP64, FP32, FP32 dyn)
   // partitioned x solver
   int P, M, L[3];
   int part_req;             // NS_PART_AUTO / PPT / PDD

@@ -6,6 +6,7 @@ the same solve at ordinary magnitudes (fixed point) to the rounding of either.""
 import numpy as np
 import pytest
 
+from oracle import ns_oracle as O
 from paper_1812_01178_gb300 import binding as B
 from paper_1812_01178_gb300 import inputs as I
 
@@ -52,3 +53,91 @@ def test_poisson_of_zero_and_of_non_finite_fields(size):
         u2 = u.copy()
         u2[1, 2, 3] = bad
         assert np.isnan(_phi(case, u2, v, w, p)).any()
+
+
+def _rhs_all(s, k):
+    s.rhs(k)
+    s.sync()
+    return [s.buffer(b).cpu().numpy().copy() for b in (B.NS_BUF_RU, B.NS_BUF_RV, B.NS_BUF_RW, B.NS_BUF_NU,
+                                                       B.NS_BUF_NV, B.NS_BUF_NW)]
+
+
+def _rhs_oracle(case, fields, bl):
+    u, v, w, p = fields
+    g = O.Grid.from_case(case)
+    with np.errstate(all="ignore"):
+        if bl is not None:
+            r, n = O.rhs_bl(g, u, v, w, p, None, bl, 0, case.dt, case.re, case.fx)
+        else:
+            r, n = O.rhs(g, u, v, w, p, None, 0, case.dt, case.re, case.fx)
+        return list(r) + [-case.dt * O.RK3_GAMMA[0] * q for q in n]
+
+
+def _rhs_case(size, plate):
+    if plate:
+        case, u, v, w, p, bl = I.boundary_layer(*size, amp=0.05, seed=3, re=200.0)
+        return case, [u, v, w, p], bl
+    case, u, v, w, p = I.small_channel(*size, seed=5)
+    return case, [u, v, w, p], None
+
+
+# partial tiles in x (24, 48, 72) and z (8, 24), chunks of rows, single tiles, rows past several chunks
+RHS_SIZES = [(8, 5, 8), (24, 7, 16), (48, 6, 24), (72, 13, 8), (32, 4, 32), (96, 70, 48)]
+
+
+@pytest.mark.parametrize("plate", [False, True])
+@pytest.mark.parametrize("size", RHS_SIZES)
+def test_rhs_tiles_and_rows_of_unequal_size(size, plate):
+    """The fixed-point right-hand side on every kind of partial tile, with fields whose size changes by
+    1e12 over the rows and components 1e8 apart: row by row within the rounding of FP64 arithmetic on
+    the largest values the row reads (1e-12, as for the whole fields elsewhere)."""
+    case, f, bl = _rhs_case(size, plate)
+    ny = size[1]
+    row = 10.0 ** np.linspace(-9, 3, ny)
+    rowf = 10.0 ** np.linspace(-9, 3, ny + 1)
+    f[0] = f[0] * row[None, :, None]
+    f[1] = f[1] * rowf[None, :, None] * 1e-8
+    f[2] = f[2] * row[None, :, None] * 1e-4
+    f[3] = f[3] * row[None, :, None]
+    if bl is not None:
+        bl = dict(bl, u_out=f[0][:, :, -1].copy(), v_in=bl["v_in"] * rowf * 1e-8, v_out=f[1][:, :, -1].copy(),
+                  w_in=bl["w_in"] * row * 1e-4, w_out=f[2][:, :, -1].copy())
+    ref = _rhs_oracle(case, f, bl)
+    s = B.Solver(case, *f, bl=bl)
+    got = _rhs_all(s, 0)
+    s.close()
+    for q, (a, b) in enumerate(zip(got, ref)):
+        m = np.abs(b).max(axis=(0, 2))
+        near = np.maximum(m, np.maximum(np.r_[m[1:], 0.0], np.r_[0.0, m[:-1]]))
+        assert (np.abs(a - b).max(axis=(0, 2)) <= 1e-12 * near + 1e-300).all(), q
+
+
+@pytest.mark.parametrize("plate", [False, True])
+@pytest.mark.parametrize("size", RHS_SIZES)
+def test_rhs_outside_the_fixed_point_range(size, plate):
+    """Rows next to values outside the range: planes below 2^-895 and, at one cell, an infinity or a
+    NaN.  Cells that do not read it keep their values, those that do become non-finite where the
+    oracle's do."""
+    case, f, bl = _rhs_case(size, plate)
+    f[1] = f[1] * 1e-290
+    f[2][:, ::2] *= 1e-285
+    if bl is not None:
+        bl = dict(bl, v_in=bl["v_in"] * 1e-290, v_out=bl["v_out"] * 1e-290)
+        for q in ("w_in", "w_out"):
+            bl[q] = bl[q].copy()
+            bl[q][:, ::2] *= 1e-285
+    for bad in (None, np.nan, np.inf):
+        g = [a.copy() for a in f]
+        if bad is not None:
+            g[0][2, 2, 3] = bad
+        ref = _rhs_oracle(case, g, bl)
+        s = B.Solver(case, *g, bl=bl)
+        got = _rhs_all(s, 0)
+        s.close()
+        for q, (a, b) in enumerate(zip(got, ref)):
+            fin = np.isfinite(b)
+            if bad is not None:
+                assert not np.isfinite(a[~fin]).any(), q
+                fin[1:4, 1:4, 2:5] = False
+            scale = max(np.abs(b[fin]).max(), 1e-300)
+            assert np.abs(a[fin] - b[fin]).max() <= 1e-12 * scale, q
