@@ -85,13 +85,43 @@ FX_HD fx_t fx_from(double d, int s) {
 FX_HD double fx_to(fx_t x, int e) {
   const fx_t sg = x >> 63;
   const uint64_t m0 = (uint64_t)((x ^ sg) - sg);
-  const int lz = fx_clz(m0);
-  const uint64_t m = m0 << (lz & 63);
+  // 32-bit steps: normalise the high word, or the low one where that is zero
+  const bool low = (m0 >> 32) == 0;
+  unsigned th = low ? (unsigned)m0 : (unsigned)(m0 >> 32), tl = low ? 0u : (unsigned)m0;
+#ifdef __CUDA_ARCH__
+  const int n = __clz((int)th);
+  const bool zero = th == 0;
+  th = __funnelshift_l(tl, th, n);
+  tl <<= n & 31;
+  const unsigned bl = __funnelshift_r(tl, th, 11);
+#else
+  const bool zero = th == 0;
+  const int n = zero ? 0 : __builtin_clz(th);
+  const uint64_t m = (((uint64_t)th << 32) | tl) << n;
+  th = (unsigned)(m >> 32);
+  tl = (unsigned)m;
+  const unsigned bl = (unsigned)(m >> 11);
+#endif
   // 53 leading bits, rounded; the implicit bit and a carry out of the fraction add to the exponent
-  uint64_t b = ((uint64_t)(uint32_t)(e - lz) << 52) + (m >> 11) + ((m >> 10) & 1);
-  b = lz == 64 ? 0 : b;
+  const unsigned bh = (th >> 11) + ((unsigned)(e - n - (low ? 32 : 0)) << 20);
+  uint64_t b = (((uint64_t)bh << 32) | bl) + ((tl >> 10) & 1);
+  b = zero ? 0 : b;
   return fx_from_bits(b | ((uint64_t)sg & 0x8000000000000000ull));
 }
+
+// x as a double, rounded, by two FP64 instructions (the high limb scaled by 2^32 is exact)
+FX_HD double fx_double(fx_t x) {
+  const double h = fx_from_bits(0x4330000000000000ull | ((uint64_t)(x >> 32) & 0xffffffffull) ^ 0x80000000ull);
+  const double l = fx_from_bits(0x4330000000000000ull | (uint64_t)(uint32_t)x);
+  // h = 2^52 + 2^31 + hi, l = 2^52 + lo
+#ifdef __CUDA_ARCH__
+  return fma(h, 0x1p32, -(0x1p84 + 0x1p63 + 0x1p52)) + l;
+#else
+  return (h * 0x1p32 - (0x1p84 + 0x1p63 + 0x1p52)) + l;
+#endif
+}
+// the unit of a sum at scale e: 2^(e - 1023 - 62)
+FX_HD double fx_unit(int e) { return fx_from_bits((uint64_t)(uint32_t)(e - 62) << 52); }
 
 // Two signed limbs: x = h 2^32 + l, |l| <= 2^31.  Products drop l times l only, whose mean is zero: a
 // bias, however small, would add up in the lowest modes, which the pressure solve amplifies.
@@ -235,16 +265,3 @@ FX_HD fx_t fx_cut(double d, int s) {
   const fx_t sg = (fx_t)((int)hi >> 31);
   return (v ^ sg) - sg;
 }
-// x as a double, rounded, by two FP64 instructions (the high limb scaled by 2^32 is exact)
-FX_HD double fx_double(fx_t x) {
-  const double h = fx_from_bits(0x4330000000000000ull | ((uint64_t)(x >> 32) & 0xffffffffull) ^ 0x80000000ull);
-  const double l = fx_from_bits(0x4330000000000000ull | (uint64_t)(uint32_t)x);
-  // h = 2^52 + 2^31 + hi, l = 2^52 + lo
-#ifdef __CUDA_ARCH__
-  return fma(h, 0x1p32, -(0x1p84 + 0x1p63 + 0x1p52)) + l;
-#else
-  return (h * 0x1p32 - (0x1p84 + 0x1p63 + 0x1p52)) + l;
-#endif
-}
-// the unit of a sum at scale e: 2^(e - 1023 - 62)
-FX_HD double fx_unit(int e) { return fx_from_bits((uint64_t)(uint32_t)(e - 62) << 52); }

@@ -417,10 +417,26 @@ struct AdiLinePK {
   }
 };
 
+// Rows of a strided line stream through two register sets of U rows that take turns: while one is
+// swept the other's loads are in flight.  load(q, set) and sweep(q, set) handle rows q .. q + U - 1
+// of n (in sweep order); rows past n are theirs to skip.
+template <typename Set, int U, typename Load, typename Sweep>
+__device__ __forceinline__ void stream_rows(int n, Load load, Sweep sweep) {
+  Set A, B;
+  load(0, A);
+  for (int q = 0; q < n; q += 2 * U) {
+    load(q + U, B);
+    sweep(q, A);
+    load(q + 2 * U, A);
+    sweep(q + U, B);
+  }
+}
+
 // ----------------------------------------------------------------------------------------------
-// y: one thread per line, Thomas with precomputed factors [INV, AINV, CP][n]
+// y: one thread per line, Thomas with precomputed factors [INV, AINV, CP][n].  U: rows fetched ahead
+// (4: many lines, one set; 8: few lines, two sets, see deep_lines)
 // ----------------------------------------------------------------------------------------------
-template <typename T>
+template <typename T, int U>
 struct AdiYK {
   struct Args {
     T* ru;
@@ -432,8 +448,8 @@ struct AdiYK {
     int ny;
     int nz;
   };
-  static constexpr int kThreads = 128;
-  static constexpr int kMinBlocks = 12;  // room for the rows fetched ahead
+  static constexpr int kThreads = U == 4 ? 128 : 32;
+  static constexpr int kMinBlocks = U == 4 ? 12 : 1;  // room for the rows fetched ahead
   static Args make(T* ru, T* rv, T* rw, const T* tc, const T* tf, int nx, int ny, int nz) { return Args{ru, rv, rw, tc, tf, nx, ny, nz}; }
   static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3 gdim_) {
     T* __restrict__ ru = a_.ru;
@@ -443,7 +459,6 @@ struct AdiYK {
     const T* __restrict__ tf = a_.tf;
     int nx = a_.nx;
     int ny = a_.ny;
-    int nz = a_.nz;
 
   const int comp = bid_.z;
   const int i = bid_.x * blockDim.x + threadIdx.x;
@@ -464,8 +479,52 @@ struct AdiYK {
   const T* INV = tab;
   const T* AINV = tab + n;
   const T* CP = tab + 2 * n;
+  if constexpr (U > 4) {
+    struct Set {
+      T d[U], f[U], g[U];
+    };
+    T x = (T)0;
+    stream_rows<Set, U>(
+        n,
+        [&](int j0, Set& S) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (j0 + u < n) {
+              S.d[u] = line[(long)(j0 + u) * nx];
+              S.f[u] = __ldg(INV + j0 + u);
+              S.g[u] = __ldg(AINV + j0 + u);  // AINV[0] = 0
+            }
+        },
+        [&](int j0, const Set& S) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (j0 + u < n) {
+              x = S.d[u] * S.f[u] - S.g[u] * x;
+              line[(long)(j0 + u) * nx] = x;
+            }
+        });
+    const int m = n - 1;  // the last row is final
+    stream_rows<Set, U>(
+        m,
+        [&](int q, Set& S) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (q + u < m) {
+              S.d[u] = line[(long)(m - 1 - q - u) * nx];
+              S.f[u] = __ldg(CP + m - 1 - q - u);
+            }
+        },
+        [&](int q, const Set& S) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (q + u < m) {
+              x = S.d[u] - S.f[u] * x;
+              line[(long)(m - 1 - q - u) * nx] = x;
+            }
+        });
+    return;
+  }
   // rows are fetched U at a time ahead of the dependent recurrence (memory-level parallelism)
-  constexpr int U = 4;
   T prev = (T)0;
   for (int j0 = 0; j0 < n; j0 += U) {
     T dv[U];
@@ -499,7 +558,7 @@ struct AdiYK {
 // z: one thread per line, cyclic (Sherman-Morrison), then u* = u + delta.
 // table: [INV, AINV, CP, Q][nz] then (FAC, BG)
 // ----------------------------------------------------------------------------------------------
-template <typename T>
+template <typename T, int U>
 struct AdiZK {
   struct Args {
     T* ru;
@@ -513,8 +572,8 @@ struct AdiZK {
     int ny;
     int nz;
   };
-  static constexpr int kThreads = 128;
-  static constexpr int kMinBlocks = 10;  // room for the rows fetched ahead
+  static constexpr int kThreads = U == 4 ? 128 : 32;
+  static constexpr int kMinBlocks = U == 4 ? 10 : 1;  // room for the rows fetched ahead
   static Args make(T* ru, T* rv, T* rw, double* u, double* v, double* w, const T* tab, int nx, int ny, int nz) { return Args{ru, rv, rw, u, v, w, tab, nx, ny, nz}; }
   static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3 gdim_) {
     T* __restrict__ ru = a_.ru;
@@ -538,7 +597,6 @@ struct AdiZK {
   const long base = (long)j * nx + i;
   T* line = (comp == 0 ? ru : comp == 1 ? rv : rw) + base;
   double* f = (comp == 0 ? u : comp == 1 ? v : w) + base;
-  constexpr int U = 4;
   if constexpr (sizeof(T) == 8) {
     const T* Z = tab + 4 * nz + 2;
     if (__ldg(Z + 2) != 0.0) {  // uniform over the grid: the factorised circulant form (dt_ztab)
@@ -551,6 +609,51 @@ struct AdiZK {
       for (int q = 1; q <= NS_ZF_KMAX; ++q)
         if (q <= K) t = fma(__ldg(LP + q - 1), line[(long)(nz - q) * stride], t);
       line[0] = t;
+      struct Set {
+        double d[U], f[U];
+      };
+      if constexpr (U > 4) {
+        const int m = nz - 1;
+        stream_rows<Set, U>(
+            m,
+            [&](int q, Set& S) {
+#pragma unroll
+              for (int u = 0; u < U; ++u)
+                if (q + u < m) S.d[u] = line[(long)(1 + q + u) * stride];
+            },
+            [&](int q, const Set& S) {
+#pragma unroll
+              for (int u = 0; u < U; ++u)
+                if (q + u < m) {
+                  t = fma(lam, t, S.d[u]);
+                  line[(long)(1 + q + u) * stride] = t;
+                }
+            });
+        double x = t;
+#pragma unroll
+        for (int q = 1; q <= NS_ZF_KMAX; ++q)
+          if (q <= K) x = fma(__ldg(LP + q - 1), line[(long)(q - 1) * stride], x);
+        f[(long)m * stride] = fma(x, ia, f[(long)m * stride]);
+        stream_rows<Set, U>(
+            m,
+            [&](int q, Set& S) {
+#pragma unroll
+              for (int u = 0; u < U; ++u)
+                if (q + u < m) {
+                  S.d[u] = line[(long)(m - 1 - q - u) * stride];
+                  S.f[u] = f[(long)(m - 1 - q - u) * stride];
+                }
+            },
+            [&](int q, const Set& S) {
+#pragma unroll
+              for (int u = 0; u < U; ++u)
+                if (q + u < m) {
+                  x = fma(lam, x, S.d[u]);
+                  f[(long)(m - 1 - q - u) * stride] = fma(x, ia, S.f[u]);
+                }
+            });
+        return;
+      }
       for (int k0 = 1; k0 < nz; k0 += U) {
         double dv[U];
 #pragma unroll
@@ -763,18 +866,33 @@ cudaError_t launch_line_part(LaunchSink& s, int k, int P, int n) {
   }
 }
 
+// Whether the lines of a strided FP64 sweep are too few to hide its loads by occupancy: a thread then
+// fetches 8 rows ahead (y: with their factors) in two register sets instead of 4 in one, at the cost
+// of occupancy.  Measured at warps of lines per SM, us: y 1.3: 16.6 -> 14.6, 5.7: 24.7 -> 22.6, 7.6:
+// 34.9 -> 32.9, 15.2: 43.1 -> 59.2; z 0.3 (216 rows): 66.6 -> 45.1, 7.6: 90.4 -> 56.1, 10.1: 133.0 ->
+// 90.6, 11.8: 120.1 -> 84.3, 15.2: 87.0 -> 91.0.  The results are the same bit for bit; batched
+// launches fill the GPU together and keep the other form.
+bool deep_lines(const LaunchSink& s, long lines, long warps_per_sm) {
+  return !s.plan && lines < warps_per_sm * 32 * s.c->num_sms;
+}
+
 cudaError_t stage_adi_y(LaunchSink& s, int k) {
   ns_ctx* c = s.c;
   const int nx = c->cfg.nx, ny = c->cfg.ny, nz = c->cfg.nz;
   if (c->yP) return launch_line_part<false>(s, k, c->yP, ny);
   dim3 grid((nx + 127) / 128, nz, 3);
   if (c->cfg.precision == NS_MIXED)
-    return emit<AdiYK<float>>(s, AdiYK<float>::make((float*)c->ru, (float*)c->rv, (float*)c->rw,
-                                                    (const float*)c->ytab[k][0], (const float*)c->ytab[k][1], nx,
-                                                    ny, nz), grid, 128, 0);
-  return emit<AdiYK<double>>(s, AdiYK<double>::make((double*)c->ru, (double*)c->rv, (double*)c->rw,
-                                                    (const double*)c->ytab[k][0], (const double*)c->ytab[k][1],
-                                                    nx, ny, nz), grid, 128, 0);
+    return emit<AdiYK<float, 4>>(s, AdiYK<float, 4>::make((float*)c->ru, (float*)c->rv, (float*)c->rw,
+                                                          (const float*)c->ytab[k][0], (const float*)c->ytab[k][1],
+                                                          nx, ny, nz), grid, 128, 0);
+  const AdiYK<double, 4>::Args a = AdiYK<double, 4>::make((double*)c->ru, (double*)c->rv, (double*)c->rw,
+                                                          (const double*)c->ytab[k][0], (const double*)c->ytab[k][1],
+                                                          nx, ny, nz);
+  if (deep_lines(s, 3L * nx * nz, 8)) {
+    using D = AdiYK<double, 8>;
+    return emit<D>(s, D::make(a.ru, a.rv, a.rw, a.tc, a.tf, nx, ny, nz), dim3((nx + 31) / 32, nz, 3), 32, 0);
+  }
+  return emit<AdiYK<double, 4>>(s, a, grid, 128, 0);
 }
 
 cudaError_t stage_adi_z(LaunchSink& s, int k) {
@@ -783,11 +901,16 @@ cudaError_t stage_adi_z(LaunchSink& s, int k) {
   if (c->zP) return launch_line_part<true>(s, k, c->zP, nz);
   dim3 grid((nx + 127) / 128, ny, 3);
   if (c->cfg.precision == NS_MIXED)
-    return emit<AdiZK<float>>(s, AdiZK<float>::make((float*)c->ru, (float*)c->rv, (float*)c->rw, c->f.u, c->f.v,
-                                                    c->f.w, (const float*)c->ztab[k], nx, ny, nz), grid, 128, 0);
-  return emit<AdiZK<double>>(s, AdiZK<double>::make((double*)c->ru, (double*)c->rv, (double*)c->rw, c->f.u,
-                                                    c->f.v, c->f.w, (const double*)c->ztab[k], nx, ny, nz),
-                             grid, 128, 0);
+    return emit<AdiZK<float, 4>>(s, AdiZK<float, 4>::make((float*)c->ru, (float*)c->rv, (float*)c->rw, c->f.u,
+                                                          c->f.v, c->f.w, (const float*)c->ztab[k], nx, ny, nz),
+                                 grid, 128, 0);
+  const AdiZK<double, 4>::Args a = AdiZK<double, 4>::make((double*)c->ru, (double*)c->rv, (double*)c->rw, c->f.u,
+                                                          c->f.v, c->f.w, (const double*)c->ztab[k], nx, ny, nz);
+  if (deep_lines(s, 3L * nx * ny, 14)) {
+    using D = AdiZK<double, 8>;
+    return emit<D>(s, D::make(a.ru, a.rv, a.rw, a.u, a.v, a.w, a.tab, nx, ny, nz), dim3((nx + 31) / 32, ny, 3), 32, 0);
+  }
+  return emit<AdiZK<double, 4>>(s, a, grid, 128, 0);
 }
 
 cudaError_t launch_adi_x(ns_ctx* c, int k) {

@@ -233,6 +233,55 @@ __device__ __forceinline__ bool fx_loaded(const FxBlock& S, int nseq) {
   return ok;
 }
 
+// One radix-4 stage of power-of-two sequences (N = 2^a2, total butterflies over all sequences).
+// fx_slot is linear over exclusive or, and j, r N / 4 and r Ns have no bits in common with what they
+// are added to, so each thread takes the slot of its first element and flips the bits of the others.
+// RAW: the inputs are doubles (t0 as in fx_from); TW: twiddles; SH: the shift before the sums.
+template <int SIGN, bool RAW, bool TW, int SH>
+__device__ __forceinline__ unsigned fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, int total, int ls,
+                                              const FxTw* __restrict__ tw, const FxBlock& S) {
+  const int Ns = 1 << ls, quarter = 1 << (a2 - 2);
+  const int s1 = fx_slot(Ns), s2 = fx_slot(2 * Ns);
+  const int r1 = fx_slot(quarter), r2 = fx_slot(2 * quarter);
+  unsigned span = 0;
+  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    const int sq = idx >> (a2 - 2);
+    const int j = idx & (quarter - 1);
+    const int k = j & (Ns - 1);
+    const int base = sq * ld;
+    Fx2 x[4], y[4];
+    if (RAW) {
+      const int s = fx_exponent(S.emax[sq]) + 4;
+      const double2* X = reinterpret_cast<const double2*>(A) + base + j;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const double2 d = X[r * quarter];
+        x[r] = Fx2{fx_from(d.x, s), fx_from(d.y, s)};
+      }
+    } else {
+      const int q = fx_slot(j);
+      x[0] = A[base + q];
+      x[1] = A[base + (q ^ r1)];
+      x[2] = A[base + (q ^ r2)];
+      x[3] = A[base + (q ^ r1 ^ r2)];
+      if (TW) {
+        const FxTw* w = tw + 3 * (Ns + k);
+        x[0] = fx_shr(x[0], SH);
+#pragma unroll
+        for (int r = 1; r < 4; ++r) x[r] = fx_cmul<SIGN>(x[r], fx_ldtw(w + r - 1), SH);
+      }
+    }
+    fx_bfly4<SIGN>(x[0], x[1], x[2], x[3], y);
+    const int o = fx_slot(((j >> ls) << (ls + 2)) + k);
+    B[base + o] = y[0];
+    B[base + (o ^ s1)] = y[1];
+    B[base + (o ^ s2)] = y[2];
+    B[base + (o ^ s1 ^ s2)] = y[3];
+    span |= fx_span(y[0]) | fx_span(y[1]) | fx_span(y[2]) | fx_span(y[3]);
+  }
+  return span;
+}
+
 // FIRST: A holds doubles at [seq * ld + i], converted by the first stage; else fixed point at
 // [seq * ld + fx_slot(i)], at most 2^59.5 in modulus.  tw[3 (Ns + k) + r - 1]: the twiddle of input
 // r of a stage that follows sub-transforms of length Ns.  Returns the buffer of the result (fixed
@@ -288,8 +337,17 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
     unsigned span = 0;
     const int sh = first ? 0 : fx_stage_shift(S.span[stage - 1]);
     t += (FIRST && first) ? 4 : sh;
+    if (p2) {
+      span = first     ? fx_stage4<SIGN, FIRST, false, 0>(A, B, a2, ld, total, ls, tw, S)
+             : sh == 1 ? fx_stage4<SIGN, false, true, 1>(A, B, a2, ld, total, ls, tw, S)
+             : sh == 2 ? fx_stage4<SIGN, false, true, 2>(A, B, a2, ld, total, ls, tw, S)
+                       : fx_stage4<SIGN, false, true, 0>(A, B, a2, ld, total, ls, tw, S);
+      close(span);
+      first = false;
+      continue;
+    }
     for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-      const int sq = p2 ? idx >> (a2 - 2) : idx / quarter;
+      const int sq = idx / quarter;
       const int j = idx - sq * quarter;
       const int k = j & (Ns - 1);
       Fx2 x[4], y[4];
@@ -406,6 +464,8 @@ __device__ __noinline__ double2* plain_stockham(double2* A, double2* B, int N, i
   return A;
 }
 
+// q / N: a shift for powers of two
+__device__ __forceinline__ int fx_row(int q, int N, int plan) { return (plan >> 8) == 0 ? q >> (plan & 0xff) : q / N; }
 // max over the lanes of a warp that share lane mod n (n a power of two), then over warps into *slot
 __device__ __forceinline__ void fx_gather_max(unsigned m, int n, unsigned* slot) {
   for (int o = 16; o >= n; o >>= 1) m = max(m, __shfl_xor_sync(NS_FULL_MASK, m, o));
@@ -414,10 +474,10 @@ __device__ __forceinline__ void fx_gather_max(unsigned m, int n, unsigned* slot)
 // nseq rows of N elements, contiguous in memory, loaded by all threads: `at(row, i)` returns the
 // element, `put(row, i, v)` stores it; the rows' maxima go to S.emax
 template <typename At, typename Put>
-__device__ __forceinline__ void fx_load_rows(int nseq, int N, FxBlock& S, At at, Put put) {
+__device__ __forceinline__ void fx_load_rows(int nseq, int N, int plan, FxBlock& S, At at, Put put) {
   const bool whole = (N & 31) == 0;  // every warp's elements lie in one row
   for (int q = threadIdx.x; q < nseq * N; q += blockDim.x) {
-    const int r = q / N, i = q - r * N;
+    const int r = fx_row(q, N, plan), i = q - r * N;
     const double2 v = at(r, i);
     put(r, i, v);
     const unsigned m = max(fx_mag(v.x), fx_mag(v.y));
@@ -473,7 +533,7 @@ struct DivzK {
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FxBlock S;
-  const int nseq = TX >> 1, ld = nz + 1;
+  const int nseq = TX >> 1, ld = nz + 1, lt = __ffs(TX) - 1;  // TX is a power of two
   double2* A = reinterpret_cast<double2*>(smem_raw);
   double2* B = A + nseq * ld;
   const int i0 = bid_.x * TX;
@@ -487,8 +547,8 @@ struct DivzK {
   const long pl = (long)ny * nx, plv = (long)(ny + 1) * nx;
   unsigned mag = 0;  // of this thread's column (TX divides the block size)
   for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
-    const int il = q % TX;
-    const int k = q / TX;
+    const int il = q & (TX - 1);
+    const int k = q >> lt;
     const int i = i0 + il;
     const int ip = (i + 1 == nx) ? 0 : i + 1;
     const int kp = (k + 1 == nz) ? 0 : k + 1;
@@ -503,15 +563,15 @@ struct DivzK {
     slot[il & 1] = b;
     mag = max(mag, fx_mag(b));
   }
-  fx_gather_max(mag, TX, &S.emax[(threadIdx.x % TX) >> 1]);
+  fx_gather_max(mag, TX, &S.emax[(threadIdx.x & (TX - 1)) >> 1]);
   // unpack the two real transforms of each packed pair; write kz = 0..nz/2
   const int nh = (nz >> 1) + 1;
   if (fx_loaded(S, nseq)) {
     int t = 0;
     const Fx2* R = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, pz, nseq, twz, S, t);
     for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
-      const int il = q % TX;
-      const int m = q / TX;
+      const int il = q & (TX - 1);
+      const int m = q >> lt;
       const int c = il >> 1;
       const int e = fx_exponent(S.emax[c]) + t;
       const Fx2 zm = R[c * ld + fx_slot(m)];
@@ -523,8 +583,8 @@ struct DivzK {
   }
   const double2* R = plain_stockham<-1>(A, B, nz, ld, pz, nseq, twz);
   for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
-    const int il = q % TX;
-    const int m = q / TX;
+    const int il = q & (TX - 1);
+    const int m = q >> lt;
     const int c = il >> 1;
     const double2 zm = R[c * ld + m];
     const double2 zn = R[c * ld + (m == 0 ? 0 : nz - m)];
@@ -560,23 +620,23 @@ struct FftxK {
     const int nr = (int)min((long)R, a.nrows - row0);
     double2* g = a.spec + row0 * nx;
     fx_begin(S);
-    fx_load_rows(R, nx, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
+    fx_load_rows(R, nx, a.px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                  [&](int r, int i, double2 v) { A[r * ld + i] = v; });
     if (fx_loaded(S, R)) {
       int t = 0;
       const Fx2* X = fx_stockham<SIGN, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nx, ld, a.px, R,
                                              a.twx, S, t);
       for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-        const int r = q / nx, i = q - r * nx;
-        const int e = fx_exponent(S.emax[r]) + t;
+        const int r = fx_row(q, nx, a.px), i = q - r * nx;
+        const double e = fx_unit(fx_exponent(S.emax[r]) + t);
         const Fx2 v = X[r * ld + fx_slot(i)];
-        g[q] = make_double2(fx_to(v.x, e), fx_to(v.y, e));
+        g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
       }
       return;
     }
     const double2* X = plain_stockham<SIGN>(A, B, nx, ld, a.px, R, a.twx);
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-      const int r = q / nx, i = q - r * nx;
+      const int r = fx_row(q, nx, a.px), i = q - r * nx;
       g[q] = X[r * ld + i];
     }
   }
@@ -866,7 +926,7 @@ struct IfftzK {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ FxBlock S;
     const int nx = a.nx, ny = a.ny, nz = a.nz, TX = a.TX;
-    const int nseq = TX >> 1, ld = nz + 1;
+    const int nseq = TX >> 1, ld = nz + 1, lt = __ffs(TX) - 1;  // TX is a power of two
     double2* A = reinterpret_cast<double2*>(smem_raw);
     double2* B = A + nseq * ld;
     const int i0 = bid_.x * TX;
@@ -877,8 +937,8 @@ struct IfftzK {
     // m = nz/2 coefficients of a real sequence are real, so only their real parts are used.
     unsigned mag = 0;  // of this thread's sequence (nseq divides the block size)
     for (int q = threadIdx.x; q < nseq * (nh + 1); q += blockDim.x) {
-      const int c = q % nseq;
-      const int m = q / nseq;
+      const int c = q & (nseq - 1);
+      const int m = q >> (lt - 1);
       const long o = ((long)m * ny + j) * nx + i0 + 2 * c;
       double2 xa = a.spec[o];
       double2 xb = a.spec[o + 1];
@@ -895,24 +955,24 @@ struct IfftzK {
         mag = max(mag, max(fx_mag(y.x), fx_mag(y.y)));
       }
     }
-    fx_gather_max(mag, nseq, &S.emax[threadIdx.x % nseq]);
+    fx_gather_max(mag, nseq, &S.emax[threadIdx.x & (nseq - 1)]);
     const long pl = (long)ny * nx;
     if (fx_loaded(S, nseq)) {
       int t = 0;
       const Fx2* R = fx_stockham<1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, a.pz, nseq,
                                           a.twz, S, t);
       for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
-        const int il = q % TX;
-        const int k = q / TX;
+        const int il = q & (TX - 1);
+        const int k = q >> lt;
         const Fx2 v = R[(il >> 1) * ld + fx_slot(k)];
-        a.phi[k * pl + (long)j * nx + i0 + il] = fx_to((il & 1) ? v.y : v.x, fx_exponent(S.emax[il >> 1]) + t);
+        a.phi[k * pl + (long)j * nx + i0 + il] = fx_double((il & 1) ? v.y : v.x) * fx_unit(fx_exponent(S.emax[il >> 1]) + t);
       }
       return;
     }
     const double2* R = plain_stockham<1>(A, B, nz, ld, a.pz, nseq, a.twz);
     for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
-      const int il = q % TX;
-      const int k = q / TX;
+      const int il = q & (TX - 1);
+      const int k = q >> lt;
       const double2 v = R[(il >> 1) * ld + k];
       a.phi[k * pl + (long)j * nx + i0 + il] = (il & 1) ? v.y : v.x;
     }
@@ -952,7 +1012,7 @@ struct DivzMK {
   static __device__ __forceinline__ void run(const Args& a, const dim3 bid_, const dim3) {
     const int nx = a.nx, ny = a.ny, nz = a.nz, TX = a.TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nseq = TX >> 1;
+    const int nseq = TX >> 1, lt = __ffs(TX) - 1;  // TX is a power of two: no divisions
     float2* A = reinterpret_cast<float2*>(smem_raw);
     float2* B = A + nseq * nz;
     const int i0 = bid_.x * TX;
@@ -962,7 +1022,7 @@ struct DivzMK {
       const double scale = a.sk->pscale;
       const double idy = __ldg(a.gc + GC_IDY * (ny + 1) + j) * scale, idx = a.idx * scale, idz = a.idz * scale;
       for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
-        const int il = q % TX, k = q / TX, i = i0 + il;
+        const int il = q & (TX - 1), k = q >> lt, i = i0 + il;
         const int ip = (i + 1 == nx) ? 0 : i + 1;
         const int kp = (k + 1 == nz) ? 0 : k + 1;
         const long c = k * pl + (long)j * nx;
@@ -1004,7 +1064,7 @@ struct DivzMK {
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         const int q = min(q0 + g * (int)blockDim.x, nq - 1);
-        const int il = q % TX, k = q / TX, i = i0 + il;
+        const int il = q & (TX - 1), k = q >> lt, i = i0 + il;
         const long row = k * pl + (long)j * nx, cc = row + i;
         F0[g] = __ldg(f + cc);
         if (a.bl) {
@@ -1025,7 +1085,7 @@ struct DivzMK {
       for (int g = 0; g < G; ++g) {
         const int q = q0 + g * blockDim.x;
         if (q >= nq) break;
-        const int il = q % TX, k = q / TX;
+        const int il = q & (TX - 1), k = q >> lt;
         const float f0 = F0[g], fe = FE[g], fw = FW[g], fs = FS[g], fn = FN[g], fu = FU[g], fd = FD[g];
         float sxh, sxl, szh, szl;
         ff_two_sum(fe, fw, sxh, sxl);
@@ -1059,7 +1119,7 @@ struct DivzMK {
     const float2* R = stockham<-1, float2>(A, B, nz, a.pz, nseq, a.twz);
     const int nh = (nz >> 1) + 1;
     for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
-      const int il = q % TX, m = q / TX, c = il >> 1;
+      const int il = q & (TX - 1), m = q >> lt, c = il >> 1;
       const float2 zm = R[c * nz + m];
       const float2 zn = R[c * nz + (m == 0 ? 0 : nz - m)];
       const float2 X = (il & 1) == 0 ? make_float2(zm.x + zn.x, zm.y - zn.y) : make_float2(zm.y + zn.y, zn.x - zm.x);
@@ -1401,7 +1461,7 @@ struct IfftzMK {
   static __device__ __forceinline__ void run(const Args& a, const dim3 bid_, const dim3) {
     const int nx = a.nx, ny = a.ny, nz = a.nz, TX = a.TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nseq = TX >> 1;
+    const int nseq = TX >> 1, lt = __ffs(TX) - 1;  // TX is a power of two: no divisions
     float2* A = reinterpret_cast<float2*>(smem_raw);
     float2* B = A + nseq * nz;
     const int i0 = bid_.x * TX;
@@ -1415,14 +1475,14 @@ struct IfftzMK {
       if ((TX & 3) == 0) {
         const int pr = TX >> 2;  // 16-byte pieces per row
         for (int q = threadIdx.x; q < nz * pr; q += blockDim.x) {
-          const int k = q / pr, r = q - k * pr;
+          const int k = q >> (lt - 2), r = q & (pr - 1);
           cp_async16(reinterpret_cast<float4*>(P1 + k * TX) + r,
                      reinterpret_cast<const float4*>(a.phi1 + k * pl + (long)j * nx + i0) + r);
         }
         cp_async_commit();
       } else {
         for (int q = threadIdx.x; q < nz * TX; q += blockDim.x)
-          P1[q] = a.phi1[(q / TX) * pl + (long)j * nx + i0 + q % TX];
+          P1[q] = a.phi1[(q >> lt) * pl + (long)j * nx + i0 + (q & (TX - 1))];
       }
     }
     // spectrum loads in groups of four per thread, all issued before any is used
@@ -1434,7 +1494,7 @@ struct IfftzMK {
       for (int g = 0; g < G; ++g) {
         const int q = q0 + g * blockDim.x;
         if (q < nq) {
-          const int c = q % nseq, m = q / nseq;
+          const int c = q & (nseq - 1), m = q >> (lt - 1);
           const long o = ((long)m * ny + j) * nx + i0 + 2 * c;
           xa[g] = a.spec[o];
           xb[g] = a.spec[o + 1];
@@ -1444,7 +1504,7 @@ struct IfftzMK {
       for (int g = 0; g < G; ++g) {
         const int q = q0 + g * blockDim.x;
         if (q < nq) {
-          const int c = q % nseq, m = q / nseq;
+          const int c = q & (nseq - 1), m = q >> (lt - 1);
           if (m == 0 || m == nh) {
             xa[g].y = 0.0f;
             xb[g].y = 0.0f;
@@ -1458,7 +1518,7 @@ struct IfftzMK {
     __syncthreads();
     const float2* R = stockham<1, float2>(A, B, nz, a.pz, nseq, a.twz);
     for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
-      const int il = q % TX, k = q / TX;
+      const int il = q & (TX - 1), k = q >> lt;
       const float2 t = R[(il >> 1) * nz + k];
       const float val = (il & 1) ? t.y : t.x;
       const long cc = k * pl + (long)j * nx + i0 + il;
@@ -1586,7 +1646,7 @@ __global__ void __launch_bounds__(256, 3) dctx_fwd_kernel(double2* __restrict__ 
   const int nr = (int)min((long)R, nrows - row0);
   double2* g = spec + row0 * nx;
   fx_begin(S);
-  fx_load_rows(R, nx, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
+  fx_load_rows(R, nx, px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                [&](int r, int i, double2 v) { A[r * ld + ((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))] = v; });
   if (fx_loaded(S, R)) {
     int t = 0;
@@ -1594,20 +1654,20 @@ __global__ void __launch_bounds__(256, 3) dctx_fwd_kernel(double2* __restrict__ 
     // a, b = (V_l +- conj V_{N-l}) / 2 (b over i), times w_l
     const int sh = fx_stage_shift(S.span[fx_stages(px) - 1]);
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-      const int r = q / nx, l = q - r * nx;
+      const int r = fx_row(q, nx, px), l = q - r * nx;
       const Fx2 vl = fx_shr(V[r * ld + fx_slot(l)], 1);
       const Fx2 vn = fx_shr(V[r * ld + fx_slot(l == 0 ? 0 : nx - l)], 1);
       const FxTw w = fx_ldtw(twd + l);
-      const int e = fx_exponent(S.emax[r]) + t + sh;
+      const double e = fx_unit(fx_exponent(S.emax[r]) + t + sh);
       const Fx2 xa = fx_cmul<-1>(Fx2{vl.x + vn.x, vl.y - vn.y}, w, sh);
       const Fx2 xb = fx_cmul<-1>(Fx2{vl.y + vn.y, vn.x - vl.x}, w, sh);
-      g[q] = make_double2(fx_to(xa.x, e), fx_to(xb.x, e));
+      g[q] = make_double2(fx_double(xa.x) * e, fx_double(xb.x) * e);
     }
     return;
   }
   const double2* V = plain_stockham<-1>(A, B, nx, ld, px, R, twx);
   for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-    const int r = q / nx, l = q - r * nx;
+    const int r = fx_row(q, nx, px), l = q - r * nx;
     const double2 vl = V[r * ld + l];
     const double2 vn = V[r * ld + (l == 0 ? 0 : nx - l)];
     const double2 w = fx_twd(fx_ldtw(twd + l));
@@ -1628,12 +1688,12 @@ __global__ void __launch_bounds__(256, 3) dctx_inv_kernel(double2* __restrict__ 
   const int nr = (int)min((long)R, nrows - row0);
   double2* g = spec + row0 * nx;
   fx_begin(S);
-  fx_load_rows(R, nx, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
+  fx_load_rows(R, nx, px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                [&](int r, int i, double2 v) { A[r * ld + i] = v; });
   const bool ok = fx_loaded(S, R);
   // V_l = conj(w_l) (X_l - i X_{N-l})
   for (int q = threadIdx.x; q < R * nx; q += blockDim.x) {
-    const int r = q / nx, l = q - r * nx;
+    const int r = fx_row(q, nx, px), l = q - r * nx;
     const double2 xl = A[r * ld + l];
     const double2 xn = l == 0 ? make_double2(0.0, 0.0) : A[r * ld + nx - l];
     const FxTw w = fx_ldtw(twd + l);
@@ -1652,16 +1712,16 @@ __global__ void __launch_bounds__(256, 3) dctx_inv_kernel(double2* __restrict__ 
     int t = 5;
     const Fx2* X = fx_stockham<1, false>(reinterpret_cast<Fx2*>(B), reinterpret_cast<Fx2*>(A), nx, ld, px, R, twx, S, t);
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-      const int r = q / nx, i = q - r * nx;
-      const int e = fx_exponent(S.emax[r]) + t;
+      const int r = fx_row(q, nx, px), i = q - r * nx;
+      const double e = fx_unit(fx_exponent(S.emax[r]) + t);
       const Fx2 v = X[r * ld + fx_slot((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))];
-      g[q] = make_double2(fx_to(v.x, e), fx_to(v.y, e));
+      g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
     }
     return;
   }
   const double2* X = plain_stockham<1>(B, A, nx, ld, px, R, twx);
   for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-    const int r = q / nx, i = q - r * nx;
+    const int r = fx_row(q, nx, px), i = q - r * nx;
     g[q] = X[r * ld + ((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))];
   }
 }
