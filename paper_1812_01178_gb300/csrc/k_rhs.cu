@@ -1120,13 +1120,14 @@ cudaError_t launch_rhs(ns_ctx* c, int k) {
 // Rows of y a block marches: chunks (each re-derives one face and two or three planes) so that the
 // blocks fill whole waves of the resident capacity, minimising waves * (rows per chunk + prologue).
 // Small grids come down to a row or two a block: the march is one serial chain, and 64 x 64 x 32 cells
-// in chunks of six rows filled 44 of 152 SMs.  (Chunks of equal rows in one single wave, some spanning
+// in chunks of six rows filled 44 of 152 SMs.  least: the fewest rows of a chunk (batched instances fill
+// the GPU together and keep longer ones).  (Chunks of equal rows in one single wave, some spanning
 // two tiles, were slower: neighbouring tiles then march at different y.)
-int rhs_chunk(const ns_ctx* c, int tiles, int bps, double prologue) {
+int rhs_chunk(const ns_ctx* c, int tiles, int bps, double prologue, int least) {
   const int ny = c->cfg.ny, resident = c->num_sms * std::max(bps, 1);
   int best_nch = 1;
   double best = 1e300;
-  for (int nch = 1; nch <= ny; ++nch) {
+  for (int nch = 1; nch <= ny && (nch == 1 || (ny + nch - 1) / nch >= least); ++nch) {
     const int jc = (ny + nch - 1) / nch;
     const long nb = (long)tiles * ((ny + jc - 1) / jc);
     const long waves = (nb + resident - 1) / resident;
@@ -1142,7 +1143,7 @@ int rhs_chunk(const ns_ctx* c, int tiles, int bps, double prologue) {
 template <bool Dyn>
 cudaError_t emit_tiled(LaunchSink& s, const RhsArgs& a) {
   using K = RhsTiledK<Dyn>;
-  const int jchunk = rhs_chunk(s.c, (a.nx / RT_X) * (a.nz / RT_Z), s.c->rhs_bps[Dyn ? 2 : 1], 2.0);
+  const int jchunk = rhs_chunk(s.c, (a.nx / RT_X) * (a.nz / RT_Z), s.c->rhs_bps[Dyn ? 2 : 1], 2.0, s.plan ? 6 : 1);
   return emit<K>(s, K::make(a, jchunk), dim3(a.nx / RT_X, a.nz / RT_Z, (a.ny + jchunk - 1) / jchunk), dim3(RT_X, RT_Z),
                  sizeof(RhsTile));
 }
@@ -1187,7 +1188,7 @@ cudaError_t stage_rhs(LaunchSink& s, int k) {
   a.kc = c->stepk_h[k];
   if (c->cfg.precision != NS_MIXED) {
     const int tx = (a.nx + FXR_X - 1) / FXR_X, tz = (a.nz + FXR_Z - 1) / FXR_Z;
-    const int jchunk = rhs_chunk(c, tx * tz, c->rhs_bps[0], 4.0);
+    const int jchunk = rhs_chunk(c, tx * tz, c->rhs_bps[0], 4.0, s.plan ? 6 : 1);
     return emit<RhsFxK>(s, RhsFxK::Args{a, jchunk}, dim3(tx, tz, (a.ny + jchunk - 1) / jchunk), dim3(FXR_THREADS),
                         sizeof(RhsFxTile));
   }
