@@ -187,7 +187,11 @@ __device__ C* stockham(C* A, C* B, int N, int plan, int nseq, const C* __restric
 // on the integer pipes (fx64.cuh).  In FP64 arithmetic they ran at 0.86-0.9 of the FP64 pipe's rate
 // (22 instructions of 16 cycles a warp per radix-4 butterfly); in fixed point a butterfly is 36
 // multiply-adds of about 1.3 cycles and some 100 additions, shifts and logic operations on the
-// other pipes.  Every sequence is scaled by its own largest component; before each stage the block
+// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 216 (six FP64
+// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 117, inverse z 295 ->
+// 135; bound by instruction issue and latency (2.1 instructions a cycle at 32 warps an SM).  Results
+// go back to FP64 by two exact FP64 instructions and a scaling on the otherwise idle pipe (x,
+// inverse z), or by integer steps (after the divergence, which uses that pipe).  Every sequence is scaled by its own largest component; before each stage the block
 // shifts by 0, 1 or 2 bits, as its largest value (the or of all magnitudes, gathered while the last
 // stage was written) needs for the next sums to stay below 2^62.  The result is nearer to the exact
 // transform than FP64 butterflies were, at every length and shape of data tried (2 to 4 times on
@@ -512,7 +516,7 @@ struct DivzK {
     const double* u_out;
   };
   static constexpr int kThreads = 256;
-  static constexpr int kMinBlocks = 3;  // shared memory holds three
+  static constexpr int kMinBlocks = 4;  // 64 registers; shared memory holds four (pois_shape)
   static Args make(const double* u, const double* v, const double* w, const double* gc, const FxTw* twz, double2* spec, int nx, int ny, int nz, int pz, int TX, double idx, double idz, const StepK* sk, const double* u_out) { return Args{u, v, w, gc, twz, spec, nx, ny, nz, pz, TX, idx, idz, sk, u_out}; }
   static __device__ __forceinline__ void run(const Args& a_, const dim3 bid_, const dim3 gdim_) {
     const double* __restrict__ u = a_.u;
@@ -609,7 +613,7 @@ struct FftxK {
     int R;
   };
   static constexpr int kThreads = 256;
-  static constexpr int kMinBlocks = 3;  // shared memory holds three
+  static constexpr int kMinBlocks = 4;  // 64 registers; shared memory holds four (pois_shape)
   static __device__ __forceinline__ void run(const Args& a, const dim3 bid_, const dim3) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ FxBlock S;
@@ -921,7 +925,7 @@ struct IfftzK {
     int TX;
   };
   static constexpr int kThreads = 256;
-  static constexpr int kMinBlocks = 3;  // shared memory holds three
+  static constexpr int kMinBlocks = 4;  // 64 registers; shared memory holds four (pois_shape)
   static __device__ __forceinline__ void run(const Args& a, const dim3 bid_, const dim3) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ FxBlock S;
@@ -1634,7 +1638,7 @@ struct ProjectK {
 // absorb the 1/2 of the real / imaginary separation exactly (a power of two).
 // ------------------------------------------------------------------------------------------
 // The FP64 form: transforms and twiddles in fixed point (general path: FP64).  twd: FxTw of w_l.
-__global__ void __launch_bounds__(256, 3) dctx_fwd_kernel(double2* __restrict__ spec, const FxTw* __restrict__ twx,
+__global__ void __launch_bounds__(256, 4) dctx_fwd_kernel(double2* __restrict__ spec, const FxTw* __restrict__ twx,
                                                           const FxTw* __restrict__ twd, long nrows, int nx, int px,
                                                           int R) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1676,7 +1680,7 @@ __global__ void __launch_bounds__(256, 3) dctx_fwd_kernel(double2* __restrict__ 
   }
 }
 
-__global__ void __launch_bounds__(256, 3) dctx_inv_kernel(double2* __restrict__ spec, const FxTw* __restrict__ twx,
+__global__ void __launch_bounds__(256, 4) dctx_inv_kernel(double2* __restrict__ spec, const FxTw* __restrict__ twx,
                                                           const FxTw* __restrict__ twd, long nrows, int nx, int px,
                                                           int R) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2050,19 +2054,23 @@ cudaError_t launch_pois_factor(ns_ctx* c, const double* lamx, const double* lamz
   return cudaGetLastError();
 }
 
+// Columns of a z-transform tile (a power of two): two buffers of TX / 2 sequences within 36 KB, so that
+// registers, not shared memory, set the four blocks of an SM (nz = 256: 8 columns instead of 16,
+// divergence + z 235 -> 216 us), but at least 8 columns, then 4, while that stays within 68 KB (nz =
+// 512: 4 columns, 32-byte rows, took 2.53 ms against 2.20 at 8 and three blocks).
 static int z_tile(int nz) {
-  // complex sequences of length nz: keep 2 * (TX/2) * nz * 16 B <= 64 KB
   int tx = 16;
-  while (tx > 2 && (size_t)tx * nz * 16 > 64 * 1024) tx >>= 1;
+  while (tx > 8 && (size_t)tx * (nz + 1) * 16 > 36 * 1024) tx >>= 1;
+  while (tx > 2 && (size_t)tx * (nz + 1) * 16 > 68 * 1024) tx >>= 1;
   return tx;
 }
 
 namespace {
 struct PoisShape {
-  int nx, ny, nz, pz, px, TX, R, TXm;
+  int nx, ny, nz, pz, px, TX, R, Rm, TXm;
   size_t smz, smx, smxm;
   long nrows;
-  unsigned bx;
+  unsigned bx, bxm;
 };
 PoisShape pois_shape(const ns_ctx* c) {
   PoisShape q;
@@ -2083,11 +2091,16 @@ PoisShape pois_shape(const ns_ctx* c) {
   if (q.TXm < 8 && (size_t)8 * q.nz * 8 <= 160 * 1024) q.TXm = 8;
   while (q.nx % q.TXm) q.TXm >>= 1;
   q.nrows = (long)c->nzh * q.ny;
-  q.R = 1;
-  while (q.R < 16 && (size_t)2 * q.R * 2 * q.nx * sizeof(double2) <= 64 * 1024) q.R <<= 1;
+  // rows of an x-transform block: two buffers within 56 KB (four blocks of an SM; three of 64 KB and 80
+  // registers: 129 -> 117 us at nx = 256)
+  q.R = std::max(1, std::min(FX_SEQ, (int)(56 * 1024 / (2 * (q.nx + 1) * sizeof(double2)))));
   q.smx = (size_t)2 * q.R * (q.nx + 1) * sizeof(double2);
-  q.smxm = (size_t)2 * q.R * q.nx * sizeof(float2);
   q.bx = (unsigned)((q.nrows + q.R - 1) / q.R);
+  // ... in the mixed form (complex64, 32 KB)
+  q.Rm = 1;
+  while (q.Rm < 16 && (size_t)2 * q.Rm * 2 * q.nx * sizeof(double2) <= 64 * 1024) q.Rm <<= 1;
+  q.smxm = (size_t)2 * q.Rm * q.nx * sizeof(float2);
+  q.bxm = (unsigned)((q.nrows + q.Rm - 1) / q.Rm);
   return q;
 }
 // the mixed form's FP32 pipeline: spectrum (complex64) over the dead increments r_u, r_v; phi1 in
@@ -2131,17 +2144,17 @@ cudaError_t emit_xm(LaunchSink& s, bool fwd) {
   const PoisShape q = pois_shape(c);
   if (c->bl) {
     if (fwd)
-      dctx_fwd_m_kernel<<<q.bx, 256, q.smxm, c->launch>>>(sp32(c), c->twx32, c->twd32, q.nrows, q.nx, q.px, q.R);
+      dctx_fwd_m_kernel<<<q.bxm, 256, q.smxm, c->launch>>>(sp32(c), c->twx32, c->twd32, q.nrows, q.nx, q.px, q.Rm);
     else
-      dctx_inv_m_kernel<<<q.bx, 256, q.smxm, c->launch>>>(sp32(c), c->twx32, c->twd32, q.nrows, q.nx, q.px, q.R);
+      dctx_inv_m_kernel<<<q.bxm, 256, q.smxm, c->launch>>>(sp32(c), c->twx32, c->twd32, q.nrows, q.nx, q.px, q.Rm);
     return cudaGetLastError();
   }
   if (s.plan) {  // batched ensembles: many small instances fill the GPU with one batch per block
     if (fwd)
-      return emit<FftxMK<-1>>(s, FftxMK<-1>::Args{sp32(c), c->twx32, q.nrows, q.nx, q.px, q.R},
-                                     dim3(q.bx), dim3(256), q.smxm);
-    return emit<FftxMK<1>>(s, FftxMK<1>::Args{sp32(c), c->twx32, q.nrows, q.nx, q.px, q.R},
-                                  dim3(q.bx), dim3(256), q.smxm);
+      return emit<FftxMK<-1>>(s, FftxMK<-1>::Args{sp32(c), c->twx32, q.nrows, q.nx, q.px, q.Rm},
+                                     dim3(q.bxm), dim3(256), q.smxm);
+    return emit<FftxMK<1>>(s, FftxMK<1>::Args{sp32(c), c->twx32, q.nrows, q.nx, q.px, q.Rm},
+                                  dim3(q.bxm), dim3(256), q.smxm);
   }
   // single instance: persistent, double-buffered: R rows per batch with 4 buffers of R nx float2
   // in shared memory
