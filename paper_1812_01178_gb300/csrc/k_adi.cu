@@ -108,6 +108,78 @@ __device__ __forceinline__ void store_part(T* __restrict__ dst, const T (&d)[M])
   }
 }
 
+// ----------------------------------------------------------------------------------------------
+// x lines in 64-bit fixed point (fx64.cuh), beside the FP64 ones.  The FP64 x sweep was bound by the
+// FP64 pipe (four instructions an element of 16 cycles a warp); the same algebra in fixed point, each
+// line scaled by its own largest magnitude (the solutions of these diagonally dominant rows stay
+// below it), takes about 35 cycles of the integer pipes.  Neither alone is much faster, but the pipes
+// are different: of every eight groups of lines the first four go the fixed-point way (warps 0 to 3 of
+// a block, one on each SM sub-partition), the others the FP64 way.  The choice depends on the group's
+// number alone, so that every launch form solves a line alike.
+// ----------------------------------------------------------------------------------------------
+// (256 x 192 x 256: no group in fixed point 286 us, four of eight 186, five 194, six 195, all 222)
+__device__ __forceinline__ bool x_fixed_group(long g) { return (g & 7) < 4; }
+// An entry of the x tables as a coefficient; *ok turns false for magnitudes above 1
+__device__ __forceinline__ FxCoef x_coef(double c, bool* ok) {
+  const double m = fabs(c);
+  if (!(m <= 1.0)) *ok = false;
+  if (m < 1.0) return fx_limbs(fx_from(c, 1023));
+  const fx_t one = ((fx_t)1 << 62) - 1;
+  return fx_limbs(c < 0.0 ? -one : one);
+}
+// x w of |w| <= 1, sums of two such products, and the sum of two products with halved coefficients
+__device__ __forceinline__ fx_t x_mul(fx_t x, FxCoef w) {
+  FxAcc s = {0, (fx_t)1 << 29};
+  fx_wmac(s, x, w);
+  return s.h * 4 + (s.m >> 30);
+}
+__device__ __forceinline__ fx_t x_mul2(fx_t x, FxCoef w, fx_t y, FxCoef v) {
+  FxAcc s = {0, (fx_t)1 << 29};
+  fx_wmac(s, x, w);
+  fx_wmac(s, y, v);
+  return s.h * 4 + (s.m >> 30);
+}
+__device__ __forceinline__ fx_t x_mul2h(fx_t x, FxCoef w, fx_t y, FxCoef v) {
+  FxAcc s = {0, (fx_t)1 << 28};
+  fx_wmac(s, x, w);
+  fx_wmac(s, y, v);
+  return s.h * 8 + (s.m >> 29);
+}
+// One partition (lane r of a team of P) of a line by PDD, in place; F: the coefficients of its table
+// in the x-table layout, AINV, CP, V and W negated, the interface inverses halved; e: the line's exponent
+template <int M>
+__device__ __forceinline__ void x_solve_fixed(double (&d)[M], const FxCoef* F, int e, int r, int P, bool half) {
+  const FxCoef* INV = F + XT_INV * M * P + r;
+  const FxCoef* AINV = F + XT_AINV * M * P + r;
+  const FxCoef* CP = F + XT_CP * M * P + r;
+  const FxCoef* SV = F + XT_V * M * P + r;
+  const FxCoef* SW = F + XT_W * M * P + r;
+  const FxCoef* DINV = F + XT_NF * M * P + r;
+  const int s = e + 2;
+  fx_t q[M];
+  q[0] = x_mul(fx_cut(d[0], s), INV[0]);
+#pragma unroll
+  for (int i = 1; i < M; ++i) q[i] = x_mul2(fx_cut(d[i], s), INV[i * P], q[i - 1], AINV[i * P]);
+#pragma unroll
+  for (int i = M - 2; i >= 0; --i) q[i] += x_mul(q[i + 1], CP[i * P]);
+  const fx_t g0 = q[M - 1];
+  const fx_t g1 = __shfl_sync(NS_FULL_MASK, q[0], r + 1, P);
+  const fx_t y0 = x_mul2h(g0, DINV[0], g1, DINV[P]);
+  const fx_t y1 = x_mul2h(g0, DINV[2 * P], g1, DINV[3 * P]);
+  const fx_t left = __shfl_sync(NS_FULL_MASK, y0, r - 1 + P, P);
+  if (half) {
+#pragma unroll
+    for (int i = 0; i < M / 2; ++i) d[i] = fx_to(q[i] + x_mul(left, SV[i * P]), s);
+#pragma unroll
+    for (int i = M / 2; i < M; ++i) d[i] = fx_to(q[i] + x_mul(y1, SW[i * P]), s);
+  } else {
+#pragma unroll
+    for (int i = 0; i < M; ++i) d[i] = fx_to(q[i] + x_mul2(left, SV[i * P], y1, SW[i * P]), s);
+  }
+}
+// entries of the fixed-point part of an x table
+__host__ __device__ inline int x_fixed_count(int M, int P) { return (XT_NF * M + 4) * P; }
+
 template <typename T, int M>
 struct AdiXK {
   struct Args {
@@ -127,6 +199,20 @@ struct AdiXK {
   const int ntab = (int)xtab_count(M, P, L);
   const int ncls = a.bl ? 2 : 1;
   for (int q = threadIdx.x; q < ntab * ncls; q += blockDim.x) st[q] = q < ntab ? a.tab[0][q] : a.tab[1][q - ntab];
+  bool fixed = sizeof(T) == 8 && L == 0;  // fixed point: FP64 form, PDD, no entry above 1
+  FxCoef* ft = reinterpret_cast<FxCoef*>(st + ntab * ncls);
+  const int nf = x_fixed_count(M, P);
+  if constexpr (sizeof(T) == 8) {
+    if (fixed) {
+      bool ok = true;
+      for (int q = threadIdx.x; q < nf * ncls; q += blockDim.x) {
+        const int f = q < nf ? q : q - nf;
+        const double c = (q < nf ? a.tab[0] : a.tab[1])[f];
+        ft[q] = x_coef(f >= XT_NF * M * P ? 0.5 * c : f >= M * P ? -c : c, &ok);
+      }
+      fixed = __syncthreads_and(ok) != 0;
+    }
+  }
   __syncthreads();
 
   const int lane = threadIdx.x & 31;
@@ -159,6 +245,21 @@ struct AdiXK {
     } else {
 #pragma unroll
       for (int e = 0; e < M; ++e) d[e] = (T)0;
+    }
+    if constexpr (sizeof(T) == 8) {
+      if (fixed && x_fixed_group(l0 / teams)) {  // uniform over the warp
+        unsigned m = 0;
+#pragma unroll
+        for (int e = 0; e < M; ++e) m = max(m, fx_mag(d[e]));
+        for (int o = P >> 1; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(NS_FULL_MASK, m, o));
+        const int e = fx_exponent(m);
+        if (__all_sync(NS_FULL_MASK, fx_exponent_ok(e))) {
+          const int cls = a.bl && comp != 0 ? 1 : 0;
+          x_solve_fixed<M>(d, ft + cls * nf, e, r, P, a.sk->xhalf[cls] != 0);
+          if (valid) store_part<T, M>(row + r * M, d);
+          continue;
+        }
+      }
     }
     // A~ x~ = d on this partition (forward elimination, back substitution)
     d[0] = d[0] * INV[r];
@@ -227,6 +328,23 @@ struct AdiXLongK {
   const long warp = ((long)bid_.x * blockDim.x + threadIdx.x) >> 5;
   const long nwarps = ((long)gdim_.x * blockDim.x) >> 5;
   T* my = line_buf + r * (M + 1);
+  // FP64: rows at the ends of a partition whose spike is above the truncation tolerance (x_half_tol),
+  // by table: the first kv take v^(r), the last kw take w^(r) (a few of 32 rows; every row took both,
+  // two of its five FP64 instructions)
+  int kv[2] = {M, M}, kw[2] = {M, M};
+  if constexpr (sizeof(T) == 8) {
+    for (int c = 0; c < (a.bl ? 2 : 1); ++c) {
+      const T* V = a.tab[c] + XT_V * M * P + r;
+      const T* W = a.tab[c] + XT_W * M * P + r;
+      int v = 0, w = 0;
+      for (int e = 0; e < M; ++e) {
+        if (fabs(__ldg(V + e * P)) > 1e-17) v = e + 1;
+        if (fabs(__ldg(W + (M - 1 - e) * P)) > 1e-17) w = e + 1;
+      }
+      kv[c] = __reduce_max_sync(NS_FULL_MASK, v);
+      kw[c] = __reduce_max_sync(NS_FULL_MASK, w);
+    }
+  }
   for (long line = warp; line < a.nlines; line += nwarps) {
     int comp;
     long plane;
@@ -278,7 +396,14 @@ struct AdiXLongK {
     const T y0 = __ldg(DINV + r) * g0 + __ldg(DINV + P + r) * g1;
     const T y1 = __ldg(DINV + 2 * P + r) * g0 + __ldg(DINV + 3 * P + r) * g1;
     const T left = __shfl_sync(NS_FULL_MASK, y0, r - 1 + P, P);
-    for (int e = 0; e < M; ++e) my[e] = my[e] - __ldg(SV + e * P + r) * left - __ldg(SW + e * P + r) * y1;
+    if constexpr (sizeof(T) == 8) {
+      const int cls = a.bl && comp != 0 ? 1 : 0;
+      const int nv = cls ? kv[1] : kv[0], nw = cls ? kw[1] : kw[0];
+      for (int e = 0; e < nv; ++e) my[e] = my[e] - __ldg(SV + e * P + r) * left;
+      for (int e = M - nw; e < M; ++e) my[e] = my[e] - __ldg(SW + e * P + r) * y1;
+    } else {
+      for (int e = 0; e < M; ++e) my[e] = my[e] - __ldg(SV + e * P + r) * left - __ldg(SW + e * P + r) * y1;
+    }
     __syncwarp();
 #pragma unroll 4
     for (int q = 0; q < M; ++q) {
@@ -775,10 +900,14 @@ cudaError_t launch_x_t(LaunchSink& s, int k) {
   // room for the PPT tables: the levels are read from device memory and follow the mode in use
   int lmax = 0;
   while ((1 << lmax) < a.P) ++lmax;
-  const size_t smem = xtab_count(M, a.P, lmax) * sizeof(T) * (a.bl ? 2 : 1);
+  const size_t smem = (xtab_count(M, a.P, lmax) * sizeof(T) +
+                       (sizeof(T) == 8 ? x_fixed_count(M, a.P) * sizeof(FxCoef) : 0)) * (a.bl ? 2 : 1);
   const long teams_per_block = 8L * (32 / a.P);
   long blocks = (a.nlines + teams_per_block - 1) / teams_per_block;
-  if (blocks > 152L * 16) blocks = 152L * 16;
+  // FP64: the blocks two of which an SM holds (the tables and their coefficients are loaded once a
+  // block: 256 x 192 x 256 195 us at 2 blocks an SM, 211 at 4, 227 at 16)
+  const long most = 152L * (sizeof(T) == 8 ? 2 : 16);
+  if (blocks > most) blocks = most;
   return emit<AdiXK<T, M>>(s, AdiXK<T, M>::make(a), dim3((unsigned)blocks), dim3(256), smem);
 }
 
@@ -797,7 +926,8 @@ cudaError_t launch_x_long_t(LaunchSink& s, int k) {
   a.nlines = (long)a.nz * a.ny * 2 + (long)a.nz * (a.ny - 1);
   const size_t smem = (size_t)4 * 32 * (M + 1) * sizeof(T);
   long blocks = (a.nlines + 3) / 4;
-  if (blocks > 152L * 16) blocks = 152L * 16;
+  const long most = 152L * (sizeof(T) == 8 ? 6 : 16);  // FP64: the blocks an SM holds at 1024 rows
+  if (blocks > most) blocks = most;
   return emit<AdiXLongK<T, M>>(s, AdiXLongK<T, M>::make(a), dim3((unsigned)blocks), dim3(128), smem);
 }
 
@@ -930,7 +1060,7 @@ cudaError_t launch_adi_z(ns_ctx* c, int k) {
 
 template <typename T, int M>
 cudaError_t short_attr() {
-  return set_smem_limit<AdiXK<T, M>>(2 * 48 * 1024);
+  return set_smem_limit<AdiXK<T, M>>(2 * 64 * 1024);
 }
 
 template <typename T>

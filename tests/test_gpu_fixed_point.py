@@ -6,6 +6,8 @@ the same solve at ordinary magnitudes (fixed point) to the rounding of either.""
 import numpy as np
 import pytest
 
+torch = pytest.importorskip("torch")
+
 from oracle import ns_oracle as O
 from paper_1812_01178_gb300 import binding as B
 from paper_1812_01178_gb300 import inputs as I
@@ -141,3 +143,44 @@ def test_rhs_outside_the_fixed_point_range(size, plate):
                 fin[1:4, 1:4, 2:5] = False
             scale = max(np.abs(b[fin]).max(), 1e-300)
             assert np.abs(a[fin] - b[fin]).max() <= 1e-12 * scale, q
+
+
+@pytest.mark.parametrize("nx", [8, 24, 48, 64, 96, 144, 192, 256, 384, 512, 1024])
+@pytest.mark.parametrize("plate", [False, True])
+def test_x_lines_of_any_size(nx, plate):
+    """Lines solved in fixed point and in FP64 side by side, each scaled on its own: lines scaled by
+    powers of two (also out of the fixed-point range) give the scaled solution to the rounding of the
+    sweep, a line of zeros stays zero, and a NaN stays in its line."""
+    case, f, bl = _rhs_case((nx, 5, 16), plate)
+    rng = np.random.default_rng(nx)
+    s = B.Solver(case, *f, bl=bl)
+    bufs = [s.buffer(b) for b in (B.NS_BUF_RU, B.NS_BUF_RV, B.NS_BUF_RW)]
+    rows = [b.shape[0] * b.shape[1] for b in bufs]
+    base = [rng.standard_normal((n, nx)) for n in rows]
+    for b, a in zip(bufs, base):
+        b.copy_(torch.as_tensor(a.reshape(b.shape)).to(b.device))
+    s.adi(0, 0)
+    s.sync()
+    ref = [b.cpu().numpy().reshape(-1, nx).copy() for b in bufs]
+    e = [rng.choice([-940, -300, -7, 0, 11, 300, 920], n) for n in rows]
+    zero = [rng.random(n) < 0.1 for n in rows]
+    bad = [rng.random(n) < 0.1 for n in rows]
+    for b, a, ex, z, x in zip(bufs, base, e, zero, bad):
+        t = np.ldexp(a, ex[:, None]) * ~z[:, None]
+        t[x, nx // 2] = np.nan
+        b.copy_(torch.as_tensor(t.reshape(b.shape)).to(b.device))
+    s.adi(0, 0)
+    s.sync()
+    for q, (b, r, ex, z, x) in enumerate(zip(bufs, ref, e, zero, bad)):
+        got = b.cpu().numpy().reshape(-1, nx)
+        walls = np.zeros(b.shape[:2], bool)
+        if q == 1:  # v lines on the walls are not solved
+            walls[:, 0] = walls[:, -1] = True
+        live = ~walls.reshape(-1)
+        assert np.isnan(got[live & x]).any(axis=1).all()
+        ok = live & ~x
+        want = np.where(z[ok, None], 0.0, r[ok])
+        have = np.ldexp(got[ok], -ex[ok, None])
+        # a dozen roundings of the line's largest value either way
+        assert (np.abs(have - want).max(axis=1) <= 1e-14 * np.maximum(np.abs(want).max(axis=1), 0.0)).all(), q
+    s.close()
