@@ -542,24 +542,26 @@ struct RhsTiledK {
 // In FP64 arithmetic the tile was bound by the FP64 pipe: 64.8 instructions a cell of 16 cycles a
 // warp, 1.547 ms on 256 x 192 x 256 cells with the pipe 88 % busy.  Here the products and the viscous
 // sums run on the integer pipes; the FP64 pipe keeps 12 instructions a cell (pressure gradient, the
-// stored N, closing the sum): 0.737 ms, about 1000 instructions a cell and warp at 1.77 a cycle, bound
-// by the latency of their chains at 18 warps an SM (one cell a thread and twice the warps spilled at
-// 56 registers: 0.849 ms).  r is 3 to 10 times nearer to the exact sums than FP64 arithmetic was.
+// stored N, closing the sum): 0.677 ms, about a thousand instructions a cell and warp, bound by the
+// latency of their chains.  Tile and block from timings: 32 x 16 cells, two a thread, two blocks an SM
+// 0.705; 32 x 16, one a thread (56 registers, 200 bytes spilled) 0.849; 32 x 12 0.773; this one, 27
+// warps an SM, 0.677; with the viscous sum converted by the FP64 pipe (18 instructions) 0.704.  r is 3
+// to 10 times nearer to the exact sums than FP64 arithmetic was (against extended precision).
 //
-// A block marches a 32 x 16 (x, z) column along y.  The planes of u, v, w around the row stand in
+// A block marches a 32 x 8 (x, z) column along y.  The planes of u, v, w around the row stand in
 // shared memory as integers, each plane of each field scaled by its own largest magnitude in the
 // tile, so that 60 bits lie below the largest value near a cell (an FP64 result keeps 53 below its
 // own terms); p stands there in FP64.  Sums whose terms have different scales are sums of products
 // with coefficients into which the scales are folded (fx_wcoef).  One warp of the nine does nothing
 // else: it forms the coefficients of row j + 1, a term per lane and the scale of each sum from the
-// bounds of its terms, while the others (two cells in z a thread) work on row j.
+// bounds of its terms, while the others work on row j.
 //
 // A row next to a plane of u, v or w that holds an infinity, a NaN or values near the ends of the
 // binary64 range is formed in FP64 arithmetic (rhs_cell).
 // ---------------------------------------------------------------------------------------------
-constexpr int FXR_X = 32, FXR_Z = 16;
+constexpr int FXR_X = 32, FXR_Z = 8;
 constexpr int FXR_PX = FXR_X + 2, FXR_PZ = FXR_Z + 2, FXR_PLANE = FXR_PX * FXR_PZ;
-constexpr int FXR_WARPS = FXR_Z / 2;  // worker warps, two z rows each; one more forms coefficients
+constexpr int FXR_WARPS = FXR_Z;  // worker warps, a z row each; one more forms coefficients
 constexpr int FXR_THREADS = 32 * (FXR_WARPS + 1);
 
 struct RhsFxTile {
@@ -576,7 +578,7 @@ struct RhsFxTile {
   fx_t cb[2];                      // body force, at the scale of u's viscous sum
   double cgy[2];                   // pressure weight of v (zero on the wall)
   int en[2][4];                    // scales of n
-  double sr[2][4];                 // units of the viscous sums
+  int er[2][4];                    // scales of the viscous sums
   int bad[2];                      // the row takes FP64 arithmetic
   unsigned mag[4][4];              // largest high words of the planes (j mod 4) of u, v, w
 };
@@ -591,7 +593,7 @@ struct RhsFxK {
     int jchunk;
   };
   static constexpr int kThreads = FXR_THREADS;
-  static constexpr int kMinBlocks = 2;  // shared memory holds two
+  static constexpr int kMinBlocks = 3;  // shared memory holds three; 72 registers
 
   // exponent of a plane (bit 62 of its integers); zero planes take the lowest, to raise no bound
   static __device__ __forceinline__ int plane_e(unsigned m) { return (m == 0 ? 128 : (int)(m >> 20)) + 2; }
@@ -714,7 +716,7 @@ struct RhsFxK {
       }
       if (gr < 3) {
         if (qr < 5) S.cr[par][lane] = eer == FX_NONE ? FxCoef{0, 0} : fx_wcoef(cr, etr, er);
-        if (qr == 0) S.sr[par][gr] = fx_unit(er);
+        if (qr == 0) S.er[par][gr] = er;
         if (lane == 13) S.cb[par] = eer == FX_NONE ? 0 : fx_from(cr, er);
       }
       const bool good = __all_sync(NS_FULL_MASK, ok);
@@ -764,17 +766,17 @@ struct RhsFxK {
       coef_warp(a, S, jb, je);
       return;
     }
-    const int i = i0 + lane, kt = 2 * wz, k = k0 + kt;
-    const bool active0 = i < nx && k < nz, active1 = i < nx && k + 1 < nz;  // the last tiles may reach past the grid
+    const int i = i0 + lane, k = k0 + wz;
+    const bool active = i < nx && k < nz;  // the last tiles may reach past the grid
 
-    // Plane positions of this thread: rows wz and wz + 8 of the 18, and a third: rows 16, 17 (warps
-    // 0, 1) or the halo columns (warps 2, 3).  gi = -2: nothing there.
-    int gk[3], gi[3], pos[3];
+    // Plane positions of this thread: row wz of the 18, and a second: rows 16, 17 (warps 0, 1) or the
+    // halo columns (warps 2, 3).  gi = -2: nothing there.
+    int gk[2], gi[2], pos[2];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      int row = wz + 8 * r, ii = lane;
+    for (int r = 0; r < 2; ++r) {
+      int row = wz + FXR_Z * r, ii = lane;
       bool any = true;
-      if (r == 2 && wz >= 2) {
+      if (r == 1 && wz >= 2) {
         any = wz < 4 && lane < FXR_PZ;
         row = any ? lane : 0;
         ii = wz == 2 ? -1 : FXR_X;
@@ -790,8 +792,8 @@ struct RhsFxK {
     auto fetch_p = [&](int j, int sp) {
       const bool jc = j >= 0 && j < ny;
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        if (r == 2 && gi[r] == -2) continue;
+      for (int r = 0; r < 2; ++r) {
+        if (r == 1 && gi[r] == -2) continue;
         const bool in = jc && gi[r] >= 0 && gi[r] < nx;
         cp_async8(S.pp[sp] + pos[r], a.p + (in ? (long)(gk[r] * ny + j) * nx + gi[r] : 0), in);
       }
@@ -800,8 +802,8 @@ struct RhsFxK {
     auto fetch = [&](int j, int sl) {
       const bool jc = j >= 0 && j < ny, jv = j >= 0 && j <= ny;
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        if (r == 2 && gi[r] == -2) continue;
+      for (int r = 0; r < 2; ++r) {
+        if (r == 1 && gi[r] == -2) continue;
         double* d[3] = {(double*)S.pl[0][sl] + pos[r], (double*)S.pl[1][sl] + pos[r], (double*)S.pl[2][sl] + pos[r]};
         if (gi[r] >= 0 && gi[r] < nx) {
           const long oc = (long)(gk[r] * ny + j) * nx + gi[r];
@@ -828,14 +830,14 @@ struct RhsFxK {
         }
       }
     };
-    double pv[3][3];  // this thread's values of the plane that has arrived
+    double pv[2][3];  // this thread's values of the plane that has arrived
     auto gather = [&](int j, int sl) {  // ... join the maxima of plane j
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
         unsigned m = 0;
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          pv[r][f] = r < 2 || gi[r] != -2 ? ((const double*)S.pl[f][sl])[pos[r]] : 0.0;
+        for (int r = 0; r < 2; ++r) {
+          pv[r][f] = r == 0 || gi[r] != -2 ? ((const double*)S.pl[f][sl])[pos[r]] : 0.0;
           m = max(m, fx_mag(pv[r][f]));
         }
         m = __reduce_max_sync(NS_FULL_MASK, m);
@@ -847,12 +849,12 @@ struct RhsFxK {
       for (int f = 0; f < 3; ++f) {
         const int s = plane_e(S.mag[j & 3][f]);
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
-          if (r < 2 || gi[r] != -2) S.pl[f][sl][pos[r]] = fx_cut(pv[r][f], s);
+        for (int r = 0; r < 2; ++r)
+          if (r == 0 || gi[r] != -2) S.pl[f][sl][pos[r]] = fx_cut(pv[r][f], s);
       }
     };
     // plane element (z row kk, column ii) of this thread's warp: kk relative to its first cell
-    const int e0 = (kt + 1) * FXR_PX + lane + 1;
+    const int e0 = (wz + 1) * FXR_PX + lane + 1;
 
     // y-face fluxes of face jf, its planes jf - 1 and jf in slots sa and sb
     auto face_fluxes = [&](int jf, int sa, int sb) {
@@ -867,13 +869,10 @@ struct RhsFxK {
         const int e = (z + 1) * FXR_PX + x + 1;
         S.fvw[jf & 1][z][x] = fx_mulhi(fx_interpolate(w0[e], w1[e], cw0, cw1), v1[e - FXR_PX] + v1[e]);
       };
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        uv(kt + c, lane);
-        vw(kt + c, lane);
-      }
-      if (wz == 4) vw(FXR_Z, lane);  // the extra row and column (warps 0 to 3 convert the halo)
-      if (wz == 5 && lane < FXR_Z) uv(lane, FXR_X);
+      uv(wz, lane);
+      vw(wz, lane);
+      if (wz == FXR_WARPS - 4) vw(FXR_Z, lane);  // the extra row and column (warps 0 to 3 convert the halo)
+      if (wz == FXR_WARPS - 3 && lane < FXR_Z) uv(lane, FXR_X);
     };
     // Fuw of the plane in slot sl
     auto centre_products = [&](int sl) {
@@ -882,18 +881,15 @@ struct RhsFxK {
         const int e = (z + 1) * FXR_PX + x + 1;
         S.fuw[z][x] = fx_mulhi(u[e - FXR_PX] + u[e], w[e - 1] + w[e]);
       };
-#pragma unroll
-      for (int c = 0; c < 2; ++c) uw(kt + c, lane);
-      if (wz == 6) uw(FXR_Z, lane);
-      if (wz == 7 && lane <= FXR_Z) uw(lane, FXR_X);
+      uw(wz, lane);
+      if (wz == FXR_WARPS - 2) uw(FXR_Z, lane);
+      if (wz == FXR_WARPS - 1 && lane <= FXR_Z) uw(lane, FXR_X);
     };
-    // (v_j + v_{j+1})^2 of the two cells' centres j, at the larger of the planes' scales
-    auto square_v = [&](int j, int sa, int sb, fx_t* q) {
+    // (v_j + v_{j+1})^2 of the centre j, at the larger of the planes' scales
+    auto square_v = [&](int j, int sa, int sb) {
       const int ea = plane_e(S.mag[j & 3][1]), eb = plane_e(S.mag[(j + 1) & 3][1]), em = max(ea, eb);
       const int da = min(em - ea, 63), db = min(em - eb, 63);
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-        q[c] = fx_sqrhi((S.pl[1][sa][e0 + c * FXR_PX] >> da) + (S.pl[1][sb][e0 + c * FXR_PX] >> db));
+      return fx_sqrhi((S.pl[1][sa][e0] >> da) + (S.pl[1][sb][e0] >> db));
     };
 
     // ---- prologue: planes jb - 1 .. jb + 1, then (coefficients) the fluxes of face jb.  Slots of planes
@@ -912,8 +908,7 @@ struct RhsFxK {
     if (jb + 1 < je) fetch(jb + 2, s2);
     __syncthreads();
     face_fluxes(jb, sm, s0);
-    fx_t q2prev[2] = {0, 0};
-    if (jb >= 1) square_v(jb - 1, sm, s0, q2prev);
+    fx_t q2prev = jb >= 1 ? square_v(jb - 1, sm, s0) : 0;
 
     const bool use_prev = a.zet != 0.0;
     const double* kd = a.sk->kd;
@@ -924,7 +919,6 @@ struct RhsFxK {
     double* nu = (double*)a.nu;
     double* nv = (double*)a.nv;
     double* nw = (double*)a.nw;
-    const long sc = (long)ny * nx, sv = (long)(ny + 1) * nx;  // z strides
     for (int j = jb; j < je; ++j) {
       const bool next = j + 1 < je;  // another row follows
       cp_async_wait_all8();
@@ -936,143 +930,87 @@ struct RhsFxK {
         if (j + 2 < je) fetch(j + 3, s3);
         fetch_p(j + 1, pn);
       }
-      double prev[3][2] = {};  // the stored N of the last sub-step (v, u, w)
-      if (use_prev) {
-        if (active0) {
-          prev[0][0] = nv[cf];
-          prev[1][0] = nu[cc];
-          prev[2][0] = nw[cc];
-        }
-        if (active1) {
-          prev[0][1] = nv[cf + sv];
-          prev[1][1] = nu[cc + sc];
-          prev[2][1] = nw[cc + sc];
-        }
+      double prev[3] = {};  // the stored N of the last sub-step (v, u, w)
+      if (use_prev && active) {
+        prev[0] = nv[cf];
+        prev[1] = nu[cc];
+        prev[2] = nw[cc];
       }
       face_fluxes(j + 1, s0, s1);
       centre_products(s0);
-      fx_t q2[2];
-      square_v(j, s0, s1, q2);
+      const fx_t q2 = square_v(j, s0, s1);
       __syncthreads();
       const int par = j & 1, f0 = j & 1, f1 = f0 ^ 1;
       if (S.bad[par]) {
-        if (active0) rhs_cell_fp64(a, i, j, k);
-        if (active1) rhs_cell_fp64(a, i, j, k + 1);
+        if (active) rhs_cell_fp64(a, i, j, k);
       } else {
         const FxCoef* cn = S.cn[par];
         const FxCoef* cr = S.cr[par];
-        // The viscous sums of field f at the two cells; o: the plane's values (0, 1 the cells, 2, 3 the
-        // z neighbours below and above, 4, 5 and 6, 7 the x neighbours before and after)
-        auto viscous = [&](FxAcc* s, int f, const FxCoef* c, fx_t* o) {
+        // The viscous sum of field f; o: the plane's values at the cell, the z neighbours below and
+        // above, the x neighbours before and after
+        auto viscous = [&](FxAcc& s, int f, const FxCoef* c, fx_t* o) {
           const fx_t* p = S.pl[f][s0] + e0;
-          const fx_t *lo = S.pl[f][sm] + e0, *up = S.pl[f][s1] + e0;
           o[0] = p[0];
-          o[1] = p[FXR_PX];
-          o[2] = p[-FXR_PX];
-          o[3] = p[2 * FXR_PX];
-          o[4] = p[-1];
-          o[5] = p[FXR_PX - 1];
-          o[6] = p[1];
-          o[7] = p[FXR_PX + 1];
-          const FxCoef wx = c[0], wz_ = c[1], wc = c[2], wl = c[3], wu = c[4];
-          fx_wmac(s[0], o[4] + o[6], wx);
-          fx_wmac(s[1], o[5] + o[7], wx);
-          fx_wmac(s[0], o[1] + o[2], wz_);
-          fx_wmac(s[1], o[3] + o[0], wz_);
-          fx_wmac(s[0], o[0], wc);
-          fx_wmac(s[1], o[1], wc);
-          fx_wfold(s[0]);
-          fx_wfold(s[1]);
-          fx_wmac(s[0], lo[0], wl);
-          fx_wmac(s[1], lo[FXR_PX], wl);
-          fx_wmac(s[0], up[0], wu);
-          fx_wmac(s[1], up[FXR_PX], wu);
+          o[1] = p[-FXR_PX];
+          o[2] = p[FXR_PX];
+          o[3] = p[-1];
+          o[4] = p[1];
+          fx_wmac(s, o[3] + o[4], c[0]);
+          fx_wmac(s, o[1] + o[2], c[1]);
+          fx_wmac(s, o[0], c[2]);
+          fx_wfold(s);
+          fx_wmac(s, S.pl[f][sm][e0], c[3]);
+          fx_wmac(s, S.pl[f][s1][e0], c[4]);
         };
         const double* pj = S.pp[pc] + e0;
-        const double p0 = pj[0], p1 = pj[FXR_PX];
-        fx_t o[8];
-        double nd[3][2], rd[3][2];  // stored together at the end: the FP64 sums finish meanwhile
+        const double p0 = pj[0];
+        fx_t o[5];
+        double nd[3], rd[3];  // stored together at the end: the FP64 sums finish meanwhile
         // ---------------- v at face j
         {
-          FxAcc n[2] = {fx_wacc(0), fx_wacc(0)}, s[2] = {fx_wacc(0), fx_wacc(0)};
-          const fx_t wm = S.fvw[f0][kt][lane], w0 = S.fvw[f0][kt + 1][lane], wp = S.fvw[f0][kt + 2][lane];
-          fx_wmac(n[0], S.fuv[f0][kt][lane + 1] - S.fuv[f0][kt][lane], cn[0]);
-          fx_wmac(n[1], S.fuv[f0][kt + 1][lane + 1] - S.fuv[f0][kt + 1][lane], cn[0]);
-          fx_wmac(n[0], w0 - wm, cn[3]);
-          fx_wmac(n[1], wp - w0, cn[3]);
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            fx_wmac(n[c], q2[c], cn[1]);
-            fx_wmac(n[c], q2prev[c], cn[2]);
-          }
+          FxAcc n = fx_wacc(0), s = fx_wacc(0);
+          fx_wmac(n, S.fuv[f0][wz][lane + 1] - S.fuv[f0][wz][lane], cn[0]);
+          fx_wmac(n, S.fvw[f0][wz + 1][lane] - S.fvw[f0][wz][lane], cn[3]);
+          fx_wmac(n, q2, cn[1]);
+          fx_wmac(n, q2prev, cn[2]);
           viscous(s, 1, cr, o);
-          const double* pb = S.pp[pm] + e0;
-          const double cgy = S.cgy[par], sr = S.sr[par][0];
-          const int en = S.en[par][0];
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            nd[0][c] = fx_to(fx_wsum(n[c]), en);
-            const double dp = (c ? p1 : p0) - pb[c * FXR_PX];
-            rd[0][c] = fma(fx_double(fx_wsum(s[c])), sr, fma(cgy, dp, fma(cp, prev[0][c], nd[0][c])));
-          }
+          nd[0] = fx_to(fx_wsum(n), S.en[par][0]);
+          const double dp = p0 - S.pp[pm][e0];
+          rd[0] = (fx_to(fx_wsum(s), S.er[par][0]) + fma(S.cgy[par], dp, fma(cp, prev[0], nd[0])));
         }
         // ---------------- u at (xf_i, yc_j, zc_k)
         {
-          const fx_t cb = S.cb[par];
-          FxAcc n[2] = {fx_wacc(0), fx_wacc(0)}, s[2] = {fx_wacc(cb), fx_wacc(cb)};
-          const fx_t um = S.fuw[kt][lane], u0 = S.fuw[kt + 1][lane], up = S.fuw[kt + 2][lane];
-          fx_wmac(n[0], u0 - um, cn[7]);
-          fx_wmac(n[1], up - u0, cn[7]);
+          FxAcc n = fx_wacc(0), s = fx_wacc(S.cb[par]);
+          fx_wmac(n, S.fuw[wz + 1][lane] - S.fuw[wz][lane], cn[7]);
+          fx_wmac(n, S.fuv[f1][wz][lane], cn[5]);
+          fx_wmac(n, S.fuv[f0][wz][lane], cn[6]);
           viscous(s, 0, cr + 8, o);
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            fx_wmac(n[c], fx_sqrhi(o[c] + o[6 + c]) - fx_sqrhi(o[4 + c] + o[c]), cn[4]);
-            fx_wmac(n[c], S.fuv[f1][kt + c][lane], cn[5]);
-            fx_wmac(n[c], S.fuv[f0][kt + c][lane], cn[6]);
-          }
-          const double sr = S.sr[par][1];
-          const int en = S.en[par][1];
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            nd[1][c] = fx_to(fx_wsum(n[c]), en);
-            const double dp = (c ? p1 : p0) - pj[c * FXR_PX - 1];
-            rd[1][c] = fma(fx_double(fx_wsum(s[c])), sr, fma(cgx, dp, fma(cp, prev[1][c], nd[1][c])));
-          }
+          fx_wmac(n, fx_sqrhi(o[0] + o[4]) - fx_sqrhi(o[3] + o[0]), cn[4]);
+          nd[1] = fx_to(fx_wsum(n), S.en[par][1]);
+          rd[1] = (fx_to(fx_wsum(s), S.er[par][1]) + fma(cgx, p0 - pj[-1], fma(cp, prev[1], nd[1])));
         }
         // ---------------- w at (xc_i, yc_j, zf_k)
         {
-          FxAcc n[2] = {fx_wacc(0), fx_wacc(0)}, s[2] = {fx_wacc(0), fx_wacc(0)};
+          FxAcc n = fx_wacc(0), s = fx_wacc(0);
+          fx_wmac(n, S.fuw[wz][lane + 1] - S.fuw[wz][lane], cn[8]);
+          fx_wmac(n, S.fvw[f1][wz][lane], cn[9]);
+          fx_wmac(n, S.fvw[f0][wz][lane], cn[10]);
           viscous(s, 2, cr + 16, o);
-          const fx_t qm = fx_sqrhi(o[2] + o[0]), q0 = fx_sqrhi(o[0] + o[1]), qp = fx_sqrhi(o[1] + o[3]);
-          fx_wmac(n[0], q0 - qm, cn[11]);
-          fx_wmac(n[1], qp - q0, cn[11]);
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            fx_wmac(n[c], S.fuw[kt + c][lane + 1] - S.fuw[kt + c][lane], cn[8]);
-            fx_wmac(n[c], S.fvw[f1][kt + c][lane], cn[9]);
-            fx_wmac(n[c], S.fvw[f0][kt + c][lane], cn[10]);
-          }
-          const double sr = S.sr[par][2];
-          const int en = S.en[par][2];
-          const double dp0 = p0 - pj[-FXR_PX], dp1 = p1 - p0;
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            nd[2][c] = fx_to(fx_wsum(n[c]), en);
-            rd[2][c] = fma(fx_double(fx_wsum(s[c])), sr, fma(cgz, c ? dp1 : dp0, fma(cp, prev[2][c], nd[2][c])));
-          }
+          fx_wmac(n, fx_sqrhi(o[0] + o[2]) - fx_sqrhi(o[1] + o[0]), cn[11]);
+          nd[2] = fx_to(fx_wsum(n), S.en[par][2]);
+          rd[2] = (fx_to(fx_wsum(s), S.er[par][2]) + fma(cgz, p0 - pj[-FXR_PX], fma(cp, prev[2], nd[2])));
         }
-        const bool wall = j == 0, fixed = a.bl && i == 0;  // the wall row of v, the inflow face of u
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-          if (c ? active1 : active0) {
-            nv[cf + c * sv] = nd[0][c];
-            rv[cf + c * sv] = wall ? 0.0 : rd[0][c];
-            nu[cc + c * sc] = fixed ? 0.0 : nd[1][c];
-            ru[cc + c * sc] = fixed ? 0.0 : rd[1][c];
-            nw[cc + c * sc] = nd[2][c];
-            rw[cc + c * sc] = rd[2][c];
-          }
+        if (active) {
+          const bool wall = j == 0, fixed = a.bl && i == 0;  // the wall row of v, the inflow face of u
+          nv[cf] = nd[0];
+          rv[cf] = wall ? 0.0 : rd[0];
+          nu[cc] = fixed ? 0.0 : nd[1];
+          ru[cc] = fixed ? 0.0 : rd[1];
+          nw[cc] = nd[2];
+          rw[cc] = rd[2];
+        }
       }
+      q2prev = q2;
       {  // the rings move on by one plane
         const int t = sm;
         sm = s0;
@@ -1084,13 +1022,10 @@ struct RhsFxK {
         pc = pn;
         pn = 3 - pm - pc;
       }
-      q2prev[0] = q2[0];
-      q2prev[1] = q2[1];
     }
     if (je == ny) {  // the top wall row of v
       const long cf = ((long)k * (ny + 1) + ny) * nx + i;
-      if (active0) nv[cf] = rv[cf] = 0.0;
-      if (active1) nv[cf + sv] = rv[cf + sv] = 0.0;
+      if (active) nv[cf] = rv[cf] = 0.0;
     }
   }
 };
