@@ -96,7 +96,7 @@ ns_layout make_layout(const ns_config* c) {
   sz[LB_LAMX] = nx * 8;
   sz[LB_LAMZ] = nzh * 8;
   sz[LB_RTAB] = 3 * al256((size_t)RT_COUNT * (ny + 1) * 8) + 3 * al256((size_t)RT_COUNT * (ny + 1) * 4);
-  sz[LB_DOUT] = 3 * al256((ny + 1) * nz * 8) + 256;
+  sz[LB_DOUT] = 3 * al256((ny + 1) * nz * 8) + 256 + FLUX_BLOCKS * 8;
   sz[LB_TWD] = nx * sizeof(FxTw);
   sz[LB_RCY] = recycle_block_doubles((int)ny) * 8;
   sz[LB_STEPK] = NS_STEPK * sizeof(StepK);
@@ -410,6 +410,7 @@ ns_status ns_init(ns_ctx** out, const ns_config* cfg, const ns_fields* fields, v
   for (int q = 0; q < 3; ++q) c->dout[q] = (double*)(base + c->lay.off[LB_DOUT] + q * al256((size_t)(ny + 1) * nz * 8));
   c->flux = (double*)(base + c->lay.off[LB_DOUT] + 3 * al256((size_t)(ny + 1) * nz * 8));
   c->rate = (unsigned long long*)(c->flux + 4);
+  c->flux_part = c->flux + 32;
   c->rcy = (double*)(base + c->lay.off[LB_RCY]);
   c->stepk = (StepK*)(base + c->lay.off[LB_STEPK]);
   c->dtctl = (DtCtl*)(base + c->lay.off[LB_DT]);
