@@ -1865,36 +1865,53 @@ __global__ void outflow_kernel(const double* __restrict__ u, const double* __res
 
 // ------------------------------------------------------------------------------------------
 // outflow mass-flux correction: u_out += (Q_in - Q_out) / (Ly Lz) with Q = sum u dy_j dz over the
-// inflow face (face 0 of u) and the outflow plane.  FLUX_BLOCKS blocks sum a fixed share each, then
-// every block of a second launch adds those sums in one order and shifts its share of the plane: the
-// result does not depend on the schedule.  (One block for all of it took 158 us on 512 x 256 planes:
-// a single SM fetches a row of its own for every face of the inflow.)
+// inflow face (face 0 of u) and the outflow plane.  FLUX_PARTS partial sums, sum t over the faces
+// t, t + FLUX_PARTS, ... in turn, then a binary tree: the result does not depend on the schedule.  A
+// mixed-form step rounds to FP32 what this shift changes in the last place, so the order is part of
+// the result.  One block for all of it took 158 us on 512 x 256 planes (a single SM fetches a row of
+// its own for every face of the inflow).  Here FLUX_PARTS / 16 blocks fetch the differences of 16 x 16
+// faces at a time, the next ones while 16 threads add the last ones, and every block of a second launch
+// forms the tree for itself and shifts its share of the plane: 25 us there, 12 on 128 x 96 (was 24).
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) flux_sum_kernel(const double* __restrict__ u, const double* __restrict__ u_out,
                                                        const double* __restrict__ gc, int nx, int ny, int nz,
                                                        double* __restrict__ part) {
-  __shared__ double red[256];
+  __shared__ double sd[256], sw[256];
   const double* dy = gc + GC_DY * (ny + 1);
   const long n = (long)nz * ny;
-  double acc = 0.0;
-  for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long)FLUX_BLOCKS * blockDim.x)
-    acc += (__ldg(u + q * nx) - __ldg(u_out + q)) * __ldg(dy + (int)(q % ny));
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s2 = blockDim.x / 2; s2 > 0; s2 >>= 1) {
-    if (threadIdx.x < s2) red[threadIdx.x] += red[threadIdx.x + s2];
+  const int tid = threadIdx.x, t = blockIdx.x * 16 + (tid & 15);
+  double acc = 0.0, d = 0.0, w = 0.0;
+  long q = (long)(tid >> 4) * FLUX_PARTS + t;  // this thread's face of the next 16 x 16
+  auto fetch = [&]() {
+    if (q < n) {
+      d = __ldg(u + q * nx) - __ldg(u_out + q);
+      w = __ldg(dy + (int)(q % ny));
+    }
+    q += 16 * FLUX_PARTS;
+  };
+  fetch();
+  for (long q0 = 0; q0 < n; q0 += 16 * FLUX_PARTS) {
+    sd[tid] = d;
+    sw[tid] = w;
+    __syncthreads();
+    if (q0 + 16 * FLUX_PARTS < n) fetch();
+    if (tid < 16) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m)
+        if (q0 + (long)m * FLUX_PARTS + t < n) acc = fma(sd[m * 16 + tid], sw[m * 16 + tid], acc);
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (tid < 16) part[t] = acc;
 }
 
 __global__ void __launch_bounds__(256) flux_shift_kernel(double* __restrict__ u_out, long n, double dz_over_area,
                                                          const double* __restrict__ part, double* __restrict__ flux) {
-  __shared__ double red[FLUX_BLOCKS];
-  if (threadIdx.x < FLUX_BLOCKS) red[threadIdx.x] = part[threadIdx.x];
+  __shared__ double red[FLUX_PARTS];
+  for (int t = threadIdx.x; t < FLUX_PARTS; t += 256) red[t] = __ldg(part + t);
   __syncthreads();
-  for (int s2 = FLUX_BLOCKS / 2; s2 > 0; s2 >>= 1) {
-    if (threadIdx.x < s2) red[threadIdx.x] += red[threadIdx.x + s2];
+  for (int s2 = FLUX_PARTS / 2; s2 > 0; s2 >>= 1) {
+    for (int t = threadIdx.x; t < s2; t += 256) red[t] += red[t + s2];
     __syncthreads();
   }
   const double corr = red[0] * dz_over_area;
@@ -2383,7 +2400,7 @@ cudaError_t launch_flux_correct(ns_ctx* c, int) {
   const int ny = c->cfg.ny;
   const double area = (c->yf[ny] - c->yf[0]) * c->cfg.lz;
   const long n = (long)c->cfg.nz * ny;
-  flux_sum_kernel<<<FLUX_BLOCKS, 256, 0, c->launch>>>(c->f.u, c->f.u_out, c->gc, c->cfg.nx, ny, c->cfg.nz, c->flux_part);
+  flux_sum_kernel<<<FLUX_PARTS / 16, 256, 0, c->launch>>>(c->f.u, c->f.u_out, c->gc, c->cfg.nx, ny, c->cfg.nz, c->flux_part);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   flux_shift_kernel<<<(unsigned)std::min((n + 255) / 256, 304L), 256, 0, c->launch>>>(c->f.u_out, n, c->dz / area,

@@ -96,7 +96,7 @@ ns_layout make_layout(const ns_config* c) {
   sz[LB_LAMX] = nx * 8;
   sz[LB_LAMZ] = nzh * 8;
   sz[LB_RTAB] = 3 * al256((size_t)RT_COUNT * (ny + 1) * 8) + 3 * al256((size_t)RT_COUNT * (ny + 1) * 4);
-  sz[LB_DOUT] = 3 * al256((ny + 1) * nz * 8) + 256 + FLUX_BLOCKS * 8;
+  sz[LB_DOUT] = 3 * al256((ny + 1) * nz * 8) + 256 + FLUX_PARTS * 8;
   sz[LB_TWD] = nx * sizeof(FxTw);
   sz[LB_RCY] = recycle_block_doubles((int)ny) * 8;
   sz[LB_STEPK] = NS_STEPK * sizeof(StepK);

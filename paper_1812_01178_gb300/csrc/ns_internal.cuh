@@ -239,7 +239,7 @@ struct StepK {
                       // tolerance (x_half_tol), so each row takes one correction only
 };
 constexpr int NS_STEPK = 4;
-constexpr int FLUX_BLOCKS = 64;  // blocks that sum the outflow correction
+constexpr int FLUX_PARTS = 1024;  // partial sums of the outflow correction
 
 inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -311,7 +311,7 @@ struct ns_ctx {
   // sweeps form c/pivot from them, the FP64 tiles take a_j as a float-float pair
   float4* pois_rows32 = nullptr;
   double* flux;             // [0]: inflow flux, [1]: last outflow correction (diagnostics)
-  double* flux_part;        // FLUX_BLOCKS partial sums of the outflow correction
+  double* flux_part;        // FLUX_PARTS partial sums of the outflow correction
   unsigned long long* rate; // bits of the convective rate of ns_convective_rate (in the flux block)
   std::vector<double> gc_h; // host copy of the grid coefficients (tables are rebuilt when dt changes)
   double* rcy;              // recycling inflow: sample heights, plane means, gamma (k_recycle.cu)
