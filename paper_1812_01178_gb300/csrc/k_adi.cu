@@ -8,7 +8,8 @@
 //      Z y   = E^T x~            (Eq. Zpdd)     interface unknowns y = (x^{(r)}_m, x^{(r+1)}_1)
 //      x     = x~ - Y y          (Eq. xpdd)
 //    PDD keeps only the 2x2 diagonal blocks of Z; PPT solves all of Z exactly by block parallel
-//    cyclic reduction over the team with warp shuffles (line-independent eliminators).
+//    cyclic reduction over the team with warp shuffles (line-independent eliminators).  FP64: of each
+//    eight groups of lines four are solved in 64-bit fixed point, beside the FP64 ones.
 // y: lines have stride nx; one thread per line, Thomas with precomputed factors.
 // z: lines have stride nx*ny and are periodic; one thread per line, Thomas on the Sherman-
 //    Morrison-modified matrix plus the rank-one correction; then u* = u + delta (FP64).

@@ -1,4 +1,4 @@
-// Pressure Poisson solve and projection (Sec. 2.2), FP64 throughout.
+// Pressure Poisson solve and projection (Sec. 2.2).
 //
 //   b = D u* / (alpha_k dt)                      divergence at cell centres
 //   b^(kx, j, kz) = FFT_x FFT_z b                 real FFT along z (two real columns packed into
@@ -10,26 +10,17 @@
 //   u = u* - alpha_k dt G phi,  p = p + phi
 //
 // FFTs are mixed radix-2/4/3 Stockham autosort transforms (decimation in time) in shared memory
-// with a precomputed table of FMA-form twiddles (fft_twiddles); nx and nz are 2^a 3^b.  The y factors (1/pivot, c/pivot) of every (kx, kz)
-// system are precomputed once by pois_factor_kernel (the operator does not change).
+// with a precomputed table of twiddles; nx and nz are 2^a 3^b.  The FP64 form's butterflies run in 64-bit
+// fixed point (fx_stockham, twiddles from fx_twiddles), its divergence, y solve and projection in FP64;
+// the mixed form's transforms in FP32 (stockham, FMA-form twiddles from fft_twiddles).  The y factors
+// (1/pivot, c/pivot) of every (kx, kz) system are precomputed once by pois_factor_kernel (the operator
+// does not change).
 #include <algorithm>
 
 #include "ns_internal.cuh"
 
 namespace {
 
-// complex arithmetic on double2 (FP64 path) and float2 (the transforms of the mixed form)
-template <typename C> struct Cplx;
-template <> struct Cplx<double2> {
-  using R = double;
-  static __device__ __forceinline__ double2 mk(double x, double y) { return make_double2(x, y); }
-};
-template <> struct Cplx<float2> {
-  using R = float;
-  static __device__ __forceinline__ float2 mk(float x, float y) { return make_float2(x, y); }
-};
-__device__ __forceinline__ double fmaT(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float fmaT(float a, float b, float c) { return fmaf(a, b, c); }
 // error-free transformations (Knuth's TwoSum; TwoProd by one FMA): s + e = a + b, p + e = a b
 __device__ __forceinline__ void ff_two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
@@ -40,33 +31,30 @@ __device__ __forceinline__ void ff_two_prod(float a, float b, float& p, float& e
   p = __fmul_rn(a, b);
   e = __fmaf_rn(a, b, -p);
 }
-template <typename C>
-__device__ __forceinline__ C cadd(C a, C b) { return Cplx<C>::mk(a.x + b.x, a.y + b.y); }
-template <typename C>
-__device__ __forceinline__ C csub(C a, C b) { return Cplx<C>::mk(a.x - b.x, a.y - b.y); }
+// complex arithmetic of the mixed form's transforms
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
-// Stockham autosort FFT on nseq sequences of length N = 2^a 3^b stored contiguously in A
-// ([seq][N]); plan = a | (b << 8) (fft_plan).  B is scratch of the same size.  SIGN = -1 forward,
+// Stockham autosort FFT in FP32 (the mixed form) on nseq sequences of length N = 2^a 3^b stored
+// contiguously in A ([seq][N]); plan = a | (b << 8) (fft_plan).  B is scratch of the same size.  SIGN = -1 forward,
 // +1 inverse (unscaled).  Decimation in time: one twiddle-free radix-2 stage first when a is odd,
 // then a/2 radix-4 stages, then b radix-3 stages.  A radix-R stage that follows stages combining
 // sub-transforms of length Ns reads, for j < N/R and k = j mod Ns, the R inputs at j + r N/R,
 // multiplies input r by w^(r k) (w = exp(-2 pi i / (R Ns)), conjugated for the inverse), takes the
 // R-point DFT and writes output r to (j / Ns) R Ns + k + r Ns.
 //
-// The FP64 pipe is the bound here, so the twiddled butterflies use the tangent factorisation of
+// The twiddled butterflies use the tangent factorisation of
 // Goedecker (SIAM J. Sci. Comput. 18, 1997): b w = cos(th) (b.x + tan(th) b.y, b.y - tan(th) b.x)
 // costs two FMAs, and the cosine is folded into the following additions; inputs 1 and 3 (radix
 // 4) or 1 and 2 (radix 3) share one scale through the ratio of their cosines.  A twiddled radix-4
-// butterfly is 22 FMAs (instead of 28 instructions), a radix-3 one 16.  tw holds six doubles per
+// butterfly is 22 FMAs (instead of 28 instructions), a radix-3 one 16.  tw holds six floats per
 // entry Ns + k (fft_twiddles): radix 4, th = 2 pi k / (4 Ns): {tan th, cos th}, {tan 2th, cos 2th},
 // {tan 3th, cos 3th / cos th}; radix 3, th = 2 pi k / (3 Ns): {tan th, cos th},
 // {tan 2th, cos 2th / cos th}, {cos th / 2, (sqrt 3 / 2) cos th}.  cos th is never exactly zero in
 // floating point, so every factor is finite.  Returns the buffer that holds the result.  All
 // threads of the block take part.
-template <int SIGN, typename C = double2>
-__device__ C* stockham(C* A, C* B, int N, int plan, int nseq, const C* __restrict__ tw) {
-  using R = typename Cplx<C>::R;
-  auto mk = [](R x, R y) { return Cplx<C>::mk(x, y); };
+template <int SIGN>
+__device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, const float2* __restrict__ tw) {
   const int a2 = plan & 0xff, b3 = plan >> 8;
   const bool p2 = b3 == 0;  // N a power of two: index arithmetic by shifts
   int Ns = 1;
@@ -76,14 +64,14 @@ __device__ C* stockham(C* A, C* B, int N, int plan, int nseq, const C* __restric
     for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
       const int sq = p2 ? idx >> (a2 - 1) : idx / half;
       const int j = idx - sq * half;
-      const C* X = A + sq * N;
-      C* Y = B + sq * N;
-      const C a = X[j], b = X[j + half];
+      const float2* X = A + sq * N;
+      float2* Y = B + sq * N;
+      const float2 a = X[j], b = X[j + half];
       Y[2 * j] = cadd(a, b);
       Y[2 * j + 1] = csub(a, b);
     }
     __syncthreads();
-    C* t = A;
+    float2* t = A;
     A = B;
     B = t;
     Ns = 2;
@@ -96,36 +84,36 @@ __device__ C* stockham(C* A, C* B, int N, int plan, int nseq, const C* __restric
       const int sq = p2 ? idx >> (a2 - 2) : idx / quarter;
       const int j = idx - sq * quarter;
       const int k = j & (Ns - 1);
-      const C* X = A + sq * N + j;
-      C* Y = B + sq * N + ((j >> ls) << (ls + 2)) + k;
-      const C a = X[0], b = X[quarter], c = X[2 * quarter], d = X[3 * quarter];
-      C y0, y1, y2, y3;
+      const float2* X = A + sq * N + j;
+      float2* Y = B + sq * N + ((j >> ls) << (ls + 2)) + k;
+      const float2 a = X[0], b = X[quarter], c = X[2 * quarter], d = X[3 * quarter];
+      float2 y0, y1, y2, y3;
       if (Ns == 1) {
-        const C t0 = cadd(a, c), t1 = csub(a, c), t2 = cadd(b, d), t3 = csub(b, d);
+        const float2 t0 = cadd(a, c), t1 = csub(a, c), t2 = cadd(b, d), t3 = csub(b, d);
         // -i t3 (forward) or +i t3 (inverse)
-        const C r3 = SIGN < 0 ? mk(t3.y, -t3.x) : mk(-t3.y, t3.x);
+        const float2 r3 = SIGN < 0 ? make_float2(t3.y, -t3.x) : make_float2(-t3.y, t3.x);
         y0 = cadd(t0, t2);
         y2 = csub(t0, t2);
         y1 = cadd(t1, r3);
         y3 = csub(t1, r3);
       } else {
-        const C e1 = __ldg(tw + 3 * (Ns + k)), e2 = __ldg(tw + 3 * (Ns + k) + 1), e3 = __ldg(tw + 3 * (Ns + k) + 2);
-        const R t1 = SIGN < 0 ? e1.x : -e1.x, t2 = SIGN < 0 ? e2.x : -e2.x, t3 = SIGN < 0 ? e3.x : -e3.x;
-        const R c1 = e1.y, c2 = e2.y, r = e3.y;
+        const float2 e1 = __ldg(tw + 3 * (Ns + k)), e2 = __ldg(tw + 3 * (Ns + k) + 1), e3 = __ldg(tw + 3 * (Ns + k) + 2);
+        const float t1 = SIGN < 0 ? e1.x : -e1.x, t2 = SIGN < 0 ? e2.x : -e2.x, t3 = SIGN < 0 ? e3.x : -e3.x;
+        const float c1 = e1.y, c2 = e2.y, r = e3.y;
         // b, c, d times their twiddles, each up to its cosine
-        const C bb = mk(fmaT(t1, b.y, b.x), fmaT(-t1, b.x, b.y));
-        const C cc = mk(fmaT(t2, c.y, c.x), fmaT(-t2, c.x, c.y));
-        const C dd = mk(fmaT(t3, d.y, d.x), fmaT(-t3, d.x, d.y));
-        const C T0 = mk(fmaT(c2, cc.x, a.x), fmaT(c2, cc.y, a.y));    // a + c w^2k
-        const C T1 = mk(fmaT(-c2, cc.x, a.x), fmaT(-c2, cc.y, a.y));  // a - c w^2k
-        const C S = mk(fmaT(r, dd.x, bb.x), fmaT(r, dd.y, bb.y));    // (b w^k + d w^3k) / cos th
-        const C D = mk(fmaT(-r, dd.x, bb.x), fmaT(-r, dd.y, bb.y));  // (b w^k - d w^3k) / cos th
-        y0 = mk(fmaT(c1, S.x, T0.x), fmaT(c1, S.y, T0.y));
-        y2 = mk(fmaT(-c1, S.x, T0.x), fmaT(-c1, S.y, T0.y));
+        const float2 bb = make_float2(fmaf(t1, b.y, b.x), fmaf(-t1, b.x, b.y));
+        const float2 cc = make_float2(fmaf(t2, c.y, c.x), fmaf(-t2, c.x, c.y));
+        const float2 dd = make_float2(fmaf(t3, d.y, d.x), fmaf(-t3, d.x, d.y));
+        const float2 T0 = make_float2(fmaf(c2, cc.x, a.x), fmaf(c2, cc.y, a.y));    // a + c w^2k
+        const float2 T1 = make_float2(fmaf(-c2, cc.x, a.x), fmaf(-c2, cc.y, a.y));  // a - c w^2k
+        const float2 S = make_float2(fmaf(r, dd.x, bb.x), fmaf(r, dd.y, bb.y));    // (b w^k + d w^3k) / cos th
+        const float2 D = make_float2(fmaf(-r, dd.x, bb.x), fmaf(-r, dd.y, bb.y));  // (b w^k - d w^3k) / cos th
+        y0 = make_float2(fmaf(c1, S.x, T0.x), fmaf(c1, S.y, T0.y));
+        y2 = make_float2(fmaf(-c1, S.x, T0.x), fmaf(-c1, S.y, T0.y));
         // y1 = T1 - i (v1 - v3), y3 = T1 + i (v1 - v3) forward; signs of i swap for the inverse
-        const R s1 = SIGN < 0 ? c1 : -c1;
-        y1 = mk(fmaT(s1, D.y, T1.x), fmaT(-s1, D.x, T1.y));
-        y3 = mk(fmaT(-s1, D.y, T1.x), fmaT(s1, D.x, T1.y));
+        const float s1 = SIGN < 0 ? c1 : -c1;
+        y1 = make_float2(fmaf(s1, D.y, T1.x), fmaf(-s1, D.x, T1.y));
+        y3 = make_float2(fmaf(-s1, D.y, T1.x), fmaf(s1, D.x, T1.y));
       }
       Y[0] = y0;
       Y[Ns] = y1;
@@ -133,12 +121,12 @@ __device__ C* stockham(C* A, C* B, int N, int plan, int nseq, const C* __restric
       Y[3 * Ns] = y3;
     }
     __syncthreads();
-    C* t = A;
+    float2* t = A;
     A = B;
     B = t;
   }
   const int third = N / 3;
-  const R kS3 = (R)0.86602540378443864676;  // sqrt(3) / 2
+  const float kS3 = 0.86602540378443864676f;  // sqrt(3) / 2
   for (int st = 0; st < b3; ++st, Ns *= 3) {
     const int total = nseq * third;
     for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
@@ -146,36 +134,36 @@ __device__ C* stockham(C* A, C* B, int N, int plan, int nseq, const C* __restric
       const int j = idx - sq * third;
       const int g = j / Ns;
       const int k = j - g * Ns;
-      const C* X = A + sq * N + j;
-      C* Y = B + sq * N + g * 3 * Ns + k;
-      const C a = X[0], b = X[third], c = X[2 * third];
-      C S, D, y0, T;
-      R gs;
+      const float2* X = A + sq * N + j;
+      float2* Y = B + sq * N + g * 3 * Ns + k;
+      const float2 a = X[0], b = X[third], c = X[2 * third];
+      float2 S, D, y0, T;
+      float gs;
       if (Ns == 1) {
         S = cadd(b, c);
         D = csub(b, c);
         y0 = cadd(a, S);
-        T = mk(fmaT((R)-0.5, S.x, a.x), fmaT((R)-0.5, S.y, a.y));
+        T = make_float2(fmaf(-0.5f, S.x, a.x), fmaf(-0.5f, S.y, a.y));
         gs = SIGN < 0 ? kS3 : -kS3;
       } else {
-        const C e1 = __ldg(tw + 3 * (Ns + k)), e2 = __ldg(tw + 3 * (Ns + k) + 1), e3 = __ldg(tw + 3 * (Ns + k) + 2);
-        const R t1 = SIGN < 0 ? e1.x : -e1.x, t2 = SIGN < 0 ? e2.x : -e2.x;
-        const R c1 = e1.y, r = e2.y, h = e3.x;
-        const C bb = mk(fmaT(t1, b.y, b.x), fmaT(-t1, b.x, b.y));
-        const C cc = mk(fmaT(t2, c.y, c.x), fmaT(-t2, c.x, c.y));
-        S = mk(fmaT(r, cc.x, bb.x), fmaT(r, cc.y, bb.y));    // (b w^k + c w^2k) / cos th
-        D = mk(fmaT(-r, cc.x, bb.x), fmaT(-r, cc.y, bb.y));  // (b w^k - c w^2k) / cos th
-        y0 = mk(fmaT(c1, S.x, a.x), fmaT(c1, S.y, a.y));
-        T = mk(fmaT(-h, S.x, a.x), fmaT(-h, S.y, a.y));      // a - (v1 + v2) / 2
+        const float2 e1 = __ldg(tw + 3 * (Ns + k)), e2 = __ldg(tw + 3 * (Ns + k) + 1), e3 = __ldg(tw + 3 * (Ns + k) + 2);
+        const float t1 = SIGN < 0 ? e1.x : -e1.x, t2 = SIGN < 0 ? e2.x : -e2.x;
+        const float c1 = e1.y, r = e2.y, h = e3.x;
+        const float2 bb = make_float2(fmaf(t1, b.y, b.x), fmaf(-t1, b.x, b.y));
+        const float2 cc = make_float2(fmaf(t2, c.y, c.x), fmaf(-t2, c.x, c.y));
+        S = make_float2(fmaf(r, cc.x, bb.x), fmaf(r, cc.y, bb.y));    // (b w^k + c w^2k) / cos th
+        D = make_float2(fmaf(-r, cc.x, bb.x), fmaf(-r, cc.y, bb.y));  // (b w^k - c w^2k) / cos th
+        y0 = make_float2(fmaf(c1, S.x, a.x), fmaf(c1, S.y, a.y));
+        T = make_float2(fmaf(-h, S.x, a.x), fmaf(-h, S.y, a.y));      // a - (v1 + v2) / 2
         gs = SIGN < 0 ? e3.y : -e3.y;                                // (sqrt 3 / 2) cos th
       }
       // y1 = T - i (sqrt 3 / 2)(v1 - v2), y2 = T + i (sqrt 3 / 2)(v1 - v2) forward
       Y[0] = y0;
-      Y[Ns] = mk(fmaT(gs, D.y, T.x), fmaT(-gs, D.x, T.y));
-      Y[2 * Ns] = mk(fmaT(-gs, D.y, T.x), fmaT(gs, D.x, T.y));
+      Y[Ns] = make_float2(fmaf(gs, D.y, T.x), fmaf(-gs, D.x, T.y));
+      Y[2 * Ns] = make_float2(fmaf(-gs, D.y, T.x), fmaf(gs, D.x, T.y));
     }
     __syncthreads();
-    C* t = A;
+    float2* t = A;
     A = B;
     B = t;
   }
@@ -670,7 +658,7 @@ struct FftxMK {
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) A[q] = g[q];
     for (int q = nr * nx + threadIdx.x; q < R * nx; q += blockDim.x) A[q] = make_float2(0.0f, 0.0f);
     __syncthreads();
-    const float2* X = stockham<SIGN, float2>(A, B, nx, a.px, R, a.twx);
+    const float2* X = stockham<SIGN>(A, B, nx, a.px, R, a.twx);
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) g[q] = X[q];
   }
 };
@@ -797,7 +785,7 @@ struct FftxPK {
       issue(b + gdim_.x, st ^ 1);
       cp_async_wait<1>();  // every group but the newest: batch b has landed
       __syncthreads();
-      const float2* X = stockham<SIGN, float2>(buf + (2 * st) * rn, buf + (2 * st + 1) * rn, nx, a.px, R, a.twx);
+      const float2* X = stockham<SIGN>(buf + (2 * st) * rn, buf + (2 * st + 1) * rn, nx, a.px, R, a.twx);
       const long row0 = b * R;
       const int nr = (int)min((long)R, a.nrows - row0);
       float2* g = a.spec + row0 * nx;
@@ -1120,7 +1108,7 @@ struct DivzMK {
       }
     }
     __syncthreads();
-    const float2* R = stockham<-1, float2>(A, B, nz, a.pz, nseq, a.twz);
+    const float2* R = stockham<-1>(A, B, nz, a.pz, nseq, a.twz);
     const int nh = (nz >> 1) + 1;
     for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
       const int il = q & (TX - 1), m = q >> lt, c = il >> 1;
@@ -1520,7 +1508,7 @@ struct IfftzMK {
     }
     if (ACC) cp_async_wait<0>();
     __syncthreads();
-    const float2* R = stockham<1, float2>(A, B, nz, a.pz, nseq, a.twz);
+    const float2* R = stockham<1>(A, B, nz, a.pz, nseq, a.twz);
     for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
       const int il = q & (TX - 1), k = q >> lt;
       const float2 t = R[(il >> 1) * nz + k];
@@ -1533,8 +1521,8 @@ struct IfftzMK {
 };
 
 // ------------------------------------------------------------------------------------------
-// projection u = u* - s G phi; p += phi (if update_p).  One thread per (i, j) of kZ consecutive
-// z-planes, j = 0..ny.
+// projection u = u* - s G phi; p += phi (if update_p).  A thread takes kX cells in x of one
+// row j = 0..ny and kZ consecutive z-planes.
 // ------------------------------------------------------------------------------------------
 // Dyn: sx, sz, s, beta_p from device memory, else from the arguments; KM: the Kim-Moin pressure
 // update (compiled only into the variants that use it)
@@ -1785,7 +1773,7 @@ __global__ void __launch_bounds__(256) dctx_fwd_m_kernel(float2* __restrict__ sp
     A[rr * nx + dst] = rr < nr ? g[q] : make_float2(0, 0);
   }
   __syncthreads();
-  const float2* V = stockham<-1, float2>(A, B, nx, px, R, twx);
+  const float2* V = stockham<-1>(A, B, nx, px, R, twx);
   for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
     const int rr = q / nx, l = q - rr * nx;
     const float2 vl = V[rr * nx + l];
@@ -1793,7 +1781,7 @@ __global__ void __launch_bounds__(256) dctx_fwd_m_kernel(float2* __restrict__ sp
     const float2 w = __ldg(twd + nx + l);  // w_l / 2
     const float ax = vl.x + vn.x, ay = vl.y - vn.y;
     const float bx = vl.y + vn.y, by = vn.x - vl.x;
-    g[q] = make_float2(fmaT(w.x, ax, -w.y * ay), fmaT(w.x, bx, -w.y * by));
+    g[q] = make_float2(fmaf(w.x, ax, -w.y * ay), fmaf(w.x, bx, -w.y * by));
   }
 }
 
@@ -1814,12 +1802,12 @@ __global__ void __launch_bounds__(256) dctx_inv_m_kernel(float2* __restrict__ sp
       const float2 xn = l == 0 ? make_float2(0, 0) : g[rr * nx + nx - l];
       const float2 w = __ldg(twd + l);
       const auto ax = xl.x + xn.y, ay = xl.y - xn.x;  // X_l - i X_{N-l}
-      v = make_float2(fmaT(w.x, ax, w.y * ay), fmaT(w.x, ay, -w.y * ax));  // conj(w) (..)
+      v = make_float2(fmaf(w.x, ax, w.y * ay), fmaf(w.x, ay, -w.y * ax));  // conj(w) (..)
     }
     A[q] = v;
   }
   __syncthreads();
-  const float2* X = stockham<1, float2>(A, B, nx, px, R, twx);
+  const float2* X = stockham<1>(A, B, nx, px, R, twx);
   for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
     const int rr = q / nx, i = q - rr * nx;
     const int src = (i & 1) ? nx - 1 - (i >> 1) : (i >> 1);
