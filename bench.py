@@ -83,6 +83,11 @@ def kernel_model(nx, ny, nz, es):
     return m
 
 
+# Stages of the FP64 form whose products and sums run in 64-bit fixed point on the integer pipes
+# (csrc/fx64.cuh): the FP64 FMA rate is not their roof, and they are measured against HBM.
+FIXED_POINT = ("rhs", "adi_x", "poisson_div_fftz", "poisson_x_fwd", "poisson_x_inv", "poisson_ifftz")
+
+
 def load_peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
@@ -795,7 +800,7 @@ def main():
     else:
         alu_peak = (fp64_peak_tflops(smax) if fp64 else fp32_peak_tflops(smax)) * 1e12
         alu_src = "derived: 152 SMs x %s FMA/clk/SM x 2 x %.0f MHz" % ("2 FP64" if fp64 else "128 FP32", smax)
-    t_alu = f * cells / alu_peak
+    t_alu = 0.0 if es == 8 and top in FIXED_POINT else f * cells / alu_peak
     t_mem = b * cells / (hbm * 1e9)
     traffic = load_traffic(config["workload"], top)
     if t_alu >= t_mem:
@@ -813,7 +818,7 @@ def main():
         ach = b * cells / (per * 1e-3) / 1e9
         roof = {"kernel": top, "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
                 "frac": ach / hbm, "traffic": traffic, "peak_source": "%s hbm_gbs" % hbm_kind,
-                "algorithmic_bytes_per_launch": b * cells}
+                "algorithmic_bytes_per_launch": b * cells, "ms_per_launch": per}
 
     # end to end through the host-buffer entry point (pinned host memory)
     hu = torch.from_numpy(np.ascontiguousarray(u0)).pin_memory().numpy()
