@@ -85,7 +85,7 @@ def kernel_model(nx, ny, nz, es):
 
 # Stages of the FP64 form whose products and sums run in 64-bit fixed point on the integer pipes
 # (csrc/fx64.cuh): the FP64 FMA rate is not their roof, and they are measured against HBM.
-FIXED_POINT = ("rhs", "adi_x", "poisson_div_fftz", "poisson_x_fwd", "poisson_x_inv", "poisson_ifftz")
+FIXED_POINT = ("rhs", "poisson_div_fftz", "poisson_x_fwd", "poisson_x_inv", "poisson_ifftz")
 
 
 def load_peaks():

@@ -70,8 +70,8 @@ typedef enum {
 
 /* Precision of the increment path (Sec. 2.2 solves everything in one precision; the mixed
  * form is this library's addition):
- *   NS_FP64  : every stage on FP64 arrays; the right-hand side, the transforms and part of the x lines
- *              compute in 64-bit fixed point, with errors no larger than FP64 arithmetic leaves.
+ *   NS_FP64  : every stage on FP64 arrays; the right-hand side and the transforms compute in 64-bit
+ *              fixed point, with errors no larger than FP64 arithmetic leaves.
  *   NS_MIXED : RHS stencils and the ADI increment solves in FP32 (r, delta and N_prev stored
  *              as float); state accumulation u* = u + delta, divergence, the Poisson solve
  *              (all modes) and the projection stay FP64. */

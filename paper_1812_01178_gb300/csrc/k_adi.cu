@@ -8,8 +8,7 @@
 //      Z y   = E^T x~            (Eq. Zpdd)     interface unknowns y = (x^{(r)}_m, x^{(r+1)}_1)
 //      x     = x~ - Y y          (Eq. xpdd)
 //    PDD keeps only the 2x2 diagonal blocks of Z; PPT solves all of Z exactly by block parallel
-//    cyclic reduction over the team with warp shuffles (line-independent eliminators).  FP64: of each
-//    eight groups of lines four are solved in 64-bit fixed point, beside the FP64 ones.
+//    cyclic reduction over the team with warp shuffles (line-independent eliminators).
 // y: lines have stride nx; one thread per line, Thomas with precomputed factors.
 // z: lines have stride nx*ny and are periodic; one thread per line, Thomas on the Sherman-
 //    Morrison-modified matrix plus the rank-one correction; then u* = u + delta (FP64).
@@ -109,78 +108,6 @@ __device__ __forceinline__ void store_part(T* __restrict__ dst, const T (&d)[M])
   }
 }
 
-// ----------------------------------------------------------------------------------------------
-// x lines in 64-bit fixed point (fx64.cuh), beside the FP64 ones.  The FP64 x sweep was bound by the
-// FP64 pipe (four instructions an element of 16 cycles a warp); the same algebra in fixed point, each
-// line scaled by its own largest magnitude (the solutions of these diagonally dominant rows stay
-// below it), takes about 35 cycles of the integer pipes.  Neither alone is much faster, but the pipes
-// are different: of every eight groups of lines the first four go the fixed-point way (warps 0 to 3 of
-// a block, one on each SM sub-partition), the others the FP64 way.  The choice depends on the group's
-// number alone, so that every launch form solves a line alike.
-// ----------------------------------------------------------------------------------------------
-// (256 x 192 x 256: no group in fixed point 286 us, four of eight 186, five 194, six 195, all 222)
-__device__ __forceinline__ bool x_fixed_group(long g) { return (g & 7) < 4; }
-// An entry of the x tables as a coefficient; *ok turns false for magnitudes above 1
-__device__ __forceinline__ FxCoef x_coef(double c, bool* ok) {
-  const double m = fabs(c);
-  if (!(m <= 1.0)) *ok = false;
-  if (m < 1.0) return fx_limbs(fx_from(c, 1023));
-  const fx_t one = ((fx_t)1 << 62) - 1;
-  return fx_limbs(c < 0.0 ? -one : one);
-}
-// x w of |w| <= 1, sums of two such products, and the sum of two products with halved coefficients
-__device__ __forceinline__ fx_t x_mul(fx_t x, FxCoef w) {
-  FxAcc s = {0, (fx_t)1 << 29};
-  fx_wmac(s, x, w);
-  return s.h * 4 + (s.m >> 30);
-}
-__device__ __forceinline__ fx_t x_mul2(fx_t x, FxCoef w, fx_t y, FxCoef v) {
-  FxAcc s = {0, (fx_t)1 << 29};
-  fx_wmac(s, x, w);
-  fx_wmac(s, y, v);
-  return s.h * 4 + (s.m >> 30);
-}
-__device__ __forceinline__ fx_t x_mul2h(fx_t x, FxCoef w, fx_t y, FxCoef v) {
-  FxAcc s = {0, (fx_t)1 << 28};
-  fx_wmac(s, x, w);
-  fx_wmac(s, y, v);
-  return s.h * 8 + (s.m >> 29);
-}
-// One partition (lane r of a team of P) of a line by PDD, in place; F: the coefficients of its table
-// in the x-table layout, AINV, CP, V and W negated, the interface inverses halved; e: the line's exponent
-template <int M>
-__device__ __forceinline__ void x_solve_fixed(double (&d)[M], const FxCoef* F, int e, int r, int P, bool half) {
-  const FxCoef* INV = F + XT_INV * M * P + r;
-  const FxCoef* AINV = F + XT_AINV * M * P + r;
-  const FxCoef* CP = F + XT_CP * M * P + r;
-  const FxCoef* SV = F + XT_V * M * P + r;
-  const FxCoef* SW = F + XT_W * M * P + r;
-  const FxCoef* DINV = F + XT_NF * M * P + r;
-  const int s = e + 2;
-  fx_t q[M];
-  q[0] = x_mul(fx_cut(d[0], s), INV[0]);
-#pragma unroll
-  for (int i = 1; i < M; ++i) q[i] = x_mul2(fx_cut(d[i], s), INV[i * P], q[i - 1], AINV[i * P]);
-#pragma unroll
-  for (int i = M - 2; i >= 0; --i) q[i] += x_mul(q[i + 1], CP[i * P]);
-  const fx_t g0 = q[M - 1];
-  const fx_t g1 = __shfl_sync(NS_FULL_MASK, q[0], r + 1, P);
-  const fx_t y0 = x_mul2h(g0, DINV[0], g1, DINV[P]);
-  const fx_t y1 = x_mul2h(g0, DINV[2 * P], g1, DINV[3 * P]);
-  const fx_t left = __shfl_sync(NS_FULL_MASK, y0, r - 1 + P, P);
-  if (half) {
-#pragma unroll
-    for (int i = 0; i < M / 2; ++i) d[i] = fx_to(q[i] + x_mul(left, SV[i * P]), s);
-#pragma unroll
-    for (int i = M / 2; i < M; ++i) d[i] = fx_to(q[i] + x_mul(y1, SW[i * P]), s);
-  } else {
-#pragma unroll
-    for (int i = 0; i < M; ++i) d[i] = fx_to(q[i] + x_mul2(left, SV[i * P], y1, SW[i * P]), s);
-  }
-}
-// entries of the fixed-point part of an x table
-__host__ __device__ inline int x_fixed_count(int M, int P) { return (XT_NF * M + 4) * P; }
-
 template <typename T, int M>
 struct AdiXK {
   struct Args {
@@ -200,20 +127,6 @@ struct AdiXK {
   const int ntab = (int)xtab_count(M, P, L);
   const int ncls = a.bl ? 2 : 1;
   for (int q = threadIdx.x; q < ntab * ncls; q += blockDim.x) st[q] = q < ntab ? a.tab[0][q] : a.tab[1][q - ntab];
-  bool fixed = sizeof(T) == 8 && L == 0;  // fixed point: FP64 form, PDD, no entry above 1
-  FxCoef* ft = reinterpret_cast<FxCoef*>(st + ntab * ncls);
-  const int nf = x_fixed_count(M, P);
-  if constexpr (sizeof(T) == 8) {
-    if (fixed) {
-      bool ok = true;
-      for (int q = threadIdx.x; q < nf * ncls; q += blockDim.x) {
-        const int f = q < nf ? q : q - nf;
-        const double c = (q < nf ? a.tab[0] : a.tab[1])[f];
-        ft[q] = x_coef(f >= XT_NF * M * P ? 0.5 * c : f >= M * P ? -c : c, &ok);
-      }
-      fixed = __syncthreads_and(ok) != 0;
-    }
-  }
   __syncthreads();
 
   const int lane = threadIdx.x & 31;
@@ -246,21 +159,6 @@ struct AdiXK {
     } else {
 #pragma unroll
       for (int e = 0; e < M; ++e) d[e] = (T)0;
-    }
-    if constexpr (sizeof(T) == 8) {
-      if (fixed && x_fixed_group(l0 / teams)) {  // uniform over the warp
-        unsigned m = 0;
-#pragma unroll
-        for (int e = 0; e < M; ++e) m = max(m, fx_mag(d[e]));
-        for (int o = P >> 1; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(NS_FULL_MASK, m, o));
-        const int e = fx_exponent(m);
-        if (__all_sync(NS_FULL_MASK, fx_exponent_ok(e))) {
-          const int cls = a.bl && comp != 0 ? 1 : 0;
-          x_solve_fixed<M>(d, ft + cls * nf, e, r, P, a.sk->xhalf[cls] != 0);
-          if (valid) store_part<T, M>(row + r * M, d);
-          continue;
-        }
-      }
     }
     // A~ x~ = d on this partition (forward elimination, back substitution)
     d[0] = d[0] * INV[r];
@@ -885,6 +783,15 @@ void fill_x_args(ns_ctx* c, int k, AdiXArgs<T>& a) {
   for (int q = 0; q < 3; ++q) a.dout[q] = c->dout[q];
 }
 
+// Most blocks of an x sweep.  FP64: those the GPU holds at once, so that the tables are loaded once a
+// block: 256 x 192 x 256 286 us, 301 at 16 an SM.  FP32: 16 an SM.
+template <typename K, bool Resident>
+long x_blocks(const ns_ctx* c, int threads, size_t smem) {
+  int bps = 16;
+  if (Resident && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, single_kernel<K>, threads, smem) != cudaSuccess) bps = 1;
+  return (long)std::max(bps, 1) * c->num_sms;
+}
+
 template <typename T, int M>
 cudaError_t launch_x_t(LaunchSink& s, int k) {
   ns_ctx* c = s.c;
@@ -901,13 +808,10 @@ cudaError_t launch_x_t(LaunchSink& s, int k) {
   // room for the PPT tables: the levels are read from device memory and follow the mode in use
   int lmax = 0;
   while ((1 << lmax) < a.P) ++lmax;
-  const size_t smem = (xtab_count(M, a.P, lmax) * sizeof(T) +
-                       (sizeof(T) == 8 ? x_fixed_count(M, a.P) * sizeof(FxCoef) : 0)) * (a.bl ? 2 : 1);
+  const size_t smem = xtab_count(M, a.P, lmax) * sizeof(T) * (a.bl ? 2 : 1);
   const long teams_per_block = 8L * (32 / a.P);
   long blocks = (a.nlines + teams_per_block - 1) / teams_per_block;
-  // FP64: the blocks two of which an SM holds (the tables and their coefficients are loaded once a
-  // block: 256 x 192 x 256 195 us at 2 blocks an SM, 211 at 4, 227 at 16)
-  const long most = 152L * (sizeof(T) == 8 ? 2 : 16);
+  const long most = x_blocks<AdiXK<T, M>, sizeof(T) == 8>(c, 256, smem);
   if (blocks > most) blocks = most;
   return emit<AdiXK<T, M>>(s, AdiXK<T, M>::make(a), dim3((unsigned)blocks), dim3(256), smem);
 }
@@ -1061,7 +965,7 @@ cudaError_t launch_adi_z(ns_ctx* c, int k) {
 
 template <typename T, int M>
 cudaError_t short_attr() {
-  return set_smem_limit<AdiXK<T, M>>(2 * 64 * 1024);
+  return set_smem_limit<AdiXK<T, M>>(2 * 48 * 1024);
 }
 
 template <typename T>
