@@ -202,6 +202,12 @@ struct AdiXK {
   }
 };
 
+// Biased exponent of a spike or an interface value; infinities and NaN above every bound
+__device__ __forceinline__ int spike_exponent(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e == 0x7ff ? 1 << 20 : e;
+}
+
 // ----------------------------------------------------------------------------------------------
 // x, long lines (M = 24 ... 128 rows per partition, P = 32): the same algebra with each warp's line
 // staged in shared memory at stride M+1 per partition (conflict-free for 8-byte elements), the
@@ -227,22 +233,20 @@ struct AdiXLongK {
   const long warp = ((long)bid_.x * blockDim.x + threadIdx.x) >> 5;
   const long nwarps = ((long)gdim_.x * blockDim.x) >> 5;
   T* my = line_buf + r * (M + 1);
-  // FP64: rows at the ends of a partition whose spike is above the truncation tolerance (x_half_tol),
-  // by table: the first kv take v^(r), the last kw take w^(r) (a few of 32 rows; every row took both,
-  // two of its five FP64 instructions)
-  int kv[2] = {M, M}, kw[2] = {M, M};
+  // FP64: a row's correction v^(r)_e x^{(r-1)}_m + w^(r)_e x^{(r+1)}_1 is formed only where it can change
+  // the row: both terms below a quarter of the last place of x~_e leave it as it is, bit for bit.  The
+  // spikes fall off by the rows' dominance, so that most of the M rows are left out (two FP64
+  // instructions of five).  The bounds are exponents: spike[table][v, w][e] is the largest of the
+  // spikes' over the partitions.
+  __shared__ int spike[2][2][sizeof(T) == 8 ? M : 1];
   if constexpr (sizeof(T) == 8) {
-    for (int c = 0; c < (a.bl ? 2 : 1); ++c) {
-      const T* V = a.tab[c] + XT_V * M * P + r;
-      const T* W = a.tab[c] + XT_W * M * P + r;
-      int v = 0, w = 0;
-      for (int e = 0; e < M; ++e) {
-        if (fabs(__ldg(V + e * P)) > 1e-17) v = e + 1;
-        if (fabs(__ldg(W + (M - 1 - e) * P)) > 1e-17) w = e + 1;
-      }
-      kv[c] = __reduce_max_sync(NS_FULL_MASK, v);
-      kw[c] = __reduce_max_sync(NS_FULL_MASK, w);
+    for (int q = threadIdx.x >> 5; q < (a.bl ? 4 : 2) * M; q += kThreads / 32) {
+      const int e = q % M, vw = q / M & 1, c = q / (2 * M);
+      const T* t = a.tab[c] + (vw ? XT_W : XT_V) * M * P + e * P + r;
+      const int x = __reduce_max_sync(NS_FULL_MASK, spike_exponent(__ldg(t)));
+      if (r == 0) spike[c][vw][e] = x;
     }
+    __syncthreads();
   }
   for (long line = warp; line < a.nlines; line += nwarps) {
     int comp;
@@ -296,10 +300,16 @@ struct AdiXLongK {
     const T y1 = __ldg(DINV + 2 * P + r) * g0 + __ldg(DINV + 3 * P + r) * g1;
     const T left = __shfl_sync(NS_FULL_MASK, y0, r - 1 + P, P);
     if constexpr (sizeof(T) == 8) {
-      const int cls = a.bl && comp != 0 ? 1 : 0;
-      const int nv = cls ? kv[1] : kv[0], nw = cls ? kw[1] : kw[0];
-      for (int e = 0; e < nv; ++e) my[e] = my[e] - __ldg(SV + e * P + r) * left;
-      for (int e = M - nw; e < M; ++e) my[e] = my[e] - __ldg(SW + e * P + r) * y1;
+      const int* sv = spike[a.bl && comp != 0 ? 1 : 0][0];
+      const int ev = spike_exponent(left), ew = spike_exponent(y1);
+#pragma unroll 4
+      for (int e = 0; e < M; ++e) {
+        const T x = my[e];
+        // |x| >= 2^(ex - 1023), each term below 2^(its two exponents - 2044)
+        const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+        if (ex == 0 || max(sv[e] + ev, sv[M + e] + ew) > ex + 966)
+          my[e] = x - __ldg(SV + e * P + r) * left - __ldg(SW + e * P + r) * y1;
+      }
     } else {
       for (int e = 0; e < M; ++e) my[e] = my[e] - __ldg(SV + e * P + r) * left - __ldg(SW + e * P + r) * y1;
     }
@@ -783,8 +793,8 @@ void fill_x_args(ns_ctx* c, int k, AdiXArgs<T>& a) {
   for (int q = 0; q < 3; ++q) a.dout[q] = c->dout[q];
 }
 
-// Most blocks of an x sweep.  FP64: those the GPU holds at once, so that the tables are loaded once a
-// block: 256 x 192 x 256 286 us, 301 at 16 an SM.  FP32: 16 an SM.
+// Most blocks of an x sweep.  FP64: those the GPU holds at once, so that the tables (and the bounds of
+// the spikes) are loaded once a block: 256 x 192 x 256 286 us, 301 at 16 an SM.  FP32: 16 an SM.
 template <typename K, bool Resident>
 long x_blocks(const ns_ctx* c, int threads, size_t smem) {
   int bps = 16;
@@ -831,7 +841,7 @@ cudaError_t launch_x_long_t(LaunchSink& s, int k) {
   a.nlines = (long)a.nz * a.ny * 2 + (long)a.nz * (a.ny - 1);
   const size_t smem = (size_t)4 * 32 * (M + 1) * sizeof(T);
   long blocks = (a.nlines + 3) / 4;
-  const long most = 152L * (sizeof(T) == 8 ? 6 : 16);  // FP64: the blocks an SM holds at 1024 rows
+  const long most = x_blocks<AdiXLongK<T, M>, sizeof(T) == 8>(c, 128, smem);
   if (blocks > most) blocks = most;
   return emit<AdiXLongK<T, M>>(s, AdiXLongK<T, M>::make(a), dim3((unsigned)blocks), dim3(128), smem);
 }

@@ -99,3 +99,47 @@ def test_small_entries_beside_a_large_one(nx, M):
         bound = _pdd(np.abs(a[live]), r, M)
         assert (np.abs(g[live] - _pdd(a[live], r, M)) <= 1e-14 * bound).all()
     s.close()
+
+
+@pytest.mark.parametrize("nx, M", [(768, 24), (1024, 32), (2048, 64), (4096, 128)])
+def test_long_lines_far_from_their_sources(nx, M):
+    """Zero lines but for one row: the solution falls off through the neighbouring partition, by the decay
+    of the rows to 1e-40 and below, and keeps its digits there (down to 1e-280: short of underflow).  Four
+    roundings a row between: the factor's pivot and quotient, the spike's product and the sweep's."""
+    r = 0.03
+    s = _solver(nx, r, M)
+    lines = [np.zeros((len(q), nx)) for q in _live(s)]
+    at = 5 * M + M - 1  # the last row of a partition
+    for a in lines:
+        a[:, at] = 1.0
+    got = _sweep(s, lines)
+    want = _pdd(lines[0][0], r, M)
+    near = np.flatnonzero(want > 1e-280)
+    near = near[(near >= 4 * M) & (near < 7 * M)]  # the partition of the source and its neighbours
+    tol = 1e-14 + 4 * 2.0 ** -53 * np.abs(near - at)
+    for g, live in zip(got, _live(s)):
+        assert (np.abs(g[live][:, near] - want[near]) <= tol * want[near]).all()
+    s.close()
+
+
+@pytest.mark.parametrize("nx, M", [(768, 24), (1024, 32)])
+def test_long_lines_of_uneven_size(nx, M):
+    """Entries that change by orders of magnitude from row to row, zeros, and an infinity or a NaN that stays
+    in the partitions next to it."""
+    r = 0.03
+    s = _solver(nx, r, M)
+    rng = np.random.default_rng(nx + 2)
+    lines = [rng.standard_normal((len(q), nx)) * 2.0 ** rng.integers(-30, 30, (len(q), nx)) for q in _live(s)]
+    for a in lines:
+        a[rng.random(a.shape) < 0.1] = 0.0
+    got = _sweep(s, lines)
+    for g, a, live in zip(got, lines, _live(s)):
+        assert (np.abs(g[live] - _pdd(a[live], r, M)) <= 1e-14 * _pdd(np.abs(a[live]), r, M)).all()
+    for bad in (np.inf, np.nan):
+        spoilt = [a.copy() for a in lines]
+        for a in spoilt:
+            a[:, 3 * M + 1] = bad
+        for g, h, live in zip(_sweep(s, spoilt), got, _live(s)):
+            assert not np.isfinite(g[live][:, 2 * M:5 * M]).any()
+            assert (g[live][:, 6 * M:] == h[live][:, 6 * M:]).all()
+    s.close()
