@@ -595,7 +595,7 @@ struct RhsFxK {
   static constexpr int kThreads = FXR_THREADS;
   static constexpr int kMinBlocks = 3;  // shared memory holds three; 72 registers
 
-  // exponent of a plane (bit 62 of its integers); zero planes take the lowest, to raise no bound
+  // exponent of a plane (bit 62 of its integers); zero planes take the lowest
   static __device__ __forceinline__ int plane_e(unsigned m) { return (m == 0 ? 128 : (int)(m >> 20)) + 2; }
   static __device__ __forceinline__ bool plane_ok(unsigned m) { return m == 0 || fx_exponent_ok((int)(m >> 20)); }
 
@@ -683,9 +683,15 @@ struct RhsFxK {
         tr.add = 1023;
       }
     }
+    // the scale of a term's values; FX_NONE where they are zero (a factor's planes are)
     auto scale = [&](const Term& t, int J) {
-      auto pe = [&](int s) { return s == ZERO ? 0 : plane_e(S.mag[(J - 1 + (s >> 2)) & 3][s & 3]); };
-      return max(pe(t.a), pe(t.b)) + max(pe(t.c), pe(t.d)) + t.add;
+      auto pe = [&](int x, int y) {
+        if (x == ZERO) return 0;
+        const unsigned m = max(S.mag[(J - 1 + (x >> 2)) & 3][x & 3], S.mag[(J - 1 + (y >> 2)) & 3][y & 3]);
+        return m == 0 ? FX_NONE : plane_e(m);
+      };
+      const int f = pe(t.a, t.b), h = pe(t.c, t.d);
+      return f == FX_NONE || h == FX_NONE ? FX_NONE : f + h + t.add;
     };
     auto row = [&](int J) {  // planes J - 1 .. J + 1 are known
       const int par = J & 1;
@@ -694,7 +700,7 @@ struct RhsFxK {
       if (wall && lane < 4) cn = 0.0;
       if (wall && gr == 0) cr = 0.0;
       const int etn = scale(tn, J), etr = scale(tr, J);
-      const int een = fx_wexp(cn, etn), eer = fx_wexp(cr, etr);
+      const int een = etn == FX_NONE ? FX_NONE : fx_wexp(cn, etn), eer = etr == FX_NONE ? FX_NONE : fx_wexp(cr, etr);
       int mn = een, mr = eer;
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) {
