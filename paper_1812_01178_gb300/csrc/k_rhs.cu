@@ -45,9 +45,10 @@ struct RhsArgs {
 
 namespace {
 
-// The right-hand side at (i, j, k): u, w of cell row j (j < ny) and v of face row j (zero on the walls)
+// The right-hand side at (i, j, k): u, w of cell row j (j < ny) and v of face row j (zero on the walls);
+// stored if `store`
 template <typename T, typename TR>
-__device__ __forceinline__ void rhs_cell(const RhsArgs& a, int i, int j, int k, T dt) {
+__device__ __forceinline__ void rhs_cell(const RhsArgs& a, int i, int j, int k, T dt, bool store) {
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const int ip = (i + 1 == nx) ? 0 : i + 1;
   const int im = (i == 0) ? nx - 1 : i - 1;
@@ -127,8 +128,10 @@ __device__ __forceinline__ void rhs_cell(const RhsArgs& a, int i, int j, int k, 
       T r = dt * (-alp * gp + avis * lap + (T)(a.alp * a.fx)) + nt;
       if (a.zet != 0.0) r += cpn * (T)nu[cc];
       const bool fixed = bl && i == 0;  // inflow face
-      ru[cc] = fixed ? (TR)0 : (TR)r;
-      nu[cc] = fixed ? (TR)0 : (TR)nt;
+      if (store) {
+        ru[cc] = fixed ? (TR)0 : (TR)r;
+        nu[cc] = fixed ? (TR)0 : (TR)nt;
+      }
     }
     // ---------------- w at (xc_i, yc_j, zf_k)
     {
@@ -153,16 +156,17 @@ __device__ __forceinline__ void rhs_cell(const RhsArgs& a, int i, int j, int k, 
       const T nt = cn * n;
       T r = dt * (-alp * gp + avis * lap) + nt;
       if (a.zet != 0.0) r += cpn * (T)nw[cc];
-      rw[cc] = (TR)r;
-      nw[cc] = (TR)nt;
+      if (store) {
+        rw[cc] = (TR)r;
+        nw[cc] = (TR)nt;
+      }
     }
   }
   // ---------------- v at (xc_i, yf_j, zc_k)
   {
     const long cf = ((long)k * ny1 + j) * nx + i;
     if (j == 0 || j == ny) {
-      rv[cf] = (TR)0;
-      nv[cf] = (TR)0;
+      if (store) rv[cf] = nv[cf] = (TR)0;
       return;
     }
     const T v0 = V(i, j, k), vxp = V(ipx, j, k), vxm = V(imx, j, k);
@@ -186,8 +190,10 @@ __device__ __forceinline__ void rhs_cell(const RhsArgs& a, int i, int j, int k, 
     const T nt = cn * n;
     T r = dt * (-alp * gp + avis * lap) + nt;
     if (a.zet != 0.0) r += cpn * (T)nv[cf];
-    rv[cf] = (TR)r;
-    nv[cf] = (TR)nt;
+    if (store) {
+      rv[cf] = (TR)r;
+      nv[cf] = (TR)nt;
+    }
   }
 }
 
@@ -207,7 +213,7 @@ struct RhsK {
     const long q = (long)bid_.x * blockDim.x + threadIdx.x;
     if (q >= (long)a.nx * (a.ny + 1)) return;
     const int j = (int)(q / a.nx);
-    rhs_cell<T, TR>(a, (int)(q - (long)j * a.nx), j, bid_.y, (T)(Dyn ? a.sk->dt : a.kc.dt));
+    rhs_cell<T, TR>(a, (int)(q - (long)j * a.nx), j, bid_.y, (T)(Dyn ? a.sk->dt : a.kc.dt), true);
   }
 };
 
@@ -542,7 +548,7 @@ struct RhsTiledK {
 // In FP64 arithmetic the tile was bound by the FP64 pipe: 64.8 instructions a cell of 16 cycles a
 // warp, 1.547 ms on 256 x 192 x 256 cells with the pipe 88 % busy.  Here the products and the viscous
 // sums run on the integer pipes; the FP64 pipe keeps 12 instructions a cell (pressure gradient, the
-// stored N, closing the sum): 0.677 ms, about a thousand instructions a cell and warp, bound by the
+// stored N, closing the sum): 0.664 ms, about a thousand instructions a cell and warp, bound by the
 // latency of their chains.  Tile and block from timings: 32 x 16 cells, two a thread, two blocks an SM
 // 0.705; 32 x 16, one a thread (56 registers, 200 bytes spilled) 0.849; 32 x 12 0.773; this one, 27
 // warps an SM, 0.677; with the viscous sum converted by the FP64 pipe (18 instructions) 0.704.  r is 3
@@ -557,12 +563,20 @@ struct RhsTiledK {
 // bounds of its terms, while the others work on row j.
 //
 // A row next to a plane of u, v or w that holds an infinity, a NaN or values near the ends of the
-// binary64 range is formed in FP64 arithmetic (rhs_cell).
+// binary64 range is formed in FP64 arithmetic (rhs_cell), and so is a cell that is quiet beside a larger
+// value of its tile: one that, with its upper neighbours in x and z, keeps fewer than 53 bits of u, v
+// or w (FXR_NEAR; of the largest of the tile's three planes, whose scales the sums share).  So the values
+// a sum is made of are held as FP64 holds them, against the largest near the cell, and its error is a few
+// 2^-60 of the largest terms that the tile's values allow.  The three values rarely are so small together:
+// the benchmark's fields take 664 us at first and 668 after 20 steps (677 without the test, whose one call
+// of rhs_cells_fp64 for both reasons also lets the compiler spill less).  At 55 bits 762; with the cell and
+// one neighbour 768 to 969; every term of every sum held to 2^-44 of its bound 720, to 2^-48 1250.
 // ---------------------------------------------------------------------------------------------
 constexpr int FXR_X = 32, FXR_Z = 8;
 constexpr int FXR_PX = FXR_X + 2, FXR_PZ = FXR_Z + 2, FXR_PLANE = FXR_PX * FXR_PZ;
 constexpr int FXR_WARPS = FXR_Z;  // worker warps, a z row each; one more forms coefficients
 constexpr int FXR_THREADS = 32 * (FXR_WARPS + 1);
+constexpr int FXR_NEAR = 20;  // 2^20 in the high word: 53 bits
 
 struct RhsFxTile {
   // u, v, w planes (ring of 5: three in use, one being converted, one arriving as FP64), p planes
@@ -580,11 +594,14 @@ struct RhsFxTile {
   int en[2][4];                    // scales of n
   int er[2][4];                    // scales of the viscous sums
   int bad[2];                      // the row takes FP64 arithmetic
+  int4 least[2];                   // least high words of u, v, w near a cell (row parity)
   unsigned mag[4][4];              // largest high words of the planes (j mod 4) of u, v, w
 };
 
-__device__ __noinline__ void rhs_cell_fp64(const RhsArgs& a, int i, int j, int k) {
-  rhs_cell<double, double>(a, i, j, k, a.sk->dt);
+// The cells of a warp in FP64 arithmetic.  Whole warps make this call, and `store` says which lanes keep the
+// result: calls by some lanes of a warp beside others in the fixed-point branch are left out of the kernel.
+__device__ __noinline__ void rhs_cells_fp64(const RhsArgs& a, int i, int j, int k, bool store) {
+  rhs_cell<double, double>(a, min(i, a.nx - 1), j, k, a.sk->dt, store);
 }
 
 struct RhsFxK {
@@ -724,6 +741,12 @@ struct RhsFxK {
         if (qr < 5) S.cr[par][lane] = eer == FX_NONE ? FxCoef{0, 0} : fx_wcoef(cr, etr, er);
         if (qr == 0) S.er[par][gr] = er;
         if (lane == 13) S.cb[par] = eer == FX_NONE ? 0 : fx_from(cr, er);
+      }
+      if (lane < 3) {
+        const unsigned lo = S.mag[(J - 1) & 3][lane], at = S.mag[J & 3][lane], up = S.mag[(J + 1) & 3][lane];
+        const unsigned m = max(at, max(lo, up));
+        const int s = FXR_NEAR + plane_e(m) - plane_e(wall && lane == V ? up : at);
+        (&S.least[par].x)[lane] = m == 0 ? 0 : s > 30 ? 0x7fffffff : 1 << s;
       }
       const bool good = __all_sync(NS_FULL_MASK, ok);
       if (lane == 0) {
@@ -947,9 +970,8 @@ struct RhsFxK {
       const fx_t q2 = square_v(j, s0, s1);
       __syncthreads();
       const int par = j & 1, f0 = j & 1, f1 = f0 ^ 1;
-      if (S.bad[par]) {
-        if (active) rhs_cell_fp64(a, i, j, k);
-      } else {
+      bool fp64 = S.bad[par] != 0;  // this cell takes FP64 arithmetic
+      if (!fp64) {
         const FxCoef* cn = S.cn[par];
         const FxCoef* cr = S.cr[par];
         // The viscous sum of field f; o: the plane's values at the cell, the z neighbours below and
@@ -971,6 +993,12 @@ struct RhsFxK {
         const double* pj = S.pp[pc] + e0;
         const double p0 = pj[0];
         fx_t o[5];
+        // the bits of the cell and its upper neighbours in x and z
+        auto bits = [](fx_t x, fx_t y, fx_t z) {
+          const int a = fx_hi(x), b = fx_hi(y), c = fx_hi(z);
+          return (a ^ (a >> 31)) | (b ^ (b >> 31)) | (c ^ (c >> 31));
+        };
+        int3 size;
         double nd[3], rd[3];  // stored together at the end: the FP64 sums finish meanwhile
         // ---------------- v at face j
         {
@@ -980,6 +1008,11 @@ struct RhsFxK {
           fx_wmac(n, q2, cn[1]);
           fx_wmac(n, q2prev, cn[2]);
           viscous(s, 1, cr, o);
+          size.y = bits(o[0], o[2], o[4]);
+          if (j == 0) {  // v is zero on the wall: the plane above decides
+            const fx_t* pv = S.pl[1][s1] + e0;
+            size.y = bits(pv[0], pv[FXR_PX], pv[1]);
+          }
           nd[0] = fx_to(fx_wsum(n), S.en[par][0]);
           const double dp = p0 - S.pp[pm][e0];
           rd[0] = (fx_to(fx_wsum(s), S.er[par][0]) + fma(S.cgy[par], dp, fma(cp, prev[0], nd[0])));
@@ -991,6 +1024,7 @@ struct RhsFxK {
           fx_wmac(n, S.fuv[f1][wz][lane], cn[5]);
           fx_wmac(n, S.fuv[f0][wz][lane], cn[6]);
           viscous(s, 0, cr + 8, o);
+          size.x = bits(o[0], o[2], o[4]);
           fx_wmac(n, fx_sqrhi(o[0] + o[4]) - fx_sqrhi(o[3] + o[0]), cn[4]);
           nd[1] = fx_to(fx_wsum(n), S.en[par][1]);
           rd[1] = (fx_to(fx_wsum(s), S.er[par][1]) + fma(cgx, p0 - pj[-1], fma(cp, prev[1], nd[1])));
@@ -1002,11 +1036,14 @@ struct RhsFxK {
           fx_wmac(n, S.fvw[f1][wz][lane], cn[9]);
           fx_wmac(n, S.fvw[f0][wz][lane], cn[10]);
           viscous(s, 2, cr + 16, o);
+          size.z = bits(o[0], o[2], o[4]);
           fx_wmac(n, fx_sqrhi(o[0] + o[2]) - fx_sqrhi(o[1] + o[0]), cn[11]);
           nd[2] = fx_to(fx_wsum(n), S.en[par][2]);
           rd[2] = (fx_to(fx_wsum(s), S.er[par][2]) + fma(cgz, p0 - pj[-FXR_PX], fma(cp, prev[2], nd[2])));
         }
-        if (active) {
+        const int4 least = S.least[par];
+        fp64 = size.x < least.x || size.y < least.y || size.z < least.z;
+        if (active && !fp64) {
           const bool wall = j == 0, fixed = a.bl && i == 0;  // the wall row of v, the inflow face of u
           nv[cf] = nd[0];
           rv[cf] = wall ? 0.0 : rd[0];
@@ -1016,6 +1053,8 @@ struct RhsFxK {
           rw[cc] = rd[2];
         }
       }
+      const bool store64 = active && fp64;
+      if (__any_sync(NS_FULL_MASK, store64)) rhs_cells_fp64(a, i, j, k, store64);
       q2prev = q2;
       {  // the rings move on by one plane
         const int t = sm;
