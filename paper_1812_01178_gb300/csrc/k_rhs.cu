@@ -564,13 +564,14 @@ struct RhsTiledK {
 //
 // A row next to a plane of u, v or w that holds an infinity, a NaN or values near the ends of the
 // binary64 range is formed in FP64 arithmetic (rhs_cell), and so is a cell that is quiet beside a larger
-// value of its tile: one that, with its upper neighbours in x and z, keeps fewer than 53 bits of u, v
-// or w (FXR_NEAR; of the largest of the tile's three planes, whose scales the sums share).  So the values
-// a sum is made of are held as FP64 holds them, against the largest near the cell, and its error is a few
-// 2^-60 of the largest terms that the tile's values allow.  The three values rarely are so small together:
-// the benchmark's fields take 664 us at first and 668 after 20 steps (677 without the test, whose one call
-// of rhs_cells_fp64 for both reasons also lets the compiler spill less).  At 55 bits 762; with the cell and
-// one neighbour 768 to 969; every term of every sum held to 2^-44 of its bound 720, to 2^-48 1250.
+// value of its tile: one that, with its neighbours in x and z, keeps fewer than 53 bits of u, v or w
+// (FXR_NEAR; of the largest of the tile's three planes, whose scales the sums share).  So the values a sum
+// is made of are held as FP64 holds them, against the largest near the cell, and its error is a few
+// 2^-60 of the largest terms that the tile's values allow.  The five values rarely are so small together,
+// and a call costs a row about 8 us: with the cell and its upper neighbours alone the benchmark's fields took
+// 664 us at first, but the flat plate of 384 x 96 x 128 went from 341 to 430 in 80 steps, as values in the first
+// tile fall off from the inflow; with all four neighbours 676 (677 without the test) and 338 to 373.  Every
+// term of every sum held to 2^-44 of its bound took 720, to 2^-48 1250.
 // ---------------------------------------------------------------------------------------------
 constexpr int FXR_X = 32, FXR_Z = 8;
 constexpr int FXR_PX = FXR_X + 2, FXR_PZ = FXR_Z + 2, FXR_PLANE = FXR_PX * FXR_PZ;
@@ -993,10 +994,12 @@ struct RhsFxK {
         const double* pj = S.pp[pc] + e0;
         const double p0 = pj[0];
         fx_t o[5];
-        // the bits of the cell and its upper neighbours in x and z
-        auto bits = [](fx_t x, fx_t y, fx_t z) {
-          const int a = fx_hi(x), b = fx_hi(y), c = fx_hi(z);
-          return (a ^ (a >> 31)) | (b ^ (b >> 31)) | (c ^ (c >> 31));
+        // the bits of the cell and its neighbours in x and z (as in `viscous`)
+        auto bits = [](const fx_t* o) {
+          int b = 0;
+#pragma unroll
+          for (int q = 0; q < 5; ++q) b |= fx_hi(o[q]) ^ (fx_hi(o[q]) >> 31);
+          return b;
         };
         int3 size;
         double nd[3], rd[3];  // stored together at the end: the FP64 sums finish meanwhile
@@ -1008,10 +1011,11 @@ struct RhsFxK {
           fx_wmac(n, q2, cn[1]);
           fx_wmac(n, q2prev, cn[2]);
           viscous(s, 1, cr, o);
-          size.y = bits(o[0], o[2], o[4]);
+          size.y = bits(o);
           if (j == 0) {  // v is zero on the wall: the plane above decides
-            const fx_t* pv = S.pl[1][s1] + e0;
-            size.y = bits(pv[0], pv[FXR_PX], pv[1]);
+            const fx_t* p = S.pl[1][s1] + e0;
+            const fx_t up[5] = {p[0], p[-FXR_PX], p[FXR_PX], p[-1], p[1]};
+            size.y = bits(up);
           }
           nd[0] = fx_to(fx_wsum(n), S.en[par][0]);
           const double dp = p0 - S.pp[pm][e0];
@@ -1024,7 +1028,7 @@ struct RhsFxK {
           fx_wmac(n, S.fuv[f1][wz][lane], cn[5]);
           fx_wmac(n, S.fuv[f0][wz][lane], cn[6]);
           viscous(s, 0, cr + 8, o);
-          size.x = bits(o[0], o[2], o[4]);
+          size.x = bits(o);
           fx_wmac(n, fx_sqrhi(o[0] + o[4]) - fx_sqrhi(o[3] + o[0]), cn[4]);
           nd[1] = fx_to(fx_wsum(n), S.en[par][1]);
           rd[1] = (fx_to(fx_wsum(s), S.er[par][1]) + fma(cgx, p0 - pj[-1], fma(cp, prev[1], nd[1])));
@@ -1036,7 +1040,7 @@ struct RhsFxK {
           fx_wmac(n, S.fvw[f1][wz][lane], cn[9]);
           fx_wmac(n, S.fvw[f0][wz][lane], cn[10]);
           viscous(s, 2, cr + 16, o);
-          size.z = bits(o[0], o[2], o[4]);
+          size.z = bits(o);
           fx_wmac(n, fx_sqrhi(o[0] + o[2]) - fx_sqrhi(o[1] + o[0]), cn[11]);
           nd[2] = fx_to(fx_wsum(n), S.en[par][2]);
           rd[2] = (fx_to(fx_wsum(s), S.er[par][2]) + fma(cgz, p0 - pj[-FXR_PX], fma(cp, prev[2], nd[2])));
