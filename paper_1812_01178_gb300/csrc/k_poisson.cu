@@ -175,25 +175,33 @@ __device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, con
 // on the integer pipes (fx64.cuh).  In FP64 arithmetic they ran at 0.86-0.9 of the FP64 pipe's rate
 // (22 instructions of 16 cycles a warp per radix-4 butterfly); in fixed point a butterfly is 36
 // multiply-adds of about 1.3 cycles and some 100 additions, shifts and logic operations on the
-// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 216 (six FP64
-// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 117, inverse z 295 ->
-// 135; bound by instruction issue and latency (2.1 instructions a cycle at 32 warps an SM).  Results
-// go back to FP64 by two exact FP64 instructions and a scaling on the otherwise idle pipe (x,
-// inverse z), or by integer steps (after the divergence, which uses that pipe).  Every sequence is scaled by its own largest component; before each stage the block
-// shifts by 0, 1 or 2 bits, as its largest value (the or of all magnitudes, gathered while the last
-// stage was written) needs for the next sums to stay below 2^62.  The result is nearer to the exact
-// transform than FP64 butterflies were, at every length and shape of data tried (2 to 4 times on
-// noise and smooth data, 1.3 times on 1/i^2 decay at 1024).  Sequences that hold an infinity, a
-// NaN or values near the ends of the binary64 range take FP64 butterflies (plain_stockham).
+// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 220 (six FP64
+// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 123, inverse z 295 -> 136.
+// Results go back to FP64 by two exact FP64 instructions and a scaling on the otherwise idle pipe (x,
+// inverse z), or by integer steps (after the divergence, which uses that pipe).
+//
+// Every sequence is scaled by its own largest component, and before each stage shifted by 0, 1 or 2 bits,
+// as its own largest value (the or of its magnitudes, gathered while the last stage was written) needs for
+// the next sums to stay below 2^62.  (One shift for all sequences of a block took 583 us for the four
+// transforms, 602 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
+// 1024 where FP64 butterflies leave 1.6e-16.)  A sequence's relative error in the 2-norm is then 4e-17 to
+// 1e-16, against 1.1e-16 to 7e-16 with FP64 butterflies, on noise, smooth and decaying data, pulses and steps of 24
+// to 4096 points.  It is one of the whole sequence: of the two real columns that a z sequence packs, one whose sum
+// grows lets the other lose digits (a pulse beside a constant: below FP64's 1.5e-16 up to 256 points, 1.9e-16 at 512,
+// 5e-16 at 1024, 1.5e-15 at 4096), where FP64 butterflies lose them only to a larger column (of 1000 times
+// the size: 3e-13 against 3e-14 here).  Sequences that hold an infinity, a NaN or values near the ends of the
+// binary64 range take FP64 butterflies (plain_stockham).
 //
 // Sequences stand in shared memory with a pitch of N + 1 elements of 16 bytes (columns of one row
 // fall into different banks) and, in fixed point, element i at fx_slot(i): the stages' writes at
 // strides 4, 8 and 16 are then free of bank conflicts, and so are their contiguous reads.
 // ------------------------------------------------------------------------------------------
-constexpr int FX_SEQ = 16;  // sequences a block holds at most
+constexpr int FX_SEQ = 16;     // sequences a block holds at most
+constexpr int FX_STAGES = 8;   // of lengths 2^a 3^b <= 4096, a >= 3: at most 7
 struct FxBlock {
-  unsigned emax[FX_SEQ];  // largest high word of each sequence
-  unsigned span[16];      // or of the magnitudes after each stage
+  unsigned emax[FX_SEQ];             // by sequence: the largest high word,
+  unsigned span[FX_STAGES][FX_SEQ];  // the or of the magnitudes after each stage,
+  int t[FX_SEQ];                     // where its results stand: bit 62 is exponent(emax) + t
 };
 __device__ __forceinline__ int fx_slot(int i) {
   const int t = (i >> 3) & 3;
@@ -211,10 +219,8 @@ __device__ __forceinline__ double2 fx_twd(FxTw w) {  // as doubles (general path
 __host__ __device__ __forceinline__ int fx_stages(int plan) { return (plan & 1) + ((plan & 0xff) >> 1) + (plan >> 8); }
 // all threads, before the loads of a block
 __device__ __forceinline__ void fx_begin(FxBlock& S) {
-  if (threadIdx.x < FX_SEQ) {
-    S.emax[threadIdx.x] = 0;
-    S.span[threadIdx.x] = 0;
-  }
+  if (threadIdx.x < FX_SEQ) S.emax[threadIdx.x] = 0;
+  if (threadIdx.x < FX_STAGES * FX_SEQ) (&S.span[0][0])[threadIdx.x] = 0;
   __syncthreads();
 }
 // The barrier after the loads: whether every sequence's exponent suits the fixed-point path
@@ -225,17 +231,33 @@ __device__ __forceinline__ bool fx_loaded(const FxBlock& S, int nseq) {
   return ok;
 }
 
-// One radix-4 stage of power-of-two sequences (N = 2^a2, total butterflies over all sequences).
-// fx_slot is linear over exclusive or, and j, r N / 4 and r Ns have no bits in common with what they
-// are added to, so each thread takes the slot of its first element and flips the bits of the others.
-// RAW: the inputs are doubles (t0 as in fx_from); TW: twiddles; SH: the shift before the sums.
-template <int SIGN, bool RAW, bool TW, int SH>
-__device__ __forceinline__ unsigned fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, int total, int ls,
-                                              const FxTw* __restrict__ tw, const FxBlock& S) {
+// `span` of the lanes of a warp that work on sequence sq joins *slot; `lanes`: those lanes
+__device__ __forceinline__ void fx_gather_span(unsigned span, unsigned lanes, unsigned* slot) {
+  span = __reduce_or_sync(lanes, span);
+  if ((threadIdx.x & 31) == __ffs(lanes) - 1) atomicOr(slot, span);
+}
+
+// x[1..3] times their twiddles, and all four 2^-SH
+template <int SIGN, int SH>
+__device__ __forceinline__ void fx_twiddle4(Fx2 (&x)[4], const FxTw (&w)[3]) {
+  x[0] = fx_shr(x[0], SH);
+#pragma unroll
+  for (int r = 1; r < 4; ++r) x[r] = fx_cmul<SIGN>(x[r], w[r - 1], SH);
+}
+
+// One radix-4 stage of power-of-two sequences (N = 2^a2), `total` butterflies over all of them.  fx_slot is
+// linear over exclusive or, and j, r N / 4 and r Ns have no bits in common with what they are added to, so
+// each thread takes the slot of its first element and flips the bits of the others.  RAW: the inputs are
+// doubles; TW: twiddles.  before: the spans the sequences' shifts follow from, after: those of the results.
+template <int SIGN, bool RAW, bool TW>
+__device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, int total, int ls,
+                                          const FxTw* __restrict__ tw, const FxBlock& S, const unsigned* before,
+                                          unsigned* after) {
   const int Ns = 1 << ls, quarter = 1 << (a2 - 2);
   const int s1 = fx_slot(Ns), s2 = fx_slot(2 * Ns);
   const int r1 = fx_slot(quarter), r2 = fx_slot(2 * quarter);
-  unsigned span = 0;
+  // lanes that share a sequence: all, or groups of N / 4
+  const unsigned lanes = quarter >= 32 ? NS_FULL_MASK : ((1u << quarter) - 1) << (threadIdx.x & 31 & -quarter);
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
     const int sq = idx >> (a2 - 2);
     const int j = idx & (quarter - 1);
@@ -257,10 +279,12 @@ __device__ __forceinline__ unsigned fx_stage4(const Fx2* A, Fx2* B, int a2, int 
       x[2] = A[base + (q ^ r2)];
       x[3] = A[base + (q ^ r1 ^ r2)];
       if (TW) {
-        const FxTw* w = tw + 3 * (Ns + k);
-        x[0] = fx_shr(x[0], SH);
-#pragma unroll
-        for (int r = 1; r < 4; ++r) x[r] = fx_cmul<SIGN>(x[r], fx_ldtw(w + r - 1), SH);
+        const FxTw* t = tw + 3 * (Ns + k);
+        const FxTw w[3] = {fx_ldtw(t), fx_ldtw(t + 1), fx_ldtw(t + 2)};
+        const int sh = fx_stage_shift(before[sq]);  // one for the lanes of a sequence
+        if (sh == 1) fx_twiddle4<SIGN, 1>(x, w);
+        else if (sh == 2) fx_twiddle4<SIGN, 2>(x, w);
+        else fx_twiddle4<SIGN, 0>(x, w);
       }
     }
     fx_bfly4<SIGN>(x[0], x[1], x[2], x[3], y);
@@ -269,38 +293,47 @@ __device__ __forceinline__ unsigned fx_stage4(const Fx2* A, Fx2* B, int a2, int 
     B[base + (o ^ s1)] = y[1];
     B[base + (o ^ s2)] = y[2];
     B[base + (o ^ s1 ^ s2)] = y[3];
-    span |= fx_span(y[0]) | fx_span(y[1]) | fx_span(y[2]) | fx_span(y[3]);
+    fx_gather_span(fx_span(y[0]) | fx_span(y[1]) | fx_span(y[2]) | fx_span(y[3]), lanes, after + sq);
   }
-  return span;
 }
 
 // FIRST: A holds doubles at [seq * ld + i], converted by the first stage; else fixed point at
-// [seq * ld + fx_slot(i)], at most 2^59.5 in modulus.  tw[3 (Ns + k) + r - 1]: the twiddle of input
-// r of a stage that follows sub-transforms of length Ns.  Returns the buffer of the result (fixed
-// point, slots) and adds to t: bit 62 of a result of sequence q stands for exponent(q) + t.
+// [seq * ld + fx_slot(i)], at most 2^59.5 in modulus, bit 62 standing for exponent + t0.
+// tw[3 (Ns + k) + r - 1]: the twiddle of input r of a stage that follows sub-transforms of length Ns.
+// Returns the buffer of the result (fixed point, slots): bit 62 of a result of sequence q stands for
+// exponent(q) + S.t[q].
 template <int SIGN, bool FIRST>
 __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, const FxTw* __restrict__ tw,
-                            FxBlock& S, int& t) {
+                            FxBlock& S, int t0 = 0) {
   const int a2 = plan & 0xff, b3 = plan >> 8;
   const bool p2 = b3 == 0;  // N a power of two: index arithmetic by shifts
+  const int tid = threadIdx.x;
   int stage = 0;
-  auto close = [&](unsigned span) {  // end of a stage
-    span = __reduce_or_sync(NS_FULL_MASK, span);
-    if ((threadIdx.x & 31) == 0) atomicOr(&S.span[stage], span);
+  auto close = [&]() {  // end of a stage
     __syncthreads();
     Fx2* x = A;
     A = B;
     B = x;
     ++stage;
   };
+  // a stage's `total` butterflies where the lanes of a warp may work on any sequences: body(idx, span)
+  // returns the sequence
+  auto each = [&](int total, auto body) {
+    for (int base = tid & ~31; base < total; base += blockDim.x) {
+      const int idx = base + (tid & 31);
+      unsigned span = 0;
+      const int sq = idx < total ? body(idx, span) : nseq;
+      const unsigned lanes = __match_any_sync(NS_FULL_MASK, sq);
+      if (sq < nseq) fx_gather_span(span, lanes, &S.span[stage][sq]);
+    }
+  };
+  auto shift = [&](int sq) { return fx_stage_shift(S.span[stage - 1][sq]); };
   int Ns = 1;
   bool first = true;  // the stage with Ns = 1, which has no twiddles
   if (a2 & 1) {
-    if (FIRST) t += 3;
     const int half = N >> 1;
-    const int total = nseq * half;
-    unsigned span = 0;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    if (tid < nseq) S.t[tid] = FIRST ? 3 : t0;
+    each(nseq * half, [&](int idx, unsigned& span) {
       const int sq = p2 ? idx >> (a2 - 1) : idx / half;
       const int j = idx - sq * half;
       Fx2 x[2];
@@ -316,9 +349,10 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
       const Fx2 y0 = fx_add(x[0], x[1]), y1 = fx_sub(x[0], x[1]);
       B[sq * ld + fx_slot(2 * j)] = y0;
       B[sq * ld + fx_slot(2 * j + 1)] = y1;
-      span |= fx_span(y0) | fx_span(y1);
-    }
-    close(span);
+      span = fx_span(y0) | fx_span(y1);
+      return sq;
+    });
+    close();
     Ns = 2;
     first = false;
   }
@@ -326,19 +360,17 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
   for (int st = 0; st < (a2 >> 1); ++st, Ns <<= 2) {
     const int ls = __ffs(Ns) - 1;  // Ns is a power of two in the radix-4 stages
     const int total = nseq * quarter;
-    unsigned span = 0;
-    const int sh = first ? 0 : fx_stage_shift(S.span[stage - 1]);
-    t += (FIRST && first) ? 4 : sh;
+    if (tid < nseq) S.t[tid] = first ? (FIRST ? 4 : t0) : S.t[tid] + shift(tid);
     if (p2) {
-      span = first     ? fx_stage4<SIGN, FIRST, false, 0>(A, B, a2, ld, total, ls, tw, S)
-             : sh == 1 ? fx_stage4<SIGN, false, true, 1>(A, B, a2, ld, total, ls, tw, S)
-             : sh == 2 ? fx_stage4<SIGN, false, true, 2>(A, B, a2, ld, total, ls, tw, S)
-                       : fx_stage4<SIGN, false, true, 0>(A, B, a2, ld, total, ls, tw, S);
-      close(span);
+      if (first)
+        fx_stage4<SIGN, FIRST, false>(A, B, a2, ld, total, ls, tw, S, nullptr, S.span[stage]);
+      else
+        fx_stage4<SIGN, false, true>(A, B, a2, ld, total, ls, tw, S, S.span[stage - 1], S.span[stage]);
+      close();
       first = false;
       continue;
     }
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    each(total, [&](int idx, unsigned& span) {
       const int sq = idx / quarter;
       const int j = idx - sq * quarter;
       const int k = j & (Ns - 1);
@@ -355,6 +387,7 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
 #pragma unroll
         for (int r = 0; r < 4; ++r) x[r] = A[sq * ld + fx_slot(j + r * quarter)];
         if (!first) {
+          const int sh = shift(sq);
           x[0] = fx_shr(x[0], sh);
 #pragma unroll
           for (int r = 1; r < 4; ++r) x[r] = fx_cmul<SIGN>(x[r], fx_ldtw(tw + 3 * (Ns + k) + r - 1), sh);
@@ -367,21 +400,20 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
         B[sq * ld + fx_slot(o + r * Ns)] = y[r];
         span |= fx_span(y[r]);
       }
-    }
-    close(span);
+      return sq;
+    });
+    close();
     first = false;
   }
   const int third = N / 3;
   for (int st = 0; st < b3; ++st, Ns *= 3) {
-    const int total = nseq * third;
-    unsigned span = 0;
-    const int sh = fx_stage_shift(S.span[stage - 1]);
-    t += sh;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    if (tid < nseq) S.t[tid] += shift(tid);
+    each(nseq * third, [&](int idx, unsigned& span) {
       const int sq = idx / third;
       const int j = idx - sq * third;
       const int g = j / Ns;
       const int k = j - g * Ns;
+      const int sh = shift(sq);
       Fx2 x[3], y[3];
       x[0] = fx_shr(A[sq * ld + fx_slot(j)], sh);
 #pragma unroll
@@ -393,8 +425,9 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
         B[sq * ld + fx_slot(g * 3 * Ns + k + r * Ns)] = y[r];
         span |= fx_span(y[r]);
       }
-    }
-    close(span);
+      return sq;
+    });
+    close();
   }
   return A;
 }
@@ -559,13 +592,12 @@ struct DivzK {
   // unpack the two real transforms of each packed pair; write kz = 0..nz/2
   const int nh = (nz >> 1) + 1;
   if (fx_loaded(S, nseq)) {
-    int t = 0;
-    const Fx2* R = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, pz, nseq, twz, S, t);
+    const Fx2* R = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, pz, nseq, twz, S);
     for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
       const int il = q & (TX - 1);
       const int m = q >> lt;
       const int c = il >> 1;
-      const int e = fx_exponent(S.emax[c]) + t;
+      const int e = fx_exponent(S.emax[c]) + S.t[c];
       const Fx2 zm = R[c * ld + fx_slot(m)];
       const Fx2 zn = R[c * ld + fx_slot(m == 0 ? 0 : nz - m)];
       spec[((long)m * ny + j) * nx + i0 + il] = (il & 1) == 0 ? make_double2(fx_to(zm.x + zn.x, e), fx_to(zm.y - zn.y, e))
@@ -615,12 +647,11 @@ struct FftxK {
     fx_load_rows(R, nx, a.px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                  [&](int r, int i, double2 v) { A[r * ld + i] = v; });
     if (fx_loaded(S, R)) {
-      int t = 0;
       const Fx2* X = fx_stockham<SIGN, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nx, ld, a.px, R,
-                                             a.twx, S, t);
+                                             a.twx, S);
       for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
         const int r = fx_row(q, nx, a.px), i = q - r * nx;
-        const double e = fx_unit(fx_exponent(S.emax[r]) + t);
+        const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r]);
         const Fx2 v = X[r * ld + fx_slot(i)];
         g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
       }
@@ -950,14 +981,13 @@ struct IfftzK {
     fx_gather_max(mag, nseq, &S.emax[threadIdx.x & (nseq - 1)]);
     const long pl = (long)ny * nx;
     if (fx_loaded(S, nseq)) {
-      int t = 0;
       const Fx2* R = fx_stockham<1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, a.pz, nseq,
-                                          a.twz, S, t);
+                                          a.twz, S);
       for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
         const int il = q & (TX - 1);
         const int k = q >> lt;
         const Fx2 v = R[(il >> 1) * ld + fx_slot(k)];
-        a.phi[k * pl + (long)j * nx + i0 + il] = fx_double((il & 1) ? v.y : v.x) * fx_unit(fx_exponent(S.emax[il >> 1]) + t);
+        a.phi[k * pl + (long)j * nx + i0 + il] = fx_double((il & 1) ? v.y : v.x) * fx_unit(fx_exponent(S.emax[il >> 1]) + S.t[il >> 1]);
       }
       return;
     }
@@ -1680,16 +1710,16 @@ __global__ void __launch_bounds__(256, 4) dctx_fwd_kernel(double2* __restrict__ 
   fx_load_rows(R, nx, px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                [&](int r, int i, double2 v) { A[r * ld + ((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))] = v; });
   if (fx_loaded(S, R)) {
-    int t = 0;
-    const Fx2* V = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nx, ld, px, R, twx, S, t);
+    const Fx2* V = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nx, ld, px, R, twx, S);
     // a, b = (V_l +- conj V_{N-l}) / 2 (b over i), times w_l
-    const int sh = fx_stage_shift(S.span[fx_stages(px) - 1]);
+    const unsigned* span = S.span[fx_stages(px) - 1];
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
       const int r = fx_row(q, nx, px), l = q - r * nx;
       const Fx2 vl = fx_shr(V[r * ld + fx_slot(l)], 1);
       const Fx2 vn = fx_shr(V[r * ld + fx_slot(l == 0 ? 0 : nx - l)], 1);
       const FxTw w = fx_ldtw(twd + l);
-      const double e = fx_unit(fx_exponent(S.emax[r]) + t + sh);
+      const int sh = fx_stage_shift(span[r]);
+      const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r] + sh);
       const Fx2 xa = fx_cmul<-1>(Fx2{vl.x + vn.x, vl.y - vn.y}, w, sh);
       const Fx2 xb = fx_cmul<-1>(Fx2{vl.y + vn.y, vn.x - vl.x}, w, sh);
       g[q] = make_double2(fx_double(xa.x) * e, fx_double(xb.x) * e);
@@ -1740,11 +1770,10 @@ __global__ void __launch_bounds__(256, 4) dctx_inv_kernel(double2* __restrict__ 
   }
   __syncthreads();
   if (ok) {
-    int t = 5;
-    const Fx2* X = fx_stockham<1, false>(reinterpret_cast<Fx2*>(B), reinterpret_cast<Fx2*>(A), nx, ld, px, R, twx, S, t);
+    const Fx2* X = fx_stockham<1, false>(reinterpret_cast<Fx2*>(B), reinterpret_cast<Fx2*>(A), nx, ld, px, R, twx, S, 5);
     for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
       const int r = fx_row(q, nx, px), i = q - r * nx;
-      const double e = fx_unit(fx_exponent(S.emax[r]) + t);
+      const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r]);
       const Fx2 v = X[r * ld + fx_slot((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))];
       g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
     }
