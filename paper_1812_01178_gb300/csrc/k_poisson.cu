@@ -175,22 +175,22 @@ __device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, con
 // on the integer pipes (fx64.cuh).  In FP64 arithmetic they ran at 0.86-0.9 of the FP64 pipe's rate
 // (22 instructions of 16 cycles a warp per radix-4 butterfly); in fixed point a butterfly is 36
 // multiply-adds of about 1.3 cycles and some 100 additions, shifts and logic operations on the
-// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 220 (six FP64
-// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 123, inverse z 295 -> 136.
+// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 218 (six FP64
+// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 125, inverse z 295 -> 137.
 // Results go back to FP64 by two exact FP64 instructions and a scaling on the otherwise idle pipe (x,
 // inverse z), or by integer steps (after the divergence, which uses that pipe).
 //
 // Every sequence is scaled by its own largest component, and before each stage shifted by 0, 1 or 2 bits,
 // as its own largest value (the or of its magnitudes, gathered while the last stage was written) needs for
 // the next sums to stay below 2^62.  (One shift for all sequences of a block took 583 us for the four
-// transforms, 602 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
+// transforms, 604 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
 // 1024 where FP64 butterflies leave 1.6e-16.)  A sequence's relative error in the 2-norm is then 4e-17 to
 // 1e-16, against 1.1e-16 to 7e-16 with FP64 butterflies, on noise, smooth and decaying data, pulses and steps of 24
 // to 4096 points.  It is one of the whole sequence: of the two real columns that a z sequence packs, one whose sum
 // grows lets the other lose digits (a pulse beside a constant: below FP64's 1.5e-16 up to 256 points, 1.9e-16 at 512,
 // 5e-16 at 1024, 1.5e-15 at 4096), where FP64 butterflies lose them only to a larger column (of 1000 times
 // the size: 3e-13 against 3e-14 here).  Sequences that hold an infinity, a NaN or values near the ends of the
-// binary64 range take FP64 butterflies (plain_stockham).
+// binary64 range take FP64 butterflies (plain_stockham), and leave the others of their block as they are.
 //
 // Sequences stand in shared memory with a pitch of N + 1 elements of 16 bytes (columns of one row
 // fall into different banks) and, in fixed point, element i at fx_slot(i): the stages' writes at
@@ -223,13 +223,13 @@ __device__ __forceinline__ void fx_begin(FxBlock& S) {
   if (threadIdx.x < FX_STAGES * FX_SEQ) (&S.span[0][0])[threadIdx.x] = 0;
   __syncthreads();
 }
-// The barrier after the loads: whether every sequence's exponent suits the fixed-point path
-__device__ __forceinline__ bool fx_loaded(const FxBlock& S, int nseq) {
+// The barrier after the loads: the sequences whose exponents suit the fixed-point path, a bit each
+__device__ __forceinline__ unsigned fx_loaded(const FxBlock& S, int nseq) {
   __syncthreads();
-  bool ok = true;
-  for (int q = 0; q < nseq; ++q) ok = ok && fx_exponent_ok(fx_exponent(S.emax[q]));
-  return ok;
+  const int q = threadIdx.x & 31;
+  return __ballot_sync(NS_FULL_MASK, q < nseq && fx_exponent_ok(fx_exponent(S.emax[q & (FX_SEQ - 1)])));
 }
+__device__ __forceinline__ bool fx_all(unsigned ok, int nseq) { return ok + 1 == 1u << nseq; }
 
 // `span` of the lanes of a warp that work on sequence sq joins *slot; `lanes`: those lanes
 __device__ __forceinline__ void fx_gather_span(unsigned span, unsigned lanes, unsigned* slot) {
@@ -251,7 +251,7 @@ __device__ __forceinline__ void fx_twiddle4(Fx2 (&x)[4], const FxTw (&w)[3]) {
 // doubles; TW: twiddles.  before: the spans the sequences' shifts follow from, after: those of the results.
 template <int SIGN, bool RAW, bool TW>
 __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, int total, int ls,
-                                          const FxTw* __restrict__ tw, const FxBlock& S, const unsigned* before,
+                                          const FxTw* __restrict__ tw, const unsigned* emax, const unsigned* before,
                                           unsigned* after) {
   const int Ns = 1 << ls, quarter = 1 << (a2 - 2);
   const int s1 = fx_slot(Ns), s2 = fx_slot(2 * Ns);
@@ -265,7 +265,7 @@ __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, 
     const int base = sq * ld;
     Fx2 x[4], y[4];
     if (RAW) {
-      const int s = fx_exponent(S.emax[sq]) + 4;
+      const int s = fx_exponent(emax[sq]) + 4;
       const double2* X = reinterpret_cast<const double2*>(A) + base + j;
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
@@ -301,10 +301,10 @@ __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, 
 // [seq * ld + fx_slot(i)], at most 2^59.5 in modulus, bit 62 standing for exponent + t0.
 // tw[3 (Ns + k) + r - 1]: the twiddle of input r of a stage that follows sub-transforms of length Ns.
 // Returns the buffer of the result (fixed point, slots): bit 62 of a result of sequence q stands for
-// exponent(q) + S.t[q].
+// exponent(q) + S.t[q].  q0: the number in S of the first sequence.
 template <int SIGN, bool FIRST>
-__device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, const FxTw* __restrict__ tw,
-                            FxBlock& S, int t0 = 0) {
+__device__ __forceinline__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq,
+                                            const FxTw* __restrict__ tw, FxBlock& S, int t0 = 0, int q0 = 0) {
   const int a2 = plan & 0xff, b3 = plan >> 8;
   const bool p2 = b3 == 0;  // N a power of two: index arithmetic by shifts
   const int tid = threadIdx.x;
@@ -324,21 +324,21 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
       unsigned span = 0;
       const int sq = idx < total ? body(idx, span) : nseq;
       const unsigned lanes = __match_any_sync(NS_FULL_MASK, sq);
-      if (sq < nseq) fx_gather_span(span, lanes, &S.span[stage][sq]);
+      if (sq < nseq) fx_gather_span(span, lanes, &S.span[stage][q0 + sq]);
     }
   };
-  auto shift = [&](int sq) { return fx_stage_shift(S.span[stage - 1][sq]); };
+  auto shift = [&](int sq) { return fx_stage_shift(S.span[stage - 1][q0 + sq]); };
   int Ns = 1;
   bool first = true;  // the stage with Ns = 1, which has no twiddles
   if (a2 & 1) {
     const int half = N >> 1;
-    if (tid < nseq) S.t[tid] = FIRST ? 3 : t0;
+    if (tid < nseq) S.t[q0 + tid] = FIRST ? 3 : t0;
     each(nseq * half, [&](int idx, unsigned& span) {
       const int sq = p2 ? idx >> (a2 - 1) : idx / half;
       const int j = idx - sq * half;
       Fx2 x[2];
       if (FIRST) {
-        const int s = fx_exponent(S.emax[sq]) + 3;
+        const int s = fx_exponent(S.emax[q0 + sq]) + 3;
         const double2* X = reinterpret_cast<const double2*>(A) + sq * ld + j;
 #pragma unroll
         for (int r = 0; r < 2; ++r) x[r] = Fx2{fx_from(X[r * half].x, s), fx_from(X[r * half].y, s)};
@@ -360,12 +360,12 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
   for (int st = 0; st < (a2 >> 1); ++st, Ns <<= 2) {
     const int ls = __ffs(Ns) - 1;  // Ns is a power of two in the radix-4 stages
     const int total = nseq * quarter;
-    if (tid < nseq) S.t[tid] = first ? (FIRST ? 4 : t0) : S.t[tid] + shift(tid);
+    if (tid < nseq) S.t[q0 + tid] = first ? (FIRST ? 4 : t0) : S.t[q0 + tid] + shift(tid);
     if (p2) {
       if (first)
-        fx_stage4<SIGN, FIRST, false>(A, B, a2, ld, total, ls, tw, S, nullptr, S.span[stage]);
+        fx_stage4<SIGN, FIRST, false>(A, B, a2, ld, total, ls, tw, S.emax + q0, nullptr, S.span[stage] + q0);
       else
-        fx_stage4<SIGN, false, true>(A, B, a2, ld, total, ls, tw, S, S.span[stage - 1], S.span[stage]);
+        fx_stage4<SIGN, false, true>(A, B, a2, ld, total, ls, tw, S.emax + q0, S.span[stage - 1] + q0, S.span[stage] + q0);
       close();
       first = false;
       continue;
@@ -376,7 +376,7 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
       const int k = j & (Ns - 1);
       Fx2 x[4], y[4];
       if (FIRST && first) {
-        const int s = fx_exponent(S.emax[sq]) + 4;
+        const int s = fx_exponent(S.emax[q0 + sq]) + 4;
         const double2* X = reinterpret_cast<const double2*>(A) + sq * ld + j;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -407,7 +407,7 @@ __device__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq, c
   }
   const int third = N / 3;
   for (int st = 0; st < b3; ++st, Ns *= 3) {
-    if (tid < nseq) S.t[tid] += shift(tid);
+    if (tid < nseq) S.t[q0 + tid] += shift(tid);
     each(nseq * third, [&](int idx, unsigned& span) {
       const int sq = idx / third;
       const int j = idx - sq * third;
@@ -489,6 +489,21 @@ __device__ __noinline__ double2* plain_stockham(double2* A, double2* B, int N, i
   return A;
 }
 
+// A block of sequences, ok: those that suit the fixed-point path (fx_loaded).  Where some do not, each is
+// transformed alone, so that one with an infinity or a NaN leaves the others as they are.  Returns the buffer
+// of the results, fixed point (as fx_stockham) or FP64 by the sequence's bit.
+template <int SIGN, bool FIRST>
+__device__ __noinline__ Fx2* fx_each_alone(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq,
+                                           const FxTw* __restrict__ tw, FxBlock& S, int t0, unsigned ok) {
+  Fx2* r = A;
+  for (int q = 0; q < nseq; ++q, A += ld, B += ld) {
+    Fx2* const x = ok >> q & 1 ? fx_stockham<SIGN, FIRST>(A, B, N, ld, plan, 1, tw, S, t0, q)
+                               : reinterpret_cast<Fx2*>(plain_stockham<SIGN>(reinterpret_cast<double2*>(A),
+                                                                             reinterpret_cast<double2*>(B), N, ld, plan, 1, tw));
+    if (q == 0) r = x;
+  }
+  return r;
+}
 // q / N: a shift for powers of two
 __device__ __forceinline__ int fx_row(int q, int N, int plan) { return (plan >> 8) == 0 ? q >> (plan & 0xff) : q / N; }
 // max over the lanes of a warp that share lane mod n (n a power of two), then over warps into *slot
@@ -591,30 +606,34 @@ struct DivzK {
   fx_gather_max(mag, TX, &S.emax[(threadIdx.x & (TX - 1)) >> 1]);
   // unpack the two real transforms of each packed pair; write kz = 0..nz/2
   const int nh = (nz >> 1) + 1;
-  if (fx_loaded(S, nseq)) {
-    const Fx2* R = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, pz, nseq, twz, S);
-    for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
-      const int il = q & (TX - 1);
-      const int m = q >> lt;
-      const int c = il >> 1;
-      const int e = fx_exponent(S.emax[c]) + S.t[c];
-      const Fx2 zm = R[c * ld + fx_slot(m)];
-      const Fx2 zn = R[c * ld + fx_slot(m == 0 ? 0 : nz - m)];
-      spec[((long)m * ny + j) * nx + i0 + il] = (il & 1) == 0 ? make_double2(fx_to(zm.x + zn.x, e), fx_to(zm.y - zn.y, e))
-                                                              : make_double2(fx_to(zm.y + zn.y, e), fx_to(zn.x - zm.x, e));
-    }
-    return;
-  }
-  const double2* R = plain_stockham<-1>(A, B, nz, ld, pz, nseq, twz);
-  for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) {
+  const unsigned ok = fx_loaded(S, nseq);
+  auto put = [&](const Fx2* R, int q, bool fixed) {
     const int il = q & (TX - 1);
     const int m = q >> lt;
     const int c = il >> 1;
-    const double2 zm = R[c * ld + m];
-    const double2 zn = R[c * ld + (m == 0 ? 0 : nz - m)];
-    spec[((long)m * ny + j) * nx + i0 + il] = (il & 1) == 0 ? make_double2(zm.x + zn.x, zm.y - zn.y)
-                                                            : make_double2(zm.y + zn.y, zn.x - zm.x);
+    const int n = m == 0 ? 0 : nz - m;
+    double2 x;
+    if (fixed) {
+      const int e = fx_exponent(S.emax[c]) + S.t[c];
+      const Fx2 zm = R[c * ld + fx_slot(m)];
+      const Fx2 zn = R[c * ld + fx_slot(n)];
+      x = (il & 1) == 0 ? make_double2(fx_to(zm.x + zn.x, e), fx_to(zm.y - zn.y, e))
+                        : make_double2(fx_to(zm.y + zn.y, e), fx_to(zn.x - zm.x, e));
+    } else {
+      const double2 zm = reinterpret_cast<const double2*>(R)[c * ld + m];
+      const double2 zn = reinterpret_cast<const double2*>(R)[c * ld + n];
+      x = (il & 1) == 0 ? make_double2(zm.x + zn.x, zm.y - zn.y) : make_double2(zm.y + zn.y, zn.x - zm.x);
+    }
+    spec[((long)m * ny + j) * nx + i0 + il] = x;
+  };
+  Fx2 *fa = reinterpret_cast<Fx2*>(A), *fb = reinterpret_cast<Fx2*>(B);
+  if (!fx_all(ok, nseq)) {
+    const Fx2* R = fx_each_alone<-1, true>(fa, fb, nz, ld, pz, nseq, twz, S, 0, ok);
+    for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) put(R, q, ok >> ((q & (TX - 1)) >> 1) & 1);
+    return;
   }
+  const Fx2* R = fx_stockham<-1, true>(fa, fb, nz, ld, pz, nseq, twz, S);
+  for (int q = threadIdx.x; q < nh * TX; q += blockDim.x) put(R, q, true);
 
   }
 };
@@ -646,22 +665,28 @@ struct FftxK {
     fx_begin(S);
     fx_load_rows(R, nx, a.px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                  [&](int r, int i, double2 v) { A[r * ld + i] = v; });
-    if (fx_loaded(S, R)) {
-      const Fx2* X = fx_stockham<SIGN, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nx, ld, a.px, R,
-                                             a.twx, S);
-      for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-        const int r = fx_row(q, nx, a.px), i = q - r * nx;
+    const unsigned ok = fx_loaded(S, R);
+    auto put = [&](const Fx2* X, int q, int r, bool fixed) {
+      const int i = q - r * nx;
+      if (fixed) {
         const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r]);
         const Fx2 v = X[r * ld + fx_slot(i)];
         g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
+      } else {
+        g[q] = reinterpret_cast<const double2*>(X)[r * ld + i];
+      }
+    };
+    Fx2 *fa = reinterpret_cast<Fx2*>(A), *fb = reinterpret_cast<Fx2*>(B);
+    if (!fx_all(ok, R)) {
+      const Fx2* X = fx_each_alone<SIGN, true>(fa, fb, nx, ld, a.px, R, a.twx, S, 0, ok);
+      for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
+        const int r = fx_row(q, nx, a.px);
+        put(X, q, r, ok >> r & 1);
       }
       return;
     }
-    const double2* X = plain_stockham<SIGN>(A, B, nx, ld, a.px, R, a.twx);
-    for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-      const int r = fx_row(q, nx, a.px), i = q - r * nx;
-      g[q] = X[r * ld + i];
-    }
+    const Fx2* X = fx_stockham<SIGN, true>(fa, fb, nx, ld, a.px, R, a.twx, S);
+    for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) put(X, q, fx_row(q, nx, a.px), true);
   }
 };
 
@@ -980,24 +1005,28 @@ struct IfftzK {
     }
     fx_gather_max(mag, nseq, &S.emax[threadIdx.x & (nseq - 1)]);
     const long pl = (long)ny * nx;
-    if (fx_loaded(S, nseq)) {
-      const Fx2* R = fx_stockham<1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nz, ld, a.pz, nseq,
-                                          a.twz, S);
-      for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
-        const int il = q & (TX - 1);
-        const int k = q >> lt;
-        const Fx2 v = R[(il >> 1) * ld + fx_slot(k)];
-        a.phi[k * pl + (long)j * nx + i0 + il] = fx_double((il & 1) ? v.y : v.x) * fx_unit(fx_exponent(S.emax[il >> 1]) + S.t[il >> 1]);
-      }
-      return;
-    }
-    const double2* R = plain_stockham<1>(A, B, nz, ld, a.pz, nseq, a.twz);
-    for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) {
+    const unsigned ok = fx_loaded(S, nseq);
+    auto put = [&](const Fx2* R, int q, bool fixed) {
       const int il = q & (TX - 1);
       const int k = q >> lt;
-      const double2 v = R[(il >> 1) * ld + k];
-      a.phi[k * pl + (long)j * nx + i0 + il] = (il & 1) ? v.y : v.x;
+      const int c = il >> 1;
+      double* phi = a.phi + k * pl + (long)j * nx + i0 + il;
+      if (fixed) {
+        const Fx2 v = R[c * ld + fx_slot(k)];
+        *phi = fx_double((il & 1) ? v.y : v.x) * fx_unit(fx_exponent(S.emax[c]) + S.t[c]);
+      } else {
+        const double2 v = reinterpret_cast<const double2*>(R)[c * ld + k];
+        *phi = (il & 1) ? v.y : v.x;
+      }
+    };
+    Fx2 *fa = reinterpret_cast<Fx2*>(A), *fb = reinterpret_cast<Fx2*>(B);
+    if (!fx_all(ok, nseq)) {
+      const Fx2* R = fx_each_alone<1, true>(fa, fb, nz, ld, a.pz, nseq, a.twz, S, 0, ok);
+      for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) put(R, q, ok >> ((q & (TX - 1)) >> 1) & 1);
+      return;
     }
+    const Fx2* R = fx_stockham<1, true>(fa, fb, nz, ld, a.pz, nseq, a.twz, S);
+    for (int q = threadIdx.x; q < TX * nz; q += blockDim.x) put(R, q, true);
   }
 };
 
@@ -1709,32 +1738,39 @@ __global__ void __launch_bounds__(256, 4) dctx_fwd_kernel(double2* __restrict__ 
   fx_begin(S);
   fx_load_rows(R, nx, px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                [&](int r, int i, double2 v) { A[r * ld + ((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))] = v; });
-  if (fx_loaded(S, R)) {
-    const Fx2* V = fx_stockham<-1, true>(reinterpret_cast<Fx2*>(A), reinterpret_cast<Fx2*>(B), nx, ld, px, R, twx, S);
-    // a, b = (V_l +- conj V_{N-l}) / 2 (b over i), times w_l
-    const unsigned* span = S.span[fx_stages(px) - 1];
-    for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-      const int r = fx_row(q, nx, px), l = q - r * nx;
+  const unsigned ok = fx_loaded(S, R);
+  // a, b = (V_l +- conj V_{N-l}) / 2 (b over i), times w_l
+  const unsigned* span = S.span[fx_stages(px) - 1];
+  auto put = [&](const Fx2* V, int q, int r, bool fixed) {
+    const int l = q - r * nx, n = l == 0 ? 0 : nx - l;
+    const FxTw w = fx_ldtw(twd + l);
+    if (fixed) {
       const Fx2 vl = fx_shr(V[r * ld + fx_slot(l)], 1);
-      const Fx2 vn = fx_shr(V[r * ld + fx_slot(l == 0 ? 0 : nx - l)], 1);
-      const FxTw w = fx_ldtw(twd + l);
+      const Fx2 vn = fx_shr(V[r * ld + fx_slot(n)], 1);
       const int sh = fx_stage_shift(span[r]);
       const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r] + sh);
       const Fx2 xa = fx_cmul<-1>(Fx2{vl.x + vn.x, vl.y - vn.y}, w, sh);
       const Fx2 xb = fx_cmul<-1>(Fx2{vl.y + vn.y, vn.x - vl.x}, w, sh);
       g[q] = make_double2(fx_double(xa.x) * e, fx_double(xb.x) * e);
+    } else {
+      const double2 vl = reinterpret_cast<const double2*>(V)[r * ld + l];
+      const double2 vn = reinterpret_cast<const double2*>(V)[r * ld + n];
+      const double2 d = fx_twd(w);
+      const double c = 0.5 * d.x, s = 0.5 * d.y;
+      g[q] = make_double2(c * (vl.x + vn.x) + s * (vl.y - vn.y), c * (vl.y + vn.y) + s * (vn.x - vl.x));
+    }
+  };
+  Fx2 *fa = reinterpret_cast<Fx2*>(A), *fb = reinterpret_cast<Fx2*>(B);
+  if (!fx_all(ok, R)) {
+    const Fx2* V = fx_each_alone<-1, true>(fa, fb, nx, ld, px, R, twx, S, 0, ok);
+    for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
+      const int r = fx_row(q, nx, px);
+      put(V, q, r, ok >> r & 1);
     }
     return;
   }
-  const double2* V = plain_stockham<-1>(A, B, nx, ld, px, R, twx);
-  for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-    const int r = fx_row(q, nx, px), l = q - r * nx;
-    const double2 vl = V[r * ld + l];
-    const double2 vn = V[r * ld + (l == 0 ? 0 : nx - l)];
-    const double2 w = fx_twd(fx_ldtw(twd + l));
-    const double c = 0.5 * w.x, s = 0.5 * w.y;
-    g[q] = make_double2(c * (vl.x + vn.x) + s * (vl.y - vn.y), c * (vl.y + vn.y) + s * (vn.x - vl.x));
-  }
+  const Fx2* V = fx_stockham<-1, true>(fa, fb, nx, ld, px, R, twx, S);
+  for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) put(V, q, fx_row(q, nx, px), true);
 }
 
 __global__ void __launch_bounds__(256, 4) dctx_inv_kernel(double2* __restrict__ spec, const FxTw* __restrict__ twx,
@@ -1751,14 +1787,15 @@ __global__ void __launch_bounds__(256, 4) dctx_inv_kernel(double2* __restrict__ 
   fx_begin(S);
   fx_load_rows(R, nx, px, S, [&](int r, int i) { return r < nr ? g[r * nx + i] : make_double2(0.0, 0.0); },
                [&](int r, int i, double2 v) { A[r * ld + i] = v; });
-  const bool ok = fx_loaded(S, R);
+  const unsigned ok = fx_loaded(S, R);
+  const bool all = fx_all(ok, R);
   // V_l = conj(w_l) (X_l - i X_{N-l})
   for (int q = threadIdx.x; q < R * nx; q += blockDim.x) {
     const int r = fx_row(q, nx, px), l = q - r * nx;
     const double2 xl = A[r * ld + l];
     const double2 xn = l == 0 ? make_double2(0.0, 0.0) : A[r * ld + nx - l];
     const FxTw w = fx_ldtw(twd + l);
-    if (ok) {
+    if (all || (ok >> r & 1)) {
       const int s = fx_exponent(S.emax[r]) + 3;
       reinterpret_cast<Fx2*>(B)[r * ld + fx_slot(l)] =
           fx_cmul<1>(Fx2{fx_from(xl.x, s) + fx_from(xn.y, s), fx_from(xl.y, s) - fx_from(xn.x, s)}, w, 2);
@@ -1769,21 +1806,27 @@ __global__ void __launch_bounds__(256, 4) dctx_inv_kernel(double2* __restrict__ 
     }
   }
   __syncthreads();
-  if (ok) {
-    const Fx2* X = fx_stockham<1, false>(reinterpret_cast<Fx2*>(B), reinterpret_cast<Fx2*>(A), nx, ld, px, R, twx, S, 5);
-    for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-      const int r = fx_row(q, nx, px), i = q - r * nx;
+  auto put = [&](const Fx2* X, int q, int r, bool fixed) {
+    const int i = q - r * nx, l = (i & 1) ? nx - 1 - (i >> 1) : (i >> 1);
+    if (fixed) {
       const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r]);
-      const Fx2 v = X[r * ld + fx_slot((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))];
+      const Fx2 v = X[r * ld + fx_slot(l)];
       g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
+    } else {
+      g[q] = reinterpret_cast<const double2*>(X)[r * ld + l];
+    }
+  };
+  Fx2 *fa = reinterpret_cast<Fx2*>(A), *fb = reinterpret_cast<Fx2*>(B);
+  if (!all) {
+    const Fx2* X = fx_each_alone<1, false>(fb, fa, nx, ld, px, R, twx, S, 5, ok);
+    for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
+      const int r = fx_row(q, nx, px);
+      put(X, q, r, ok >> r & 1);
     }
     return;
   }
-  const double2* X = plain_stockham<1>(B, A, nx, ld, px, R, twx);
-  for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) {
-    const int r = fx_row(q, nx, px), i = q - r * nx;
-    g[q] = X[r * ld + ((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))];
-  }
+  const Fx2* X = fx_stockham<1, false>(fb, fa, nx, ld, px, R, twx, S, 5);
+  for (int q = threadIdx.x; q < nr * nx; q += blockDim.x) put(X, q, fx_row(q, nx, px), true);
 }
 
 // The FP32 form (mixed precision)

@@ -19,16 +19,17 @@ SOURCE = r"""
 #include "k_poisson.cu"
 #include <cstdio>
 #include <cstdlib>
-// rows of n doubles pairs from a file -> their transform (sign) in another, R rows a block
+// rows of n pairs of doubles from a file -> their transform (sign; Fourier or cosine) in another, R rows a block
 int main(int argc, char** argv) {
-  const int n = atoi(argv[3]), R = atoi(argv[4]), rows = atoi(argv[5]), sign = atoi(argv[6]);
+  const int n = atoi(argv[3]), R = atoi(argv[4]), rows = atoi(argv[5]), sign = atoi(argv[6]), cosine = atoi(argv[7]);
   const size_t bytes = (size_t)rows * n * sizeof(double2);
   std::vector<char> h(bytes);
   FILE* f = fopen(argv[1], "rb");
   if (!f || fread(h.data(), 1, bytes, f) != bytes) return 2;
   fclose(f);
-  std::vector<FxTw> tw(3 * (size_t)n);
+  std::vector<FxTw> tw(4 * (size_t)n);
   fx_twiddles(n, tw.data());
+  fx_dct_twiddles(n, tw.data() + 3 * n);
   double2* d;
   FxTw* t;
   if (cudaMalloc(&d, bytes) != cudaSuccess || cudaMalloc(&t, tw.size() * sizeof(FxTw)) != cudaSuccess) return 3;
@@ -37,7 +38,11 @@ int main(int argc, char** argv) {
   if (poisson_set_attributes() != cudaSuccess) return 4;
   const size_t smem = (size_t)2 * R * (n + 1) * sizeof(double2);
   const unsigned blocks = (rows + R - 1) / R;
-  if (sign < 0)
+  if (cosine && sign < 0)
+    dctx_fwd_kernel<<<blocks, 256, smem>>>(d, t, t + 3 * n, rows, n, fft_plan(n), R);
+  else if (cosine)
+    dctx_inv_kernel<<<blocks, 256, smem>>>(d, t, t + 3 * n, rows, n, fft_plan(n), R);
+  else if (sign < 0)
     single_kernel<FftxK<-1>><<<blocks, 256, smem>>>(FftxK<-1>::Args{d, t, rows, n, fft_plan(n), R});
   else
     single_kernel<FftxK<1>><<<blocks, 256, smem>>>(FftxK<1>::Args{d, t, rows, n, fft_plan(n), R});
@@ -57,11 +62,11 @@ def transform(tmp_path_factory):
     subprocess.run([build._nvcc(), *build.NVCC_FLAGS, "-I", build.CSRC, str(d / "main.cu"), *objs, "-lcudart", "-o",
                     str(d / "main")], check=True, capture_output=True)
 
-    def run(x, R, sign):
+    def run(x, R, sign, cosine=0):
         x = np.ascontiguousarray(x, dtype=np.complex128)
         x.tofile(d / "in")
         subprocess.run([str(d / "main"), str(d / "in"), str(d / "out"), str(x.shape[1]), str(R), str(x.shape[0]),
-                        str(sign)], check=True, timeout=120)
+                        str(sign), str(cosine)], check=True, timeout=120)
         return np.fromfile(d / "out", dtype=np.complex128).reshape(x.shape)
 
     return run
@@ -107,3 +112,31 @@ def test_error_of_each_sequence(transform, n, R, sign):
     err = np.hypot(got.real - ref[..., 0], got.imag - ref[..., 1])
     rel = np.sqrt((err ** 2).sum(1) / (ref ** 2).sum((1, 2)))
     assert rel.max() <= 1.2e-16, [(float(r), int(q)) for r, q in zip(rel, range(len(x))) if r > 1.2e-16][:8]
+
+
+@pytest.mark.parametrize("cosine", [0, 1])
+@pytest.mark.parametrize("n, R", [(24, 16), (64, 16), (216, 8), (256, 4), (512, 3)])
+@pytest.mark.parametrize("sign", [-1, 1])
+def test_sequences_outside_the_range_leave_the_others(transform, n, R, sign, cosine):
+    """An infinity, a NaN or values near an end of the binary64 range in some sequences: the others come out
+    the same, bit for bit, those scaled by a power of two as FP64 arithmetic leaves them.  (In FP64 throughout,
+    those would be the scaled results bit for bit: that they differ shows that the others were not.)"""
+    rng = np.random.default_rng(n)
+    rows = 4 * R + 1
+    x = rng.standard_normal((rows, n)) + 1j * rng.standard_normal((rows, n))
+    clean = transform(x, R, sign, cosine)
+    odd = np.arange(rows) % 3 == 1
+    kind = np.arange(rows) // 3 % 4
+    y = x.copy()
+    y[odd & (kind == 0), 1] = np.inf
+    y[odd & (kind == 1), n // 2] = complex(0.0, np.nan)
+    y[odd & (kind == 2)] *= 2.0 ** -960
+    y[odd & (kind == 3)] *= 2.0 ** 930
+    got = transform(y, R, sign, cosine)
+    assert (got[~odd] == clean[~odd]).all()
+    assert not np.isfinite(got[odd & (kind < 2)]).all(1).any()
+    for k, e in ((2, 960), (3, -930)):
+        a, b = got[odd & (kind == k)] * 2.0 ** e, clean[odd & (kind == k)]
+        # 3 log2(n) roundings at most, either way
+        assert (a != b).any()
+        assert (np.abs(a - b).max(1) <= 6 * np.log2(n) * 2.0 ** -53 * np.abs(b).max(1)).all()
