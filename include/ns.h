@@ -70,8 +70,11 @@ typedef enum {
 
 /* Precision of the increment path (Sec. 2.2 solves everything in one precision; the mixed
  * form is this library's addition):
- *   NS_FP64  : every stage on FP64 arrays; the right-hand side and the transforms compute in 64-bit
- *              fixed point, with errors no larger than FP64 arithmetic leaves.
+ *   NS_FP64  : every stage on FP64 arrays.  The transforms compute in 64-bit fixed point at the scale of
+ *              a sequence's largest value (errors about 1e-16 of the sequence's 2-norm; z sequences are
+ *              pairs of x columns), the right-hand side at the scale of a 32 x 8 tile's: a few 2^-60 of
+ *              the largest terms its values allow.  A cell around which u, v or w hold fewer than
+ *              53 bits at that scale, and whatever is out of range, take FP64 arithmetic.
  *   NS_MIXED : RHS stencils and the ADI increment solves in FP32 (r, delta and N_prev stored
  *              as float); state accumulation u* = u + delta, divergence, the Poisson solve
  *              (all modes) and the projection stay FP64. */

@@ -200,8 +200,6 @@ FX_HD unsigned fx_span(Fx2 a) {
   const int x = fx_hi(a.x), y = fx_hi(a.y);
   return (unsigned)((x ^ (x >> 31)) | (y ^ (y >> 31)));
 }
-// Right shift before a stage that sums up to four values: keeps the sums below 2^61.5 in modulus
-FX_HD int fx_stage_shift(unsigned span) { return (span >> 28) ? 2 : (span >> 27) ? 1 : 0; }
 
 // ---- sums of products with coefficients of any size (the stencils)
 //

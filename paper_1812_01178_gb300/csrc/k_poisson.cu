@@ -175,15 +175,17 @@ __device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, con
 // on the integer pipes (fx64.cuh).  In FP64 arithmetic they ran at 0.86-0.9 of the FP64 pipe's rate
 // (22 instructions of 16 cycles a warp per radix-4 butterfly); in fixed point a butterfly is 36
 // multiply-adds of about 1.3 cycles and some 100 additions, shifts and logic operations on the
-// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 218 (six FP64
-// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 125, inverse z 295 -> 137.
+// other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 216 (six FP64
+// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 125, inverse z 295 -> 135.
+// All issue 2.4 instructions a cycle of four, at 30 warps an SM, the ALU pipe 53 to 57 % and in the z kernels
+// the FP64 pipe 62 % busy; warps wait for shared and global memory between the stages.
 // Results go back to FP64 by two exact FP64 instructions and a scaling on the otherwise idle pipe (x,
 // inverse z), or by integer steps (after the divergence, which uses that pipe).
 //
 // Every sequence is scaled by its own largest component, and before each stage shifted by 0, 1 or 2 bits,
 // as its own largest value (the or of its magnitudes, gathered while the last stage was written) needs for
 // the next sums to stay below 2^62.  (One shift for all sequences of a block took 583 us for the four
-// transforms, 604 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
+// transforms, 602 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
 // 1024 where FP64 butterflies leave 1.6e-16.)  A sequence's relative error in the 2-norm is then 4e-17 to
 // 1e-16, against 1.1e-16 to 7e-16 with FP64 butterflies, on noise, smooth and decaying data, pulses and steps of 24
 // to 4096 points.  It is one of the whole sequence: of the two real columns that a z sequence packs, one whose sum
@@ -196,12 +198,13 @@ __device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, con
 // fall into different banks) and, in fixed point, element i at fx_slot(i): the stages' writes at
 // strides 4, 8 and 16 are then free of bank conflicts, and so are their contiguous reads.
 // ------------------------------------------------------------------------------------------
-constexpr int FX_SEQ = 16;     // sequences a block holds at most
-constexpr int FX_STAGES = 8;   // of lengths 2^a 3^b <= 4096, a >= 3: at most 7
+constexpr int FX_SEQ = 16;  // sequences a block holds at most
+// By sequence.  (128 bytes: 640 took three blocks of nz = 1024 past 196 KB an SM and left L1 28 KB instead of
+// 60, divergence + z 142 -> 172 us on 96 x 64 x 1024.)
 struct FxBlock {
-  unsigned emax[FX_SEQ];             // by sequence: the largest high word,
-  unsigned span[FX_STAGES][FX_SEQ];  // the or of the magnitudes after each stage,
-  int t[FX_SEQ];                     // where its results stand: bit 62 is exponent(emax) + t
+  unsigned emax[FX_SEQ];  // the largest high word; from the second stage on, where its values stand: the
+                          // exponent of bit 62
+  unsigned grow[FX_SEQ];  // four bits a stage: bits 27 to 30 of the or of the magnitudes after it
 };
 __device__ __forceinline__ int fx_slot(int i) {
   const int t = (i >> 3) & 3;
@@ -219,8 +222,10 @@ __device__ __forceinline__ double2 fx_twd(FxTw w) {  // as doubles (general path
 __host__ __device__ __forceinline__ int fx_stages(int plan) { return (plan & 1) + ((plan & 0xff) >> 1) + (plan >> 8); }
 // all threads, before the loads of a block
 __device__ __forceinline__ void fx_begin(FxBlock& S) {
-  if (threadIdx.x < FX_SEQ) S.emax[threadIdx.x] = 0;
-  if (threadIdx.x < FX_STAGES * FX_SEQ) (&S.span[0][0])[threadIdx.x] = 0;
+  if (threadIdx.x < FX_SEQ) {
+    S.emax[threadIdx.x] = 0;
+    S.grow[threadIdx.x] = 0;
+  }
   __syncthreads();
 }
 // The barrier after the loads: the sequences whose exponents suit the fixed-point path, a bit each
@@ -231,11 +236,11 @@ __device__ __forceinline__ unsigned fx_loaded(const FxBlock& S, int nseq) {
 }
 __device__ __forceinline__ bool fx_all(unsigned ok, int nseq) { return ok + 1 == 1u << nseq; }
 
-// `span` of the lanes of a warp that work on sequence sq joins *slot; `lanes`: those lanes
-__device__ __forceinline__ void fx_gather_span(unsigned span, unsigned lanes, unsigned* slot) {
-  span = __reduce_or_sync(lanes, span);
-  if ((threadIdx.x & 31) == __ffs(lanes) - 1) atomicOr(slot, span);
-}
+// Right shift before the stage after stage `st`: keeps the next sums (of up to four values) below 2^61.5 in
+// modulus.  At most seven stages: lengths 2^a 3^b <= 4096, a >= 3
+__device__ __forceinline__ int fx_shift_after(unsigned grow, int st) { return min((int)(grow >> (4 * st) & 15u), 2); }
+// the or of magnitudes of a sequence after stage st
+__device__ __forceinline__ void fx_grow(unsigned* grow, unsigned span, int st) { atomicOr(grow, (span >> 27) << (4 * st)); }
 
 // x[1..3] times their twiddles, and all four 2^-SH
 template <int SIGN, int SH>
@@ -248,16 +253,13 @@ __device__ __forceinline__ void fx_twiddle4(Fx2 (&x)[4], const FxTw (&w)[3]) {
 // One radix-4 stage of power-of-two sequences (N = 2^a2), `total` butterflies over all of them.  fx_slot is
 // linear over exclusive or, and j, r N / 4 and r Ns have no bits in common with what they are added to, so
 // each thread takes the slot of its first element and flips the bits of the others.  RAW: the inputs are
-// doubles; TW: twiddles.  before: the spans the sequences' shifts follow from, after: those of the results.
+// doubles; TW: twiddles.  emax, grow: of the first sequence; st: the stage's number.
 template <int SIGN, bool RAW, bool TW>
 __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, int total, int ls,
-                                          const FxTw* __restrict__ tw, const unsigned* emax, const unsigned* before,
-                                          unsigned* after) {
+                                          const FxTw* __restrict__ tw, const unsigned* emax, unsigned* grow, int st) {
   const int Ns = 1 << ls, quarter = 1 << (a2 - 2);
   const int s1 = fx_slot(Ns), s2 = fx_slot(2 * Ns);
   const int r1 = fx_slot(quarter), r2 = fx_slot(2 * quarter);
-  // lanes that share a sequence: all, or groups of N / 4
-  const unsigned lanes = quarter >= 32 ? NS_FULL_MASK : ((1u << quarter) - 1) << (threadIdx.x & 31 & -quarter);
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
     const int sq = idx >> (a2 - 2);
     const int j = idx & (quarter - 1);
@@ -281,7 +283,7 @@ __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, 
       if (TW) {
         const FxTw* t = tw + 3 * (Ns + k);
         const FxTw w[3] = {fx_ldtw(t), fx_ldtw(t + 1), fx_ldtw(t + 2)};
-        const int sh = fx_stage_shift(before[sq]);  // one for the lanes of a sequence
+        const int sh = fx_shift_after(grow[sq], st - 1);  // one for the lanes of a sequence
         if (sh == 1) fx_twiddle4<SIGN, 1>(x, w);
         else if (sh == 2) fx_twiddle4<SIGN, 2>(x, w);
         else fx_twiddle4<SIGN, 0>(x, w);
@@ -293,15 +295,23 @@ __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, 
     B[base + (o ^ s1)] = y[1];
     B[base + (o ^ s2)] = y[2];
     B[base + (o ^ s1 ^ s2)] = y[3];
-    fx_gather_span(fx_span(y[0]) | fx_span(y[1]) | fx_span(y[2]) | fx_span(y[3]), lanes, after + sq);
+    unsigned span = fx_span(y[0]) | fx_span(y[1]) | fx_span(y[2]) | fx_span(y[3]);
+    if (quarter >= 32) {  // a warp works on one sequence
+      span = __reduce_or_sync(NS_FULL_MASK, span);
+      if ((threadIdx.x & 31) == 0) fx_grow(grow + sq, span, st);
+    } else {  // groups of N / 4 lanes do
+      const unsigned lanes = ((1u << quarter) - 1) << (threadIdx.x & 31 & -quarter);
+      for (int o = quarter >> 1; o > 0; o >>= 1) span |= __shfl_xor_sync(lanes, span, o);
+      if ((threadIdx.x & (quarter - 1)) == 0) fx_grow(grow + sq, span, st);
+    }
   }
 }
 
 // FIRST: A holds doubles at [seq * ld + i], converted by the first stage; else fixed point at
 // [seq * ld + fx_slot(i)], at most 2^59.5 in modulus, bit 62 standing for exponent + t0.
 // tw[3 (Ns + k) + r - 1]: the twiddle of input r of a stage that follows sub-transforms of length Ns.
-// Returns the buffer of the result (fixed point, slots): bit 62 of a result of sequence q stands for
-// exponent(q) + S.t[q].  q0: the number in S of the first sequence.
+// Returns the buffer of the result (fixed point, slots): bit 62 of a result of sequence q stands for the
+// exponent S.emax[q].  q0: the number in S of the first sequence.
 template <int SIGN, bool FIRST>
 __device__ __forceinline__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int plan, int nseq,
                                             const FxTw* __restrict__ tw, FxBlock& S, int t0 = 0, int q0 = 0) {
@@ -316,24 +326,39 @@ __device__ __forceinline__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int p
     B = x;
     ++stage;
   };
-  // a stage's `total` butterflies where the lanes of a warp may work on any sequences: body(idx, span)
+  // a stage's butterflies, `part` a sequence, where the lanes of a warp may work on several: body(idx, span)
   // returns the sequence
-  auto each = [&](int total, auto body) {
+  auto each = [&](int part, auto body) {
+    const int total = nseq * part;
     for (int base = tid & ~31; base < total; base += blockDim.x) {
       const int idx = base + (tid & 31);
       unsigned span = 0;
       const int sq = idx < total ? body(idx, span) : nseq;
-      const unsigned lanes = __match_any_sync(NS_FULL_MASK, sq);
-      if (sq < nseq) fx_gather_span(span, lanes, &S.span[stage][q0 + sq]);
+      if (part >= 32) {  // two at most (the second may be none)
+        const bool one = sq == __shfl_sync(NS_FULL_MASK, sq, 0);
+        const unsigned a = __reduce_or_sync(NS_FULL_MASK, one ? span : 0u);
+        const unsigned b = __reduce_or_sync(NS_FULL_MASK, one ? 0u : span);
+        if ((tid & 31) == 0) fx_grow(S.grow + q0 + sq, a, stage);
+        if ((tid & 31) == 31 && !one && sq < nseq) fx_grow(S.grow + q0 + sq, b, stage);
+      } else if (sq < nseq) {
+        fx_grow(S.grow + q0 + sq, span, stage);
+      }
     }
   };
-  auto shift = [&](int sq) { return fx_stage_shift(S.span[stage - 1][q0 + sq]); };
+  auto shift = [&](int sq) { return fx_shift_after(S.grow[q0 + sq], stage - 1); };
+  // where the values of each sequence stand, kept by one thread each from the second stage on
+  auto stand = [&](int t) {
+    if (tid < nseq) {
+      const unsigned e = S.emax[q0 + tid];
+      S.emax[q0 + tid] = (stage == 1 ? fx_exponent(e) + t : (int)e) + shift(tid);
+    }
+  };
+  const int t_first = FIRST ? ((a2 & 1) ? 3 : 4) : t0;
   int Ns = 1;
   bool first = true;  // the stage with Ns = 1, which has no twiddles
   if (a2 & 1) {
     const int half = N >> 1;
-    if (tid < nseq) S.t[q0 + tid] = FIRST ? 3 : t0;
-    each(nseq * half, [&](int idx, unsigned& span) {
+    each(half, [&](int idx, unsigned& span) {
       const int sq = p2 ? idx >> (a2 - 1) : idx / half;
       const int j = idx - sq * half;
       Fx2 x[2];
@@ -360,17 +385,17 @@ __device__ __forceinline__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int p
   for (int st = 0; st < (a2 >> 1); ++st, Ns <<= 2) {
     const int ls = __ffs(Ns) - 1;  // Ns is a power of two in the radix-4 stages
     const int total = nseq * quarter;
-    if (tid < nseq) S.t[q0 + tid] = first ? (FIRST ? 4 : t0) : S.t[q0 + tid] + shift(tid);
+    if (!first) stand(t_first);
     if (p2) {
       if (first)
-        fx_stage4<SIGN, FIRST, false>(A, B, a2, ld, total, ls, tw, S.emax + q0, nullptr, S.span[stage] + q0);
+        fx_stage4<SIGN, FIRST, false>(A, B, a2, ld, total, ls, tw, S.emax + q0, S.grow + q0, stage);
       else
-        fx_stage4<SIGN, false, true>(A, B, a2, ld, total, ls, tw, S.emax + q0, S.span[stage - 1] + q0, S.span[stage] + q0);
+        fx_stage4<SIGN, false, true>(A, B, a2, ld, total, ls, tw, S.emax + q0, S.grow + q0, stage);
       close();
       first = false;
       continue;
     }
-    each(total, [&](int idx, unsigned& span) {
+    each(quarter, [&](int idx, unsigned& span) {
       const int sq = idx / quarter;
       const int j = idx - sq * quarter;
       const int k = j & (Ns - 1);
@@ -407,8 +432,8 @@ __device__ __forceinline__ Fx2* fx_stockham(Fx2* A, Fx2* B, int N, int ld, int p
   }
   const int third = N / 3;
   for (int st = 0; st < b3; ++st, Ns *= 3) {
-    if (tid < nseq) S.t[q0 + tid] += shift(tid);
-    each(nseq * third, [&](int idx, unsigned& span) {
+    stand(t_first);
+    each(third, [&](int idx, unsigned& span) {
       const int sq = idx / third;
       const int j = idx - sq * third;
       const int g = j / Ns;
@@ -614,7 +639,7 @@ struct DivzK {
     const int n = m == 0 ? 0 : nz - m;
     double2 x;
     if (fixed) {
-      const int e = fx_exponent(S.emax[c]) + S.t[c];
+      const int e = (int)S.emax[c];
       const Fx2 zm = R[c * ld + fx_slot(m)];
       const Fx2 zn = R[c * ld + fx_slot(n)];
       x = (il & 1) == 0 ? make_double2(fx_to(zm.x + zn.x, e), fx_to(zm.y - zn.y, e))
@@ -669,7 +694,7 @@ struct FftxK {
     auto put = [&](const Fx2* X, int q, int r, bool fixed) {
       const int i = q - r * nx;
       if (fixed) {
-        const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r]);
+        const double e = fx_unit((int)S.emax[r]);
         const Fx2 v = X[r * ld + fx_slot(i)];
         g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
       } else {
@@ -1013,7 +1038,7 @@ struct IfftzK {
       double* phi = a.phi + k * pl + (long)j * nx + i0 + il;
       if (fixed) {
         const Fx2 v = R[c * ld + fx_slot(k)];
-        *phi = fx_double((il & 1) ? v.y : v.x) * fx_unit(fx_exponent(S.emax[c]) + S.t[c]);
+        *phi = fx_double((il & 1) ? v.y : v.x) * fx_unit((int)S.emax[c]);
       } else {
         const double2 v = reinterpret_cast<const double2*>(R)[c * ld + k];
         *phi = (il & 1) ? v.y : v.x;
@@ -1720,8 +1745,8 @@ struct ProjectK {
 // the real and imaginary parts of v (separated through V_{N-l}), X_l = Re(w_l V_a) + i Re(w_l V_b),
 // w_l = exp(-i pi l / (2N)).  Inverse (unnormalised, N times the DCT-III inverse):
 // V_l = conj(w_l) (X_l - i X_{N-l}) (X_N = 0), v = IFFT(V), x_{2n} = v_n, x_{2n+1} = v_{N-1-n}.
-// twd holds w_l for l < N and then w_l / 2: the forward kernel takes the halved entries, which
-// absorb the 1/2 of the real / imaginary separation exactly (a power of two).
+// twd holds w_l for l < N; in the FP32 form also w_l / 2 after them, which the forward kernel takes to
+// absorb the 1/2 of the real / imaginary separation exactly (in fixed point that is a shift).
 // ------------------------------------------------------------------------------------------
 // The FP64 form: transforms and twiddles in fixed point (general path: FP64).  twd: FxTw of w_l.
 __global__ void __launch_bounds__(256, 4) dctx_fwd_kernel(double2* __restrict__ spec, const FxTw* __restrict__ twx,
@@ -1740,15 +1765,15 @@ __global__ void __launch_bounds__(256, 4) dctx_fwd_kernel(double2* __restrict__ 
                [&](int r, int i, double2 v) { A[r * ld + ((i & 1) ? nx - 1 - (i >> 1) : (i >> 1))] = v; });
   const unsigned ok = fx_loaded(S, R);
   // a, b = (V_l +- conj V_{N-l}) / 2 (b over i), times w_l
-  const unsigned* span = S.span[fx_stages(px) - 1];
+  const int last = fx_stages(px) - 1;
   auto put = [&](const Fx2* V, int q, int r, bool fixed) {
     const int l = q - r * nx, n = l == 0 ? 0 : nx - l;
     const FxTw w = fx_ldtw(twd + l);
     if (fixed) {
       const Fx2 vl = fx_shr(V[r * ld + fx_slot(l)], 1);
       const Fx2 vn = fx_shr(V[r * ld + fx_slot(n)], 1);
-      const int sh = fx_stage_shift(span[r]);
-      const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r] + sh);
+      const int sh = fx_shift_after(S.grow[r], last);
+      const double e = fx_unit((int)S.emax[r] + sh);
       const Fx2 xa = fx_cmul<-1>(Fx2{vl.x + vn.x, vl.y - vn.y}, w, sh);
       const Fx2 xb = fx_cmul<-1>(Fx2{vl.y + vn.y, vn.x - vl.x}, w, sh);
       g[q] = make_double2(fx_double(xa.x) * e, fx_double(xb.x) * e);
@@ -1809,7 +1834,7 @@ __global__ void __launch_bounds__(256, 4) dctx_inv_kernel(double2* __restrict__ 
   auto put = [&](const Fx2* X, int q, int r, bool fixed) {
     const int i = q - r * nx, l = (i & 1) ? nx - 1 - (i >> 1) : (i >> 1);
     if (fixed) {
-      const double e = fx_unit(fx_exponent(S.emax[r]) + S.t[r]);
+      const double e = fx_unit((int)S.emax[r]);
       const Fx2 v = X[r * ld + fx_slot(l)];
       g[q] = make_double2(fx_double(v.x) * e, fx_double(v.y) * e);
     } else {

@@ -547,17 +547,17 @@ struct RhsTiledK {
 //
 // In FP64 arithmetic the tile was bound by the FP64 pipe: 64.8 instructions a cell of 16 cycles a
 // warp, 1.547 ms on 256 x 192 x 256 cells with the pipe 88 % busy.  Here the products and the viscous
-// sums run on the integer pipes; the FP64 pipe keeps 12 instructions a cell (pressure gradient, the
-// stored N, closing the sum): 0.664 ms, about a thousand instructions a cell and warp, bound by the
-// latency of their chains.  Tile and block from timings: 32 x 16 cells, two a thread, two blocks an SM
+// sums run on the integer pipes; the FP64 pipe keeps 13 instructions a cell (pressure gradient, the
+// stored N, closing the sum): 0.676 ms, 1257 instructions a warp of cells (with the coefficients), 2.44 a
+// cycle; the ALU pipe is 62 % busy, and warps wait at the two barriers of a row, for fixed latencies and for
+// the math pipes, in that order.  Tile and block from timings: 32 x 16 cells, two a thread, two blocks an SM
 // 0.705; 32 x 16, one a thread (56 registers, 200 bytes spilled) 0.849; 32 x 12 0.773; this one, 27
 // warps an SM, 0.677; with the viscous sum converted by the FP64 pipe (18 instructions) 0.704.  r is 3
 // to 10 times nearer to the exact sums than FP64 arithmetic was (against extended precision).
 //
 // A block marches a 32 x 8 (x, z) column along y.  The planes of u, v, w around the row stand in
 // shared memory as integers, each plane of each field scaled by its own largest magnitude in the
-// tile, so that 60 bits lie below the largest value near a cell (an FP64 result keeps 53 below its
-// own terms); p stands there in FP64.  Sums whose terms have different scales are sums of products
+// tile and cut (towards zero) to 60 bits below it; p stands there in FP64.  Sums whose terms have different scales are sums of products
 // with coefficients into which the scales are folded (fx_wcoef).  One warp of the nine does nothing
 // else: it forms the coefficients of row j + 1, a term per lane and the scale of each sum from the
 // bounds of its terms, while the others work on row j.
@@ -799,7 +799,7 @@ struct RhsFxK {
     const int i = i0 + lane, k = k0 + wz;
     const bool active = i < nx && k < nz;  // the last tiles may reach past the grid
 
-    // Plane positions of this thread: row wz of the 18, and a second: rows 16, 17 (warps 0, 1) or the
+    // Plane positions of this thread: row wz of the 10, and a second: rows 8, 9 (warps 0, 1) or the
     // halo columns (warps 2, 3).  gi = -2: nothing there.
     int gk[2], gi[2], pos[2];
 #pragma unroll
