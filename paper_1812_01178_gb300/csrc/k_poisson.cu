@@ -176,7 +176,7 @@ __device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, con
 // (22 instructions of 16 cycles a warp per radix-4 butterfly); in fixed point a butterfly is 36
 // multiply-adds of about 1.3 cycles and some 100 additions, shifts and logic operations on the
 // other pipes.  256 x 192 x 256, us a launch, FP64 -> fixed point: divergence + z 434 -> 216 (six FP64
-// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 125, inverse z 295 -> 135.
+// instructions a cell of the divergence remain, 120 us of that pipe), x 236 -> 121, inverse z 295 -> 132.
 // All issue 2.4 instructions a cycle of four, at 30 warps an SM, the ALU pipe 53 to 57 % and in the z kernels
 // the FP64 pipe 62 % busy; warps wait for shared and global memory between the stages.
 // Results go back to FP64 by two exact FP64 instructions and a scaling on the otherwise idle pipe (x,
@@ -185,7 +185,7 @@ __device__ float2* stockham(float2* A, float2* B, int N, int plan, int nseq, con
 // Every sequence is scaled by its own largest component, and before each stage shifted by 0, 1 or 2 bits,
 // as its own largest value (the or of its magnitudes, gathered while the last stage was written) needs for
 // the next sums to stay below 2^62.  (One shift for all sequences of a block took 583 us for the four
-// transforms, 602 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
+// transforms, 589 now, but cost those that do not grow beside one that does two bits a stage: 6.5e-16 at
 // 1024 where FP64 butterflies leave 1.6e-16.)  A sequence's relative error in the 2-norm is then 4e-17 to
 // 1e-16, against 1.1e-16 to 7e-16 with FP64 butterflies, on noise, smooth and decaying data, pulses and steps of 24
 // to 4096 points.  It is one of the whole sequence: of the two real columns that a z sequence packs, one whose sum
@@ -299,10 +299,8 @@ __device__ __forceinline__ void fx_stage4(const Fx2* A, Fx2* B, int a2, int ld, 
     if (quarter >= 32) {  // a warp works on one sequence
       span = __reduce_or_sync(NS_FULL_MASK, span);
       if ((threadIdx.x & 31) == 0) fx_grow(grow + sq, span, st);
-    } else {  // groups of N / 4 lanes do
-      const unsigned lanes = ((1u << quarter) - 1) << (threadIdx.x & 31 & -quarter);
-      for (int o = quarter >> 1; o > 0; o >>= 1) span |= __shfl_xor_sync(lanes, span, o);
-      if ((threadIdx.x & (quarter - 1)) == 0) fx_grow(grow + sq, span, st);
+    } else {  // groups of N / 4 lanes do: shuffles or masked reductions took longer
+      fx_grow(grow + sq, span, st);
     }
   }
 }
@@ -2246,8 +2244,11 @@ PoisShape pois_shape(const ns_ctx* c) {
   while (q.nx % q.TXm) q.TXm >>= 1;
   q.nrows = (long)c->nzh * q.ny;
   // rows of an x-transform block: two buffers within 56 KB (four blocks of an SM; three of 64 KB and 80
-  // registers: 129 -> 117 us at nx = 256)
+  // registers: 129 -> 117 us at nx = 256), and, of power-of-two lengths, as many as fill whole passes of the
+  // 256 threads with radix-4 butterflies (1024 / nx a pass: 4 rows instead of 6 at nx = 256, 124 -> 121 us; 8 instead
+  // of 13 at 128, 16.3 -> 12.2 on 128 x 32 x 64)
   q.R = std::max(1, std::min(FX_SEQ, (int)(56 * 1024 / (2 * (q.nx + 1) * sizeof(double2)))));
+  if (const int pass = std::max(1, 1024 / q.nx); q.px >> 8 == 0 && q.R > pass) q.R -= q.R % pass;
   q.smx = (size_t)2 * q.R * (q.nx + 1) * sizeof(double2);
   q.bx = (unsigned)((q.nrows + q.R - 1) / q.R);
   // ... in the mixed form (complex64, 32 KB)
